@@ -797,7 +797,7 @@ void tlu_factor_t(Context& c, TileLU& L) {
   LAUNCH_NAMED(D, "k_tlu_to_band", (k_tlu_to_band<FT, TS>), grid_for_n(nb), 256, 0, N0, b0, TB, T, DG, (FT*)D.A0f);
   constexpr int BS = dev::SolveBlock<FT>::BS;
   const int nblk = (N0 + BS - 1) / BS;
-  LAUNCH_NAMED(D, "k_band_pack", k_band_pack<FT>, (nblk + 7) / 8, 256, sizeof(FT) * 8 * BS * (BS + 1), N0, b0,
+  LAUNCH_NAMED(D, "k_band_pack", k_band_pack<FT>, (nblk + 7) / 8, 256, sizeof(FT) * 8 * dev::pack_scratch<FT>(), N0, b0,
                (const FT*)D.A0f, (FT*)D.A0dinv);
   L.launches_per_factor = D.launches - l0;
 }
@@ -846,13 +846,13 @@ void tlu_prepare(Context& c, bool f32) {
     allow_smem(k_tile_solve_products, kTcSmem);
     allow_smem(k_tile_inverses, kInvSmem);
     if (L->solve_tiles) allow_smem(k_tile_solve, tile_solve_smem(L->NT));
-    allow_smem(k_band_pack<float>, sizeof(float) * 8 * 32 * 33);
+    allow_smem(k_band_pack<float>, sizeof(float) * 8 * dev::pack_scratch<float>());
   } else {
     L->T = D.alloc<double>((size_t)L->NT * L->SW * per);
     L->DG = D.alloc<double>((size_t)L->NT * per);
     allow_smem(k_tlu_panel<double, kTS64, kNS64>, panel_smem<double, kTS64, kNS64>());
     allow_smem(k_tlu_update_simt<double, kTS64, kNS64>, update_simt_smem<double, kTS64, kNS64>());
-    allow_smem(k_band_pack<double>, sizeof(double) * 8 * 16 * 17);
+    allow_smem(k_band_pack<double>, sizeof(double) * 8 * dev::pack_scratch<double>());
   }
 }
 

@@ -2,14 +2,15 @@
 //
 // * element routines of Eq. 1 (P1 nonlinear diffusion) and Eq. 2 (Q1 compressible Neo-Hooke),
 // * block reductions with a fixed summation order (results do not depend on scheduling),
-// * the no-pivoting band LU with a sliding shared-memory window over (b + 2) rows, reading
-//   the assembled CSR rows of a local Jacobian and streaming finished factor rows to global
-//   memory,
+// * the no-pivoting band LU: in place by square tiles in a shared-memory window (the local and
+//   coarse matrices), and row by row from CSR rows (the harmonic extension),
 // * blocked forward / backward substitution with the band factors (one warp solves each
 //   32-row diagonal block, the whole CTA applies its coupling to the next b rows).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "nls_internal.h"
 
@@ -325,12 +326,32 @@ __device__ int band_lu(int n, int b, const RowSource& src, FT* __restrict__ F, F
 }
 
 // ------------------------------------------------------------------------------------------
-// In-place band LU with asynchronous row staging.  F holds the assembled band rows on entry
-// (row-major, W = 2b + 1) and the factors on exit (layout as above).  Rows are copied into the
-// shared-memory ring with cp.async PD rows ahead of use, so the global-memory latency of a
-// row overlaps the PD elimination steps before it is needed; each row is read exactly once
-// and written back exactly once.
-// smem: win [(b + 2 + PD) * W], rp [b + 2 + PD], flag [1].
+// In-place band LU by square tiles.  F holds the assembled band rows on entry (row-major,
+// W = 2b + 1) and the factors on exit (layout as above).
+//
+// What bounds it: the chain of pivots (a reciprocal, a product and an update per pivot), and what
+// every elimination step costs besides.  One step per pivot with a CTA barrier, a shared-memory
+// load and a store per updated entry costs 1400 (b = 42) to 2600 cycles (b = 83) in FP32.  Here NB
+// pivots are eliminated per panel with two barriers:
+//   A  one thread per row (column) finishes the panel's L (U) tiles in registers;
+//   B  warp 0 updates the next diagonal tile and factors it, while the other warps fetch the tiles
+//      that enter with the next panel (cp.async), apply the NB rank-1 updates to the trailing
+//      tiles with one load and one store per entry (G x G entries per lane, 16-byte loads), and
+//      write the finished tiles out.
+// Every entry still receives its updates one pivot after the other in ascending order, each one
+// fused multiply-add with the multiplier rounded before it, so the FP32 factors are bit for bit
+// those of the step-by-step elimination.  Factorization with packing, one CTA per SM, before and
+// now: n = 1598, b = 42, FP32 1.06 ms (128 threads) -> 0.39 ms (256 threads); n = 3120, b = 83, FP32
+// 3.9 -> 1.0 ms (512 threads); n = 2520, b = 75, FP64 8.8 -> 5.9 ms (4.6 ms of it FP64 instructions at
+// the part's rate).
+//
+// The window holds the active tiles: tile (I, J) of the matrix sits in slot (I mod RT, J mod RT),
+// RT = tb + 2 with tb = ceil(b / NB) -- the tb + 1 tile rows and columns a panel touches, and the
+// ones entering with the next panel (RT = tb + 1 and no copy ahead where that does not fit).  Tile
+// entries outside the band are exact zeros and stay zero; rows past n hold the identity.  A tile
+// row is 64 bytes: its 16-byte groups are permuted by the row pair, and the rows of a pair swapped
+// in odd slot columns, so that the vector loads of rows and of columns across two neighbouring
+// tiles hit distinct banks.
 // ------------------------------------------------------------------------------------------
 template <typename FT>
 __device__ inline void cp_async_elem(FT* sdst, const FT* gsrc) {
@@ -346,126 +367,310 @@ __device__ inline void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// One warp stages band row `row` (if it exists) into dst and commits one copy group per lane.
+// Entries per 16-byte group, and rows of a tile: 16 in FP32, 8 in FP64 (64-byte tile rows).
 template <typename FT>
-__device__ inline void stage_row_async(int row, int n, int W, const FT* F, FT* dst) {
-  const int lane = threadIdx.x & 31;
-  if (row < n) {
-    const FT* src = F + (int64_t)row * W;
-    for (int d = lane; d < W; d += 32) cp_async_elem<FT>(dst + d, src + d);
-  }
-  cp_async_commit();
+struct LuTile {
+  static constexpr int G = 16 / (int)sizeof(FT);
+  static constexpr int NB = 4 * G;
+  static constexpr int TE = NB * NB;
+};
+
+// Tiles of half a band, and window entries of the tiled band LU (the tiles, with the next panel's
+// for ahead = 1, and the transposed multipliers of one diagonal tile).
+template <typename FT>
+__host__ __device__ constexpr int band_lu_half(int b) {
+  return b > 0 ? (b + LuTile<FT>::NB - 1) / LuTile<FT>::NB : 1;
+}
+template <typename FT>
+__host__ __device__ constexpr size_t band_lu_window(int b, int ahead) {
+  const size_t rt = (size_t)(band_lu_half<FT>(b) + 1 + ahead);
+  return (rt * rt + 1) * LuTile<FT>::TE;
 }
 
-constexpr int kLuPrefetch = 8;
-
-// Rows of the shared-memory window of the band LU: the b + 2 rows an elimination step touches
-// plus the rows staged ahead.
-__host__ __device__ constexpr int band_lu_window_rows(int b) { return b + 2 + kLuPrefetch; }
-
-// Row stride of the window (>= 2b + 1 entries).  One warp of the 2D-tiled update touches 4
-// consecutive rows x 8 consecutive columns, at addresses (stride - 1) apart from row to row;
-// with (stride - 1) = 8 or 24 (mod 32) the four rows land on disjoint groups of 8 banks.
-__host__ __device__ constexpr int band_lu_window_stride(int b) {
+// Rows and row stride of a (b + 10)-row window: the size that the limits on the half bandwidth and
+// on the subdomain size are stated for (no tiled window that such a window allows is larger).
+__host__ __device__ constexpr int band_limit_rows(int b) { return b + 10; }
+__host__ __device__ constexpr int band_limit_stride(int b) {
   int w = 2 * b + 1;
   while (((w - 1) & 31) != 8 && ((w - 1) & 31) != 24) ++w;
   return w;
 }
 
-// Thread mapping of one elimination step (2D tiling): the CTA is TY x 8 threads, thread
-// (ty, tx) updates rows k+1+ri with ri = ty, ty + TY, ... and columns k+1+cj with
-// cj = tx, tx + 8, ..., tx + 8 (QM - 1) (b <= 8 QM).  Every thread loads its QM pivot-row
-// values once per step and one multiplier per row, so the per-row overhead is shared by QM
-// entries and at most 7 column slots per row are idle.  Every thread forms 1 / pivot itself
-// after the step's barrier (no single-thread step on the critical path); thread 0 records it
-// in rp (per ring slot) for the write-back of the L part and flags a bad pivot.
 template <typename FT>
 __device__ inline FT recip(FT p) {
   if constexpr (sizeof(FT) == 4) return __frcp_rn(p);
   else return (FT)1 / p;
 }
 
-template <typename FT, int QM>
-__device__ int band_lu_inplace_q(int n, int b, FT* __restrict__ F, FT* win, FT* rp, int* flag) {
-  constexpr int PD = kLuPrefetch, TX = 8;
-  const int W = 2 * b + 1, WS = band_lu_window_stride(b), R = b + 2 + PD;
-  const int tid = threadIdx.x, T = blockDim.x, tx = tid % TX, ty = tid / TX, TY = T / TX;
-  if (tid == 0) *flag = 0;
-  // stage rows 0 .. b + PD (one copy group per row and thread)
-  for (int i = 0; i <= b + PD; ++i) {
-    if (i < n)
-      for (int d = tid; d < W; d += T) cp_async_elem<FT>(win + i * WS + d, F + (int64_t)i * W + d);
-    cp_async_commit();
+// f(integral_constant<int, I>) for I = I0 .. N - 1: a loop whose index is a constant in its body
+template <int I, int N, typename F>
+__device__ __forceinline__ void static_for(F&& f) {
+  if constexpr (I < N) {
+    f(std::integral_constant<int, I>{});
+    static_for<I + 1, N>(f);
   }
-  cp_async_wait<PD>();
-  __syncthreads();
-  int sk = 0, s1 = 1;  // ring slots of rows k and k + 1 (R >= b + 2 >= 2)
-  for (int k = 0; k < n; ++k) {
-    const FT* rowk = win + sk * WS;
-    const FT piv = rowk[b];
-    const FT rpk = recip<FT>(piv);
-    if (tid == 0) {
-      if (!(piv != (FT)0) || !isfinite((double)piv)) *flag = 1;
-      rp[sk] = rpk;
-    }
-    const int lim = min(b, n - 1 - k);
-    // row k is final: write it back in place (scaled L part, reciprocal pivot, U part)
-    for (int d = tid; d < W; d += T) {
-      FT v = rowk[d];
-      if (d < b) {
-        int sj = sk - b + d;
-        if (sj < 0) sj += R;
-        v = (k - b + d >= 0) ? v * rp[sj] : (FT)0;
-      } else if (d == b) {
-        v = rpk;
-      }
-      F[(int64_t)k * W + d] = v;
-    }
-    // stage row k + b + 1 + PD into the slot row k - 1 used
-    {
-      const int rs = k + b + 1 + PD;
-      const int ss = (sk == 0) ? R - 1 : sk - 1;
-      if (rs < n)
-        for (int d = tid; d < W; d += T) cp_async_elem<FT>(win + ss * WS + d, F + (int64_t)rs * W + d);
-      cp_async_commit();
-    }
-    // rank-1 update of rows k+1..k+lim, columns k+1..k+lim
-    FT u[QM];
-#pragma unroll
-    for (int q = 0; q < QM; ++q) u[q] = (tx + TX * q < lim) ? rowk[b + 1 + tx + TX * q] : (FT)0;
-    for (int ri = ty; ri < lim; ri += TY) {
-      int slot = s1 + ri;
-      if (slot >= R) slot -= R;
-      FT* rowi = win + slot * WS + b - ri;
-      const FT l = rowi[-1] * rpk;
-#pragma unroll
-      for (int q = 0; q < QM; ++q) {
-        const int cj = tx + TX * q;
-        if (cj < lim) rowi[cj] -= l * u[q];
-      }
-    }
-    // rows up to k + b + 1 must have landed before step k + 1
-    cp_async_wait<PD>();
-    __syncthreads();
-    sk = s1;
-    s1 = (s1 + 1 == R) ? 0 : s1 + 1;
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-  return *flag;
 }
 
-
-// Dispatch on the number of column slots per thread (half bandwidth up to 128).  blockDim.x
-// must be a multiple of 8.
 template <typename FT>
-__device__ int band_lu_inplace(int n, int b, FT* __restrict__ F, FT* win, FT* rp, int* flag) {
+struct alignas(16) LuVec {
+  FT v[LuTile<FT>::G];
+};
+
+// Returns (to every thread) 0 on success, 1 if a pivot was zero or not finite.  `flag`: three ints
+// of shared memory.  `win`: at least
+// band_lu_window<FT>(b, 0) entries, 16-byte aligned, win_cap of them usable.  blockDim.x: a
+// multiple of 32, at least 64.
+template <typename FT>
+__device__ __noinline__ int band_lu_inplace(int n, int b, FT* __restrict__ F, FT* win, size_t win_cap, int* flag) {
+  constexpr int G = LuTile<FT>::G, NB = LuTile<FT>::NB, TE = LuTile<FT>::TE;
+  constexpr int RH = 32 / NB;       // tile rows a warp covers with one entry per lane
+  constexpr int C = NB * NB / 32;   // entries per lane of a tile spread over a warp
+  using Vec = LuVec<FT>;
   if (n <= 0) return 0;
-  if (b <= 32) return band_lu_inplace_q<FT, 4>(n, b, F, win, rp, flag);
-  if (b <= 48) return band_lu_inplace_q<FT, 6>(n, b, F, win, rp, flag);
-  if (b <= 64) return band_lu_inplace_q<FT, 8>(n, b, F, win, rp, flag);
-  if (b <= 96) return band_lu_inplace_q<FT, 12>(n, b, F, win, rp, flag);
-  return band_lu_inplace_q<FT, 16>(n, b, F, win, rp, flag);
+  int* const s_task = flag + 1;  // two task counters, used in turn
+  const int W = 2 * b + 1, tb = band_lu_half<FT>(b), NP = (n + NB - 1) / NB;
+  const bool ahead = band_lu_window<FT>(b, 1) <= win_cap;
+  const int RT = tb + 1 + (ahead ? 1 : 0);
+  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = T >> 5;
+  FT* const dt = win + RT * RT * TE;  // dt[k NB + i]: multiplier l_ik of the current diagonal tile
+  auto tile = [&](int si, int sj) { return win + (si * RT + sj) * TE; };
+  // entry (r, c) of a tile in slot column sj; c a multiple of G for vector access
+  auto at = [](int r, int c, int sj) {
+    return ((r ^ (sj & 1)) * 4 + (((c / G) ^ (r >> 1)) & 3)) * G + c % G;
+  };
+  auto wrap = [&](int s) { return s >= RT ? s - RT : s; };  // slot index < 2 RT into the ring
+  // one warp copies tile (I, J) into slots (si, sj): lane (r0, c) rows r0, r0 + RH, ..
+  const int lr = lane / NB, lc = lane % NB;
+  auto fetch = [&](int I, int J, int si, int sj) {
+    FT* t = tile(si, sj);
+    const int i0 = I * NB + lr, j = J * NB + lc, d0 = j - i0 + b;
+    const FT* src = F + ((int64_t)i0 * W + d0);
+    const bool jn = j < n;
+#pragma unroll
+    for (int q = 0; q < NB / RH; ++q) {
+      FT* dst = t + at(lr + q * RH, lc, sj);
+      const int i = i0 + q * RH;
+      if (jn && i < n && (unsigned)(d0 - q * RH) < (unsigned)W) cp_async_elem<FT>(dst, src + q * RH * (int64_t)(W - 1));
+      else *dst = (i == j) ? (FT)1 : (FT)0;
+    }
+  };
+  // the q-th of the 2 tb + 1 tiles that enter with tile row and column h (in slot sh): (h, h - tb ..
+  // h), then (h - tb .. h - 1, h)
+  auto enter = [&](int q, int h, int sh) {
+    const int back = q <= tb ? tb - q : 2 * tb + 1 - q;
+    if (back > h) return;
+    const int so = sh - back < 0 ? sh - back + RT : sh - back;
+    if (q <= tb) fetch(h, h - back, sh, so);
+    else fetch(h - back, h, so, sh);
+  };
+  // one warp writes the tile (I, J) of slots (si, sj) out
+  auto emit = [&](int I, int J, int si, int sj) {
+    const FT* t = tile(si, sj);
+    const int i0 = I * NB + lr, j = J * NB + lc, d0 = j - i0 + b;
+    FT* dst = F + ((int64_t)i0 * W + d0);
+    const bool jn = j < n;
+    FT v[NB / RH];
+#pragma unroll
+    for (int q = 0; q < NB / RH; ++q) v[q] = t[at(lr + q * RH, lc, sj)];
+#pragma unroll
+    for (int q = 0; q < NB / RH; ++q)
+      if (jn && i0 + q * RH < n && (unsigned)(d0 - q * RH) < (unsigned)W) dst[q * RH * (int64_t)(W - 1)] = v[q];
+  };
+  // warp 0 factors the diagonal tile in slot s: lane (r, h) = (lane % NB, lane / NB) holds row r,
+  // columns h C .. h C + C - 1; pivot rows and columns by shuffles
+  auto factor = [&](int s) {
+    FT* D = tile(s, s);
+    const int r = lane % NB, h = lane / NB;
+    FT a[C];
+#pragma unroll
+    for (int g = 0; g < C; g += G) {
+      const Vec v = *(const Vec*)(D + at(r, h * C + g, s));
+#pragma unroll
+      for (int q = 0; q < G; ++q) a[g + q] = v.v[q];
+    }
+    bool bad = false;
+    static_for<0, NB>([&](auto kc) {
+      constexpr int k = decltype(kc)::value, hk = k / C, kj = k % C, j0 = hk == NB / C - 1 ? kj + 1 : 0;
+      const FT p = __shfl_sync(0xffffffffu, a[kj], k + NB * hk);
+      const FT x = __shfl_sync(0xffffffffu, a[kj], r + NB * hk);
+      FT u[C];
+#pragma unroll
+      for (int j = j0; j < C; ++j) u[j] = __shfl_sync(0xffffffffu, a[j], k + NB * h);
+      const FT rp = recip<FT>(p);
+      bad |= !(p != (FT)0) || !(p - p == (FT)0);  // zero, infinite or NaN
+      const FT l = x * rp;
+#pragma unroll
+      for (int j = j0; j < C; ++j) {
+        const FT y = a[j] - l * u[j];
+        a[j] = (r > k && h * C + j > k) ? y : a[j];
+      }
+      if (h == hk) a[kj] = r > k ? l : (r == k ? rp : a[kj]);
+    });
+#pragma unroll
+    for (int g = 0; g < C; g += G) {
+      Vec v;
+#pragma unroll
+      for (int q = 0; q < G; ++q) v.v[q] = a[g + q];
+      *(Vec*)(D + at(r, h * C + g, s)) = v;
+    }
+#pragma unroll
+    for (int j = 0; j < C; ++j) dt[(h * C + j) * NB + r] = a[j];
+    if (bad && lane == 0) *flag = 1;
+  };
+  if (tid == 0) *flag = 0, s_task[0] = s_task[1] = 0;
+  for (int h = 0; h <= tb && h < NP; ++h)
+    for (int q = wid; q < 2 * tb + 1; q += nw) enter(q, h, h);
+  cp_async_commit();
+  cp_async_wait<0>();
+  __syncthreads();
+  if (wid == 0) factor(0);
+  __syncthreads();
+  int sK = 0;
+  for (int K = 0; K < NP; ++K) {
+    FT* D = tile(sK, sK);
+    const int s1 = wrap(sK + 1);
+    // A: L tiles (I, K) row by row, U tiles (K, J) column by column
+    for (int idx = tid; idx < 2 * tb * NB; idx += T) {
+      const bool lower = idx < tb * NB;
+      const int q = lower ? idx : idx - tb * NB;
+      const int o = q / NB, x = q % NB;  // tile K + 1 + o, row or column x
+      if (K + 1 + o >= NP) continue;
+      const int so = wrap(s1 + o);
+      FT a[NB];
+      if (lower) {
+        FT* L = tile(so, sK);
+#pragma unroll
+        for (int g = 0; g < NB; g += G) {
+          const Vec v = *(const Vec*)(L + at(x, g, sK));
+#pragma unroll
+          for (int i = 0; i < G; ++i) a[g + i] = v.v[i];
+        }
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+#pragma unroll
+          for (int g = k / G * G; g < NB; g += G) {
+            const Vec v = *(const Vec*)(D + at(k, g, sK));
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+              if (g + i == k) a[k] *= v.v[i];
+              else if (g + i > k) a[g + i] -= a[k] * v.v[i];
+            }
+          }
+        }
+#pragma unroll
+        for (int g = 0; g < NB; g += G) {
+          Vec v;
+#pragma unroll
+          for (int i = 0; i < G; ++i) v.v[i] = a[g + i];
+          *(Vec*)(L + at(x, g, sK)) = v;
+        }
+      } else {
+        FT* U = tile(sK, so);
+#pragma unroll
+        for (int k = 0; k < NB; ++k) a[k] = U[at(k, x, so)];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+#pragma unroll
+          for (int g = (k + 1) / G * G; g < NB; g += G) {
+            const Vec v = *(const Vec*)(dt + k * NB + g);
+#pragma unroll
+            for (int i = 0; i < G; ++i)
+              if (g + i > k) a[g + i] -= v.v[i] * a[k];
+          }
+        }
+#pragma unroll
+        for (int k = 1; k < NB; ++k) U[at(k, x, so)] = a[k];
+      }
+    }
+    if (tid == 0) s_task[(K + 1) & 1] = 0;
+    __syncthreads();
+    // B
+    if (wid == 0 && K + 1 < NP) {
+      // the next diagonal tile: C entries per lane
+      constexpr int RL = C / G;  // rows per lane
+      FT* O = tile(s1, s1);
+      const FT *L = tile(s1, sK), *U = tile(sK, s1);
+      const int r0 = (lane >> 2) * RL, c0 = (lane & 3) * G;
+      Vec acc[RL];
+#pragma unroll
+      for (int i = 0; i < RL; ++i) acc[i] = *(const Vec*)(O + at(r0 + i, c0, s1));
+#pragma unroll
+      for (int k = 0; k < NB; k += G) {
+        Vec l[RL], v[G];
+#pragma unroll
+        for (int i = 0; i < RL; ++i) l[i] = *(const Vec*)(L + at(r0 + i, k, sK));
+#pragma unroll
+        for (int i = 0; i < G; ++i) v[i] = *(const Vec*)(U + at(k + i, c0, s1));
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+#pragma unroll
+          for (int i = 0; i < RL; ++i)
+#pragma unroll
+            for (int j = 0; j < G; ++j) acc[i].v[j] -= l[i].v[q] * v[q].v[j];
+      }
+#pragma unroll
+      for (int i = 0; i < RL; ++i) *(Vec*)(O + at(r0 + i, c0, s1)) = acc[i];
+      __syncwarp();
+      factor(s1);
+    }
+    // tiles that enter, trailing updates, finished tiles out: handed out to the warps in that order
+    const int n_in = (ahead && K + tb + 1 < NP) ? 2 * tb + 1 : 0, pairs = (tb + 1) / 2;
+    const int n_up = K + 1 < NP ? tb * pairs : 0, n_task = n_in + n_up + 2 * tb + 1;
+    for (;;) {
+      int task = 0;
+      if (lane == 0) task = atomicAdd(&s_task[K & 1], 1);
+      task = __shfl_sync(0xffffffffu, task, 0);
+      if (task >= n_task) break;
+      if (task < n_in) {
+        enter(task, K + tb + 1, sK == 0 ? RT - 1 : sK - 1);
+      } else if (task < n_in + n_up) {
+        // one tile row by two tile columns, G x G entries per lane
+        const int u = task - n_in, oi = u / pairs, oj = 2 * (u % pairs) + ((lane & 7) >> 2);
+        if (oj >= tb || K + 1 + oi >= NP || K + 1 + oj >= NP || (oi == 0 && oj == 0)) continue;
+        const int si = wrap(s1 + oi), sj = wrap(s1 + oj);
+        const int r0 = (lane >> 3) * G, c0 = (lane & 3) * G;
+        FT* O = tile(si, sj);
+        const FT *L = tile(si, sK), *U = tile(sK, sj);
+        Vec acc[G];
+#pragma unroll
+        for (int i = 0; i < G; ++i) acc[i] = *(const Vec*)(O + at(r0 + i, c0, sj));
+        // pivots before the first one whose row or column reaches this tile contribute zeros
+        const int kb = max(0, (max(oi, 2 * (u % pairs)) + 1) * NB - b) / G * G;
+#pragma unroll
+        for (int k = 0; k < NB; k += G) {
+          if (k < kb) continue;
+          Vec l[G], v[G];
+#pragma unroll
+          for (int i = 0; i < G; ++i) l[i] = *(const Vec*)(L + at(r0 + i, k, sK));
+#pragma unroll
+          for (int i = 0; i < G; ++i) v[i] = *(const Vec*)(U + at(k + i, c0, sj));
+#pragma unroll
+          for (int q = 0; q < G; ++q)
+#pragma unroll
+            for (int i = 0; i < G; ++i)
+#pragma unroll
+              for (int j = 0; j < G; ++j) acc[i].v[j] -= l[i].v[q] * v[q].v[j];
+        }
+#pragma unroll
+        for (int i = 0; i < G; ++i) *(Vec*)(O + at(r0 + i, c0, sj)) = acc[i];
+      } else {
+        const int q = task - n_in - n_up, o = q <= tb ? q : q - tb;  // (K + o, K), then (K, K + o)
+        if (K + o >= NP) continue;
+        if (q <= tb) emit(K + o, K, wrap(sK + o), sK);
+        else emit(K, K + o, sK, wrap(sK + o));
+      }
+    }
+    if (!ahead) {
+      __syncthreads();  // slot K is free: the next panel's last row and column take it
+      if (K + tb + 1 < NP)
+        for (int q = wid; q < 2 * tb + 1; q += nw) enter(q, K + tb + 1, sK);
+    }
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    sK = s1;
+  }
+  return *flag;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -601,12 +806,23 @@ __device__ void band_solve(int n, int b, const FT* __restrict__ F, FT* y) {
 //     [2 BS^2 + b BS, + b BS) CU: entry (j, r) at j b + r = U[k0 - 1 - r][k0 + j]
 //
 // The explicit diagonal-block inverses replace the BS-step dependent shuffle chain of a
-// diagonal block by one short dot product per row.  One warp per block; `tmp` holds
-// BS x (BS + 1) FT per warp that takes part (`nwarps`).
+// diagonal block by one short dot product per row.  One warp per block; `tmp` (16-byte aligned)
+// holds pack_scratch<FT>() entries per warp that takes part (`nwarps`).
 // ------------------------------------------------------------------------------------------
 template <typename FT>
 __host__ __device__ constexpr int64_t packed_block_entries(int b) {
   return 2 * (int64_t)SolveBlock<FT>::BS * SolveBlock<FT>::BS + 2 * (int64_t)b * SolveBlock<FT>::BS;
+}
+
+// Rows of the scratch: padded to whole 16-byte groups, with the column reads of a warp spread over
+// the banks.
+template <typename FT>
+__host__ __device__ constexpr int pack_stride() {
+  return SolveBlock<FT>::BS + LuTile<FT>::G;
+}
+template <typename FT>
+__host__ __device__ constexpr size_t pack_scratch() {
+  return (size_t)SolveBlock<FT>::BS * pack_stride<FT>();
 }
 
 // Blocks t = first + wid, first + wid + stride, ... are packed by warp `wid` (< nwarps); one CTA
@@ -614,76 +830,108 @@ __host__ __device__ constexpr int64_t packed_block_entries(int b) {
 template <typename FT>
 __device__ void band_pack_solve_range(int n, int b, const FT* __restrict__ F, FT* __restrict__ P, FT* tmp, int nwarps,
                                       int first, int stride) {
-  constexpr int BS = SolveBlock<FT>::BS;
+  constexpr int BS = SolveBlock<FT>::BS, G = LuTile<FT>::G, LD = pack_stride<FT>(), E = BS * BS / 32, H = 32 / BS;
+  using Vec = LuVec<FT>;
   const int W = 2 * b + 1, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nblk = (n + BS - 1) / BS;
   const int64_t PB = packed_block_entries<FT>(b);
   if (wid < nwarps) {
-    FT* M = tmp + wid * BS * (BS + 1);
+    FT* M = tmp + wid * BS * LD;
+    const int hi = lane / BS, lo = lane % BS;  // a warp covers H rows of BS entries at once
+    // the inverses go out through the scratch: the column a lane holds becomes a row of the operands
+    auto store = [&](const FT (&x)[BS], FT* dst) {
+      __syncwarp();
+      if (lane < BS) {
+#pragma unroll
+        for (int i = 0; i < BS; ++i) M[lane * LD + i] = x[i];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < E; ++q) dst[q * 32 + lane] = M[(q * H + hi) * LD + lo];
+      __syncwarp();
+    };
     for (int t = first + wid; t < nblk; t += stride) {
       const int k0 = t * BS, bs = min(BS, n - k0);
       FT* out = P + (int64_t)t * PB;
-      // lower: M[i][j] = L[k0+i][k0+j] (j < i), unit diagonal
-      for (int e = lane; e < BS * BS; e += 32) {
-        const int i = e / BS, j = e % BS;
-        FT v = (FT)0;
-        if (i < bs && j < i && i - j <= b) v = F[(int64_t)(k0 + i) * W + (j - i + b)];
-        M[i * (BS + 1) + j] = v;
+      FT vl[E], vu[E];  // L_tt and U_tt (its diagonal stored inverted), entry (i, j) = (q H + hi, lo)
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        const int i = q * H + hi, j = lo;
+        const bool in = i < bs && j < bs && i - j <= b && j - i <= b;
+        const FT v = in ? F[(int64_t)(k0 + i) * W + (j - i + b)] : (i == j) ? (FT)1 : (FT)0;
+        vl[q] = (j < i) ? v : (FT)0;
+        vu[q] = (j < i) ? (FT)0 : v;
       }
+      FT x[BS];
+#pragma unroll
+      for (int q = 0; q < E; ++q) M[lo * LD + q * H + hi] = vl[q];  // transposed
       __syncwarp();
-      if (lane < BS) {
-        // column `lane` of inv(L): forward substitution with e_lane
-        FT x[BS];
+      // column `lane` of inv(L) (lanes past BS repeat one): forward substitution with e_lane, each
+      // unknown taken out of all later rows at once
 #pragma unroll
-        for (int i = 0; i < BS; ++i) {
-          FT acc = (i == lane) ? (FT)1 : (FT)0;
+      for (int i = 0; i < BS; ++i) x[i] = (i == lo) ? (FT)1 : (FT)0;
 #pragma unroll
-          for (int j = 0; j < i; ++j) acc -= M[i * (BS + 1) + j] * x[j];
-          x[i] = acc;
+      for (int j = 0; j < BS - 1; ++j)
+#pragma unroll
+        for (int g = (j + 1) / G * G; g < BS; g += G) {
+          const Vec v = *(const Vec*)(M + j * LD + g);
+#pragma unroll
+          for (int i = 0; i < G; ++i)
+            if (g + i > j) x[g + i] -= v.v[i] * x[j];
         }
+      store(x, out);
 #pragma unroll
-        for (int i = 0; i < BS; ++i) out[lane * BS + i] = x[i];
-      }
+      for (int q = 0; q < E; ++q) M[(q * H + hi) * LD + lo] = vu[q];
       __syncwarp();
-      // upper: M[i][j] = U[k0+i][k0+j] (j > i), M[i][i] = 1/U_ii (stored reciprocal)
-      for (int e = lane; e < BS * BS; e += 32) {
-        const int i = e / BS, j = e % BS;
-        FT v = (i == j) ? (FT)1 : (FT)0;
-        if (i < bs && j < bs && j >= i && j - i <= b) v = F[(int64_t)(k0 + i) * W + (j - i + b)];
-        M[i * (BS + 1) + j] = v;
-      }
-      __syncwarp();
-      if (lane < BS) {
-        // column `lane` of inv(U): backward substitution with e_lane (diagonal given inverted)
-        FT x[BS];
+      // column `lane` of inv(U): backward substitution with e_lane, row by row
 #pragma unroll
-        for (int i = BS - 1; i >= 0; --i) {
-          FT acc = (i == lane) ? (FT)1 : (FT)0;
+      for (int i = BS - 1; i >= 0; --i) {
+        FT acc = (i == lo) ? (FT)1 : (FT)0, diag = (FT)0;
 #pragma unroll
-          for (int j = i + 1; j < BS; ++j) acc -= M[i * (BS + 1) + j] * x[j];
-          x[i] = acc * M[i * (BS + 1) + i];
+        for (int g = i / G * G; g < BS; g += G) {
+          const Vec v = *(const Vec*)(M + i * LD + g);
+#pragma unroll
+          for (int j = 0; j < G; ++j) {
+            if (g + j == i) diag = v.v[j];
+            else if (g + j > i) acc -= v.v[j] * x[g + j];
+          }
         }
-#pragma unroll
-        for (int i = 0; i < BS; ++i) out[BS * BS + lane * BS + i] = x[i];
+        x[i] = acc * diag;
       }
-      // couplings (coalesced writes; the band is read once per factorization)
+      store(x, out + BS * BS);
+      // couplings, BS coupled rows at a time through the scratch: the band is read along its rows and
+      // the operands are written along the coupled rows, both coalesced
       FT* cl = out + 2 * BS * BS;
       FT* cu = cl + (int64_t)b * BS;
-      for (int e = lane; e < BS * b; e += 32) {
-        const int j = e / b, r = e % b;
-        const int il = k0 + BS + r, dl = j - BS - r + b;
-        cl[e] = (j < bs && il < n && dl >= 0) ? F[(int64_t)il * W + dl] : (FT)0;
-        const int iu = k0 - 1 - r;
-        cu[e] = (j < bs && iu >= 0 && j + 1 + r <= b) ? F[(int64_t)iu * W + (j + 1 + r + b)] : (FT)0;
+      for (int r0 = 0; r0 < b; r0 += BS) {
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+          const int r = r0 + q * H + hi, j = lo;
+          const int il = k0 + BS + r, dl = j - BS - r + b, iu = k0 - 1 - r, du = j + 1 + r + b;
+          const bool in = r < b && j < bs;
+          vl[q] = (in && il < n && dl >= 0) ? F[(int64_t)il * W + dl] : (FT)0;
+          vu[q] = (in && iu >= 0 && du <= 2 * b) ? F[(int64_t)iu * W + du] : (FT)0;
+        }
+#pragma unroll
+        for (int up = 0; up < 2; ++up) {
+#pragma unroll
+          for (int q = 0; q < E; ++q) M[(q * H + hi) * LD + lo] = up ? vu[q] : vl[q];
+          __syncwarp();
+          FT* dst = up ? cu : cl;
+          if (r0 + lo < b) {
+#pragma unroll
+            for (int q = 0; q < E; ++q) dst[(int64_t)(q * H + hi) * b + r0 + lo] = M[lo * LD + q * H + hi];
+          }
+          __syncwarp();
+        }
       }
-      __syncwarp();
     }
   }
   __syncthreads();
 }
 
 template <typename FT>
-__device__ void band_pack_solve(int n, int b, const FT* __restrict__ F, FT* __restrict__ P, FT* tmp, int nwarps) {
+__device__ __noinline__ void band_pack_solve(int n, int b, const FT* __restrict__ F, FT* __restrict__ P, FT* tmp, int nwarps) {
   band_pack_solve_range<FT>(n, b, F, P, tmp, nwarps, 0, nwarps);
 }
 

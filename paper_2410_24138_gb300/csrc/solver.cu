@@ -107,7 +107,7 @@ struct SmemPlan {
 };
 
 template <typename FT>
-__host__ __device__ inline SmemPlan smem_plan(int max_n, int max_nt, int max_b, bool with_window) {
+__host__ __device__ inline SmemPlan smem_plan(int max_n, int max_nt) {
   SmemPlan p;
   size_t o = 0;
   p.xt = o; o += sizeof(double) * max_nt;
@@ -116,13 +116,7 @@ __host__ __device__ inline SmemPlan smem_plan(int max_n, int max_nt, int max_b, 
   p.s = o; o += sizeof(double) * max_n;
   p.red = o; o += sizeof(double) * 40;
   p.yv = o; o += align_up(sizeof(FT) * max_n, 16);
-  {
-    const size_t lu = (size_t)dev::band_lu_window_rows(max_b) * dev::band_lu_window_stride(max_b);
-    const size_t inv = 2 * (size_t)dev::SolveBlock<FT>::BS * (dev::SolveBlock<FT>::BS + 1);
-    p.win = o;
-    o += with_window ? align_up(sizeof(FT) * (lu > inv ? lu : inv), 16) : 0;
-  }
-  p.rp = o; o += with_window ? align_up(sizeof(FT) * dev::band_lu_window_rows(max_b), 16) : 0;
+  p.win = p.rp = o;
   p.flag = o; o += 16;
   p.total = o;
   return p;
@@ -134,8 +128,11 @@ __host__ __device__ inline SmemPlan smem_plan(int max_n, int max_nt, int max_b, 
 // packed); the current residual, the Newton step and the refinement residual are per-subdomain
 // vectors in global memory (read and written O(n) times per phase, coalesced).
 struct LocalPlan {
-  size_t xt, racc, red, win, rp, flag, total;
+  size_t xt, racc, red, win, flag, total;
 };
+
+// Shared memory a CTA can opt in to (227 KB), less the kernels' static shared memory.
+constexpr size_t kSmemFull = 227 * 1024 - 128;
 
 // Shared memory of the harmonic extension (k_harmonic): the table state, the solve vector and
 // the window of dev::band_lu ((b + 2) rows of 2b + 1 entries, reciprocal pivots, flag), FP64.
@@ -155,20 +152,27 @@ __host__ __device__ inline SmemPlan harmonic_plan(int max_n, int max_nt, int max
 template <typename FT>
 __host__ __device__ inline LocalPlan newton_plan(int max_n, int max_nt, int max_b) {
   LocalPlan p;
+  const size_t inv = 4 * (size_t)dev::SolveBlock<FT>::BS * (dev::SolveBlock<FT>::BS + 1);
   size_t o = 0;
   p.xt = o; o += sizeof(double) * max_nt;
   p.racc = o; o += sizeof(double) * max_n;
   p.red = o; o += sizeof(double) * 40;
-  {
-    const size_t lu = (size_t)dev::band_lu_window_rows(max_b) * dev::band_lu_window_stride(max_b);
-    const size_t inv = 4 * (size_t)dev::SolveBlock<FT>::BS * (dev::SolveBlock<FT>::BS + 1);
-    size_t w = lu > inv ? lu : inv;
-    w = w > (size_t)max_n ? w : (size_t)max_n;
-    p.win = o; o += align_up(sizeof(FT) * w, 16);
-  }
-  p.rp = o; o += align_up(sizeof(FT) * dev::band_lu_window_rows(max_b), 16);
+  // the size the limit on the subdomains is stated for: a window of (b + 10) rows of the band
+  size_t lim = (size_t)dev::band_limit_rows(max_b) * dev::band_limit_stride(max_b);
+  lim = lim > inv ? lim : inv;
+  lim = lim > (size_t)max_n ? lim : (size_t)max_n;
+  lim = o + align_up(sizeof(FT) * lim, 16) + align_up(sizeof(FT) * dev::band_limit_rows(max_b), 16) + 16;
+  // the tiled window, with room for the next panel's tiles where that fits
+  o = align_up(o, 16);
+  p.win = o;
+  size_t w = dev::band_lu_window<FT>(max_b, 0);
+  w = w > inv ? w : inv;
+  w = w > (size_t)max_n ? w : (size_t)max_n;
+  const size_t full = dev::band_lu_window<FT>(max_b, 1);
+  if (full > w && o + sizeof(FT) * full + 16 <= kSmemFull) w = full;
+  o += align_up(sizeof(FT) * w, 16);
   p.flag = o; o += 16;
-  p.total = o;
+  p.total = o > lim ? o : lim;
   return p;
 }
 
@@ -180,7 +184,7 @@ __host__ __device__ inline LocalPlan apply_plan(int max_n, int max_nt) {
   p.racc = 0;
   p.red = o; o += sizeof(double) * 40;
   p.win = o; o += align_up(sizeof(FT) * max_n, 16);
-  p.rp = p.flag = o;
+  p.flag = o;
   p.total = o;
   return p;
 }
@@ -402,10 +406,12 @@ __global__ void __launch_bounds__(256) k_guess_smooth(LocalArgs A) {
 // ------------------------------------------------------------------------------------------
 // k_local_newton: the batched local corrections T_i of Eq. 4
 // ------------------------------------------------------------------------------------------
-// MAXT is the largest CTA the instantiation is compiled for: 128-thread CTAs keep three CTAs
-// per SM within the register file, 256-thread CTAs get the whole register budget per thread.
+// MAXT is the largest CTA the instantiation is compiled for: 128-thread CTAs keep four CTAs per SM
+// within the register file; 256-thread CTAs two (Eq. 1), or one with the whole register budget per
+// thread (Eq. 2, whose element tangents need it).
 template <int LAW, typename FT, int MAXT>
-__global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : 1)) k_local_newton(LocalArgs A) {
+__global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : LAW == NLS_LAW_DIFFUSION ? 2 : 1))
+    k_local_newton(LocalArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   const LocalPlan P = newton_plan<FT>(A.max_n, A.max_nt, A.max_b);
   double* xt = (double*)(smem + P.xt);
@@ -413,12 +419,11 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : 1)) k_local_newton(Lo
   double* red = (double*)(smem + P.red);
   FT* win = (FT*)(smem + P.win);
   FT* yv = win;  // the solve vector lives in the LU window once the factors are packed
-  FT* rp = (FT*)(smem + P.rp);
   int* flag = (int*)(smem + P.flag);
   __shared__ int s_item;
   const int tid = threadIdx.x, nd = A.ndof;
-  constexpr int BSI = dev::SolveBlock<FT>::BS;
-  const int inv_warps = min((int)(blockDim.x >> 5), (int)((P.rp - P.win) / (sizeof(FT) * BSI * (BSI + 1))));
+  const size_t win_cap = (P.flag - P.win) / sizeof(FT);
+  const int inv_warps = min((int)(blockDim.x >> 5), (int)(win_cap / dev::pack_scratch<FT>()));
   long long tp = clock64();
   // thread 0 charges the cycles since the last mark to phase `id` (profiling only)
   auto mark = [&](int id) {
@@ -497,7 +502,7 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : 1)) k_local_newton(Lo
       if (!stored) {
         local_jacobian<LAW, FT>(A, m, xt, csr, F);
         mark(1);
-        if (dev::band_lu_inplace<FT>(n, m.b, F, win, rp, flag)) {
+        if (dev::band_lu_inplace<FT>(n, m.b, F, win, win_cap, flag)) {
           status = ST_PIVOT;
           break;
         }
@@ -549,7 +554,7 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : 1)) k_local_newton(Lo
       local_jacobian<LAW, FT>(A, m, xt, csr, F);
       mark(5);
       if (!A.split_factor) {
-        if (dev::band_lu_inplace<FT>(n, m.b, F, win, rp, flag)) status = ST_PIVOT;
+        if (dev::band_lu_inplace<FT>(n, m.b, F, win, win_cap, flag)) status = ST_PIVOT;
         else dev::band_pack_solve<FT>(n, m.b, F, Dv, win, inv_warps);
       }
       mark(6);
@@ -583,31 +588,30 @@ template <typename FT>
 __host__ __device__ inline LocalPlan factor_plan(int max_b) {
   LocalPlan p{};
   size_t o = 0;
-  const size_t lu = (size_t)dev::band_lu_window_rows(max_b) * dev::band_lu_window_stride(max_b);
-  const size_t inv = 4 * (size_t)dev::SolveBlock<FT>::BS * (dev::SolveBlock<FT>::BS + 1);
+  const size_t lu = dev::band_lu_window<FT>(max_b, 1);
+  const size_t inv = 4 * dev::pack_scratch<FT>();
   p.win = o; o += align_up(sizeof(FT) * (lu > inv ? lu : inv), 16);
-  p.rp = o; o += align_up(sizeof(FT) * dev::band_lu_window_rows(max_b), 16);
   p.flag = o; o += 16;
   p.total = o;
   return p;
 }
 
-template <typename FT>
-__global__ void __launch_bounds__(256, 3) k_local_factor(LocalArgs A) {
+// MAXT = 256: three CTAs per SM; MAXT = 512: one, for at most one subdomain per SM.
+template <typename FT, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : 1) k_local_factor(LocalArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   const LocalPlan P = factor_plan<FT>(A.max_b);
   FT* win = (FT*)(smem + P.win);
-  FT* rp = (FT*)(smem + P.rp);
   int* flag = (int*)(smem + P.flag);
-  constexpr int BSI = dev::SolveBlock<FT>::BS;
-  const int inv_warps = min((int)(blockDim.x >> 5), (int)((P.rp - P.win) / (sizeof(FT) * BSI * (BSI + 1))));
+  const size_t win_cap = (P.flag - P.win) / sizeof(FT);
+  const int inv_warps = min((int)(blockDim.x >> 5), (int)(win_cap / dev::pack_scratch<FT>()));
   const int sub = A.order[blockIdx.x];
   const int st = A.status[sub];
   if (st == ST_NONFINITE || st == ST_PIVOT) return;
   const SubMeta m = A.meta[sub];
   FT* F = (FT*)A.factor + m.factor_off;
   FT* Dv = (FT*)A.dinv + m.dinv_off;
-  if (dev::band_lu_inplace<FT>(m.n, m.b, F, win, rp, flag)) {
+  if (dev::band_lu_inplace<FT>(m.n, m.b, F, win, win_cap, flag)) {
     if (threadIdx.x == 0) A.status[sub] = ST_PIVOT;
   } else {
     dev::band_pack_solve<FT>(m.n, m.b, F, Dv, win, inv_warps);
@@ -702,7 +706,7 @@ __global__ void __launch_bounds__(256) k_harmonic(LocalArgs A) {
 template <int LAW>
 __global__ void __launch_bounds__(256) k_galerkin(LocalArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const SmemPlan P = smem_plan<double>(A.max_n, A.max_nt, A.max_b, false);
+  const SmemPlan P = smem_plan<double>(A.max_n, A.max_nt);
   double* xt = (double*)(smem + P.xt);
   const int j = blockIdx.x, tid = threadIdx.x, nd = A.ndof;
   const SubMeta m = A.meta[j];
@@ -754,23 +758,29 @@ __global__ void k_gather_values32(int64_t n, const int32_t* src, const double* f
     to[k] = from[src[k]];
 }
 
-// coarse band factorization (one CTA)
+// coarse band factorization (one CTA); the window also holds the packing scratch of at least four
+// warps
+template <typename FT>
+__host__ __device__ constexpr size_t coarse_window(int b0) {
+  const size_t lu = dev::band_lu_window<FT>(b0, 1), inv = 4 * dev::pack_scratch<FT>();
+  return lu > inv ? lu : inv;
+}
 template <typename FT>
 __global__ void __launch_bounds__(1024) k_coarse_factor(int N0, int b0, const double* A0, FT* F, FT* Dinv, int* status) {
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int BS = dev::SolveBlock<FT>::BS;
-  const size_t R = (size_t)dev::band_lu_window_rows(b0);
   FT* win = (FT*)smem;
-  FT* rp = win + R * dev::band_lu_window_stride(b0);
-  FT* tmp = rp + R;
-  int* flag = (int*)(tmp + 4 * BS * (BS + 1));
+  int* flag = (int*)(smem + align_up(sizeof(FT) * coarse_window<FT>(b0), 16));
   const int64_t total = (int64_t)N0 * (2 * b0 + 1);
-  for (int64_t k = threadIdx.x; k < total; k += blockDim.x) F[k] = (FT)A0[k];
+  // entries left of the matrix count as zero, whatever the caller's band holds there
+  for (int64_t k = threadIdx.x; k < total; k += blockDim.x) {
+    const int d = (int)(k % (2 * b0 + 1));
+    F[k] = (k / (2 * b0 + 1) - b0 + d >= 0) ? (FT)A0[k] : (FT)0;
+  }
   __syncthreads();
-  const int bad = dev::band_lu_inplace<FT>(N0, b0, F, win, rp, flag);
-  // the LU window is free again: it holds the packing scratch of up to every warp
-  const int pw = min((int)(blockDim.x >> 5), (int)((R * dev::band_lu_window_stride(b0)) / (BS * (BS + 1))));
-  if (!bad) dev::band_pack_solve<FT>(N0, b0, F, Dinv, pw >= 4 ? win : tmp, pw >= 4 ? pw : 4);
+  const int bad = dev::band_lu_inplace<FT>(N0, b0, F, win, coarse_window<FT>(b0), flag);
+  // the LU window is free again: it holds the packing scratch
+  const int pw = min((int)(blockDim.x >> 5), (int)(coarse_window<FT>(b0) / dev::pack_scratch<FT>()));
+  if (!bad) dev::band_pack_solve<FT>(N0, b0, F, Dinv, win, pw);
   if (threadIdx.x == 0) *status = bad ? ST_PIVOT : ST_OK;
 }
 
@@ -1176,8 +1186,13 @@ inline int grid_for(int64_t n, int threads = 256) {
 // The triangular solves need warp 0 plus one thread per coupled row (32 + b threads).
 int min_local_threads(const Context& c) { return ((32 + c.ov.max_b + 31) / 32) * 32; }
 
+// 256 threads for Eq. 2, and for Eq. 1 while all subdomains are resident at two CTAs per SM: the
+// kernel is bound by latency, and a subdomain's factorization takes 0.39 ms with 256 threads against
+// 0.50 ms with 128 (n = 1598, b = 42, one CTA per SM).  With more subdomains than that, four CTAs of
+// 128 threads per SM.
 int local_threads(const Context& c) {
-  int pick = c.opt.threads_per_block ? c.opt.threads_per_block : (c.ndof == 1 ? 128 : 256);
+  int pick = c.opt.threads_per_block ? c.opt.threads_per_block
+             : (c.ndof == 1 && c.dev && c.ov.count > 2 * c.dev->nsm) ? 128 : 256;
   if (!c.opt.threads_per_block && c.dev && c.dev->newton_T) pick = c.dev->newton_T;
   return std::max(pick, min_local_threads(c));
 }
@@ -1368,9 +1383,9 @@ int newton_ctas_per_sm(Context& c) {
 bool split_local_factor(Context& c) {
   int occ = 0;
   if (fp32_local(c))
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local_factor<float>, 256, factor_plan<float>(c.ov.max_b).total));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local_factor<float, 256>, 256, factor_plan<float>(c.ov.max_b).total));
   else
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local_factor<double>, 256, factor_plan<double>(c.ov.max_b).total));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local_factor<double, 256>, 256, factor_plan<double>(c.ov.max_b).total));
   return newton_ctas_per_sm(c) == 1 && occ >= 2;
 }
 
@@ -1406,8 +1421,21 @@ void launch_local_newton(Context& c, const double* x, double* out, double load, 
   CK(cudaMemsetAsync(D.ov.queue, 0, sizeof(int32_t), D.s));
   dispatch_local_newton(c, c.ov, A, local_threads(c));
   if (A.split_factor) {
-    if (fp32_local(c)) LAUNCH(D, k_local_factor<float>, c.ov.count, 256, factor_plan<float>(c.ov.max_b).total, A);
-    else LAUNCH(D, k_local_factor<double>, c.ov.count, 256, factor_plan<double>(c.ov.max_b).total, A);
+    // 512 threads shorten one factorization (1.01 against 1.15 ms at n = 3120, b = 83), three CTAs of
+    // 256 threads per SM finish more of them: the larger CTA while every subdomain has an SM
+    const bool big = c.ov.count <= D.nsm;
+    auto run = [&](auto kernel, const char* name, size_t sm) {
+      LAUNCH_NAMED(D, name, kernel, c.ov.count, big ? 512 : 256, sm, A);
+    };
+    if (fp32_local(c)) {
+      const size_t sm = factor_plan<float>(c.ov.max_b).total;
+      big ? run(k_local_factor<float, 512>, "k_local_factor<float>", sm)
+          : run(k_local_factor<float, 256>, "k_local_factor<float>", sm);
+    } else {
+      const size_t sm = factor_plan<double>(c.ov.max_b).total;
+      big ? run(k_local_factor<double, 512>, "k_local_factor<double>", sm)
+          : run(k_local_factor<double, 256>, "k_local_factor<double>", sm);
+    }
   }
 }
 
@@ -1510,11 +1538,15 @@ LocalArgs coarse_args(Context& c) {
   return A;
 }
 
+// Shared memory of the one-CTA band factorization; never less than the window of (b + 10) band
+// rows that the limit on its half bandwidth is stated for.
 size_t coarse_factor_smem(const Context& c, bool f32) {
   const size_t fs = f32 ? sizeof(float) : sizeof(double);
   const size_t BS = f32 ? dev::SolveBlock<float>::BS : dev::SolveBlock<double>::BS;
-  const size_t R = (size_t)dev::band_lu_window_rows(c.cs.b0);
-  return fs * (R * dev::band_lu_window_stride(c.cs.b0) + R + 4 * BS * (BS + 1)) + 16;
+  const size_t R = (size_t)dev::band_limit_rows(c.cs.b0);
+  const size_t lim = fs * (R * dev::band_limit_stride(c.cs.b0) + R + 4 * BS * (BS + 1)) + 16;
+  const size_t need = align_up(fs * (f32 ? coarse_window<float>(c.cs.b0) : coarse_window<double>(c.cs.b0)), 16) + 16;
+  return std::max(lim, need);
 }
 
 // A_0(x) = P_0^T DF(x) P_0 -> band -> factor.  Returns false on a bad pivot.
@@ -1547,7 +1579,7 @@ void coarse_assemble_launch(Context& c, const double* x) {
   LocalArgs A = coarse_args(c);
   A.x = x;
   const int T = 256;
-  const size_t sm = smem_plan<double>(c.nov.max_n, c.nov.max_nt, c.nov.max_b, false).total;
+  const size_t sm = smem_plan<double>(c.nov.max_n, c.nov.max_nt).total;
   if (c.law == NLS_LAW_DIFFUSION) LAUNCH(D, (k_galerkin<NLS_LAW_DIFFUSION>), c.nov.count, T, sm, A);
   else LAUNCH(D, (k_galerkin<NLS_LAW_NEOHOOKE>), c.nov.count, T, sm, A);
   const int64_t ne = (int64_t)c.cs.N0 * (2 * c.cs.b0 + 1);
@@ -1910,8 +1942,10 @@ int device_setup(Context& c) {
     set_smem(k_local_newton<NLS_LAW_NEOHOOKE, float, 256>, lim);
     set_smem(k_local_newton<NLS_LAW_NEOHOOKE, double, 256>, lim);
     set_smem(k_local_apply<float>, lim);
-    set_smem(k_local_factor<float>, lim);
-    set_smem(k_local_factor<double>, lim);
+    set_smem(k_local_factor<float, 256>, lim);
+    set_smem(k_local_factor<double, 256>, lim);
+    set_smem(k_local_factor<float, 512>, lim);
+    set_smem(k_local_factor<double, 512>, lim);
     set_smem(k_guess_smooth<NLS_LAW_DIFFUSION>, lim);
     set_smem(k_guess_smooth<NLS_LAW_NEOHOOKE>, lim);
     set_smem(k_local_apply<double>, lim);
