@@ -104,6 +104,7 @@ struct Dev {
   int64_t* star_ptr = nullptr;  // node stars (ascending element ids) for the global residual's node sums
   int32_t* star_ref = nullptr;  // e nen + a per star entry
   double* Re = nullptr;         // element residuals [e][a][dof]
+  double2* logtab = nullptr;  // table of the element routines' logarithm (Eq. 2)
   double *geom = nullptr, *kcoef = nullptr, *fext = nullptr, *ubc = nullptr, *g_val = nullptr;
   uint8_t* free_dof = nullptr;
   DeviceLocalSet ov, nov;

@@ -72,7 +72,8 @@ struct LocalArgs {
   const int32_t* order;
   int32_t* queue;
   const double *geom, *kcoef, *fext;
-  double mu, lam, load;
+  dev::NHLaw nh;  // Eq. 2
+  double load;
   int ndof, nen, count, max_n, max_nt, max_b;
   double rtol, atol, armijo, ir_rtol;
   int maxit, ls_trials, ir_max;
@@ -224,7 +225,7 @@ __device__ bool local_residual(const LocalArgs& A, const SubMeta& m, const doubl
           ue[2 * a + 1] = xt[2 * lc[a] + 1];
         }
         bool eok = true;
-        dev::nh_residual(geo, ue, A.mu, A.lam, re, eok);
+        dev::nh_residual(geo, ue, A.nh, re, eok);
         ok = ok && eok;
 #pragma unroll
         for (int a = 0; a < 4; ++a)
@@ -296,19 +297,17 @@ __device__ void local_jacobian(const LocalArgs& A, const SubMeta& m, const doubl
           ue[2 * a] = xt[2 * lc[a]];
           ue[2 * a + 1] = xt[2 * lc[a] + 1];
         }
-        dev::NHGauss G;
-        dev::nh_gauss(geo, ue, A.mu, A.lam, G);
-#pragma unroll 1
+        dev::NHTangent K;
+        dev::nh_tangent(geo, ue, A.nh, K);
+#pragma unroll
         for (int a = 0; a < 4; ++a) {
-          double R[16];
-          dev::nh_tangent_rows(geo, G, A.mu, A.lam, a, R);
           const int32_t* epa = ep + 16 * a;  // rows (a, 0) and (a, 1): 16 consecutive targets
           double oc[16];
 #pragma unroll
           for (int q = 0; q < 16; ++q) oc[q] = (epa[q] >= 0) ? csr[epa[q]] : 0.0;
 #pragma unroll
           for (int q = 0; q < 16; ++q)
-            if (epa[q] >= 0) csr[epa[q]] = oc[q] + R[q];
+            if (epa[q] >= 0) csr[epa[q]] = oc[q] + K(a, q >> 3, (q & 7) >> 1, q & 1);
           if (band && lc[a] < m.nV) {
 #pragma unroll
             for (int b = 0; b < 4; ++b)
@@ -318,7 +317,7 @@ __device__ void local_jacobian(const LocalArgs& A, const SubMeta& m, const doubl
 #pragma unroll
                   for (int db = 0; db < 2; ++db) {
                     const int row = 2 * lc[a] + da, col = 2 * lc[b] + db;
-                    band[(int64_t)row * W + (col - row + m.b)] += (FT)R[da * 8 + 2 * b + db];
+                    band[(int64_t)row * W + (col - row + m.b)] += (FT)K(a, da, b, db);
                   }
               }
           }
@@ -704,7 +703,7 @@ __global__ void __launch_bounds__(256) k_harmonic(LocalArgs A) {
 }
 
 template <int LAW>
-__global__ void __launch_bounds__(256) k_galerkin(LocalArgs A) {
+__global__ void __launch_bounds__(256, 2) k_galerkin(LocalArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   const SmemPlan P = smem_plan<double>(A.max_n, A.max_nt);
   double* xt = (double*)(smem + P.xt);
@@ -924,7 +923,7 @@ __global__ void __launch_bounds__(512) k_coarse_band_solve(int N0, int b0, const
 // into Re[(e nen + a) ndof + d]; k_node_residual adds them up per node.
 template <int LAW>
 __global__ void k_elem_residual(int64_t ne, const int32_t* conn, const double* geom, const double* kcoef,
-                                const double* x, double* Re, double mu, double lam, int* bad) {
+                                const double* x, double* Re, dev::NHLaw nh, int* bad) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne; e += (int64_t)gridDim.x * blockDim.x) {
     if (LAW == NLS_LAW_DIFFUSION) {
       const int32_t* c = conn + e * 3;
@@ -944,7 +943,7 @@ __global__ void k_elem_residual(int64_t ne, const int32_t* conn, const double* g
         ue[2 * a + 1] = x[2 * (int64_t)c[a] + 1];
       }
       bool ok = true;
-      dev::nh_residual(geo, ue, mu, lam, re, ok);
+      dev::nh_residual(geo, ue, nh, re, ok);
       if (!ok) *bad = 1;
 #pragma unroll
       for (int q = 0; q < 8; ++q) Re[e * 8 + q] = re[q];
@@ -975,8 +974,8 @@ __global__ void k_node_residual(int64_t n_nodes, int nd, const int64_t* star_ptr
 
 template <int LAW>
 __global__ void k_global_jacobian(const int32_t* elems, int e0, int e1, const int32_t* conn, const double* geom,
-                                  const double* kcoef, const double* x, const int32_t* epos, double* val, double mu,
-                                  double lam) {
+                                  const double* kcoef, const double* x, const int32_t* epos, double* val,
+                                  dev::NHLaw nh) {
   for (int i = e0 + blockIdx.x * blockDim.x + threadIdx.x; i < e1; i += gridDim.x * blockDim.x) {
     const int32_t e = elems[i];
     if (LAW == NLS_LAW_DIFFUSION) {
@@ -997,16 +996,11 @@ __global__ void k_global_jacobian(const int32_t* elems, int e0, int e1, const in
         ue[2 * a] = x[2 * (int64_t)c[a]];
         ue[2 * a + 1] = x[2 * (int64_t)c[a] + 1];
       }
-      dev::NHGauss G;
-      dev::nh_gauss(geo, ue, mu, lam, G);
+      dev::NHTangent K;
+      dev::nh_tangent(geo, ue, nh, K);
       const int32_t* ep = epos + (int64_t)e * 64;
-#pragma unroll 1
-      for (int a = 0; a < 4; ++a) {
-        double R[16];
-        dev::nh_tangent_rows(geo, G, mu, lam, a, R);
 #pragma unroll
-        for (int q = 0; q < 16; ++q) val[ep[16 * a + q]] += R[q];
-      }
+      for (int q = 0; q < 64; ++q) val[ep[q]] += K(q >> 4, (q >> 3) & 1, (q & 7) >> 1, q & 1);
     }
   }
 }
@@ -1219,6 +1213,32 @@ bool coarse_tiles(const Context& c) {
 // CTA size of the one-CTA coarse band solves: warp 0 plus one thread per coupled row.
 int coarse_solve_threads(const Context& c) { return std::max(256, (32 + c.cs.b0 + 31) / 32 * 32); }
 
+dev::NHLaw nh_law(const Context& c) {
+  dev::NHLaw law;
+  lame(c, law.mu, law.lam);
+  law.tab = c.dev->logtab;
+  return law;
+}
+
+// The table of dev::log_inv: per bin of m in [0.75, 1.5) the reciprocal r of its middle (1 for the two
+// bins next to 1, where log must keep its relative accuracy) and -log r.
+std::vector<double2> log_table() {
+  auto from_hi = [](uint32_t hi) {
+    const uint64_t bits = (uint64_t)hi << 32;
+    double x;
+    std::memcpy(&x, &bits, sizeof(x));
+    return x;
+  };
+  std::vector<double2> t(dev::kLogBins);
+  for (int i = 0; i < dev::kLogBins; ++i) {
+    const double a = from_hi(0x3fe80000u + ((uint32_t)i << 13)), b = from_hi(0x3fe80000u + ((uint32_t)(i + 1) << 13));
+    const double r = (a == 1.0 || b == 1.0) ? 1.0 : (double)(2.0L / ((long double)a + (long double)b));
+    t[i].x = r;
+    t[i].y = (double)-std::log((long double)r);
+  }
+  return t;
+}
+
 LocalArgs make_args(const Context& c, const LocalSet& hs, const DeviceLocalSet& ds) {
   LocalArgs A;
   std::memset(&A, 0, sizeof(A));
@@ -1247,7 +1267,7 @@ LocalArgs make_args(const Context& c, const LocalSet& hs, const DeviceLocalSet& 
   A.geom = D.geom;
   A.kcoef = D.kcoef;
   A.fext = D.fext;
-  lame(c, A.mu, A.lam);
+  A.nh = nh_law(c);
   A.load = 1.0;
   A.ndof = c.ndof;
   A.nen = c.nen;
@@ -1296,31 +1316,29 @@ double norm2(Dev& D, int64_t n, const double* x) {
 // ---- global residual / Jacobian ------------------------------------------------------------
 void global_residual(Context& c, const double* x, double* F, double load) {
   Dev& D = *c.dev;
-  double mu, lam;
-  lame(c, mu, lam);
+  const dev::NHLaw nh = nh_law(c);
   if (c.law == NLS_LAW_DIFFUSION)
     LAUNCH(D, k_elem_residual<NLS_LAW_DIFFUSION>, grid_for(c.n_elems), 256, 0, c.n_elems, D.conn, D.geom, D.kcoef, x,
-           D.Re, mu, lam, D.bad);
+           D.Re, nh, D.bad);
   else
     LAUNCH(D, k_elem_residual<NLS_LAW_NEOHOOKE>, grid_for(c.n_elems), 256, 0, c.n_elems, D.conn, D.geom, D.kcoef, x,
-           D.Re, mu, lam, D.bad);
+           D.Re, nh, D.bad);
   LAUNCH(D, k_node_residual, grid_for(c.n_nodes), 256, 0, c.n_nodes, c.ndof, D.star_ptr, D.star_ref, D.Re, load,
          D.fext, D.free_dof, F);
 }
 
 void global_jacobian(Context& c, const double* x) {
   Dev& D = *c.dev;
-  double mu, lam;
-  lame(c, mu, lam);
+  const dev::NHLaw nh = nh_law(c);
   CK(cudaMemsetAsync(D.g_val, 0, sizeof(double) * c.g_col.size(), D.s));
   for (size_t k = 0; k + 1 < c.g_color_ptr.size(); ++k) {
     const int e0 = c.g_color_ptr[k], e1 = c.g_color_ptr[k + 1];
     if (c.law == NLS_LAW_DIFFUSION)
       LAUNCH(D, (k_global_jacobian<NLS_LAW_DIFFUSION>), grid_for(e1 - e0), 256, 0, D.g_elem, e0, e1, D.conn, D.geom,
-             D.kcoef, x, D.g_epos, D.g_val, mu, lam);
+             D.kcoef, x, D.g_epos, D.g_val, nh);
     else
       LAUNCH(D, (k_global_jacobian<NLS_LAW_NEOHOOKE>), grid_for(e1 - e0), 256, 0, D.g_elem, e0, e1, D.conn, D.geom,
-             D.kcoef, x, D.g_epos, D.g_val, mu, lam);
+             D.kcoef, x, D.g_epos, D.g_val, nh);
   }
 }
 
@@ -1862,6 +1880,7 @@ int device_setup(Context& c) {
     D.smem_optin = prop.sharedMemPerBlockOptin;
     D.conn = D.upload(c.conn);
     D.geom = D.upload(c.geom);
+    D.logtab = D.upload(log_table());
     std::vector<double> k = c.k_elem;
     if (k.empty()) k.assign(c.n_elems, 1.0);
     D.kcoef = D.upload(k);
