@@ -349,7 +349,7 @@ int nls_get_sizes(const nls_ctx* ctx, nls_sizes* o) {
   o->coarse_half_band = c.cs.b0;
   o->device_bytes = c.device_bytes;
   o->total_factor_entries = c.ov.total_factor;
-  o->total_local_nnz = c.ov.total_nnz;
+  o->total_local_nnz = c.ov.total_entries;
   o->total_table_dofs = c.ov.total_nt;
   o->factor_bytes = (c.opt.local_precision == NLS_PREC_FP32_IR) ? 4 : 8;
   o->total_solve_entries = 0;

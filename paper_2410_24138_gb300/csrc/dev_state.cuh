@@ -140,6 +140,7 @@ struct Dev {
   bool local_reuse_active = false;   // chord steps allowed (inside nls_solve with local_reuse)
   int clock_khz = 1;
   double* h_scal = nullptr;  // pinned
+  int *err_host = nullptr, *err_dev = nullptr;  // host-mapped: a local solve gave up waiting
   int m = 0;                 // GMRES restart length allocated
   bool tangent_ready = false;
   void* guess = nullptr;  // learned-guess attachment (guess.cu)

@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "nls_internal.h"
+#include "tcgen05.cuh"
 
 namespace nls {
 namespace dev {
@@ -1124,6 +1125,185 @@ __device__ void band_solve_packed(int n, int b, const FT* __restrict__ P, FT* y,
       for (int j = 0; j < BS; ++j) buf[0][j] = buf[NB - 1][j];
     }
   }
+}
+
+// ------------------------------------------------------------------------------------------
+// The same triangular solves with the operands streamed through shared memory.
+//
+// What bounds them: 2 ceil(n / BS) dependent block steps, each reading BS (BS + b) operand entries
+// once (15 KB in FP32 at b = 85).  With the operands in registers one step ahead, a step waited for
+// L2 (about 1400 cycles a step with one CTA per SM); here one thread of an extra warp keeps `stages`
+// blocks in flight by bulk copies (cp.async.bulk on mbarriers), and the chain of a step is warp 0's
+// alone: it applies the diagonal inverse, takes the coupling to the next block's rows itself and goes
+// on, while the other warps add the coupling to the rows beyond; one named barrier of the solving
+// warps per step keeps the order of the additions to every row, so the results are bit for bit those
+// of band_solve_packed.
+//
+// Ring in shared memory (16-byte aligned): 128 bytes of mbarriers and a flag, then the stages, each
+// the diagonal inverse and the coupling of one block and direction.  y: nblk BS entries, 16-byte
+// aligned.  Needs ring_threads(b) threads and two stages; every thread of the CTA calls it, after a
+// barrier that follows the writes of y and P.  Returns false if a bounded wait gave up.
+// ------------------------------------------------------------------------------------------
+constexpr int kRingMax = 6;
+constexpr int kRingHead = 128;
+template <typename FT>
+__host__ __device__ constexpr int ring_warps(int b) {  // warps that solve: warp 0 and the rows past the next block
+  return 1 + (b > SolveBlock<FT>::BS ? (b - SolveBlock<FT>::BS + 31) / 32 : 0);
+}
+template <typename FT>
+__host__ __device__ constexpr int ring_threads(int b) {
+  return 32 * (ring_warps<FT>(b) + 1);
+}
+template <typename FT>
+__host__ __device__ constexpr size_t ring_stage_bytes(int b) {
+  return sizeof(FT) * SolveBlock<FT>::BS * (size_t)(SolveBlock<FT>::BS + b);
+}
+template <typename FT>
+__host__ __device__ constexpr int ring_stages(int b, size_t bytes) {
+  const size_t s = bytes < kRingHead ? 0 : (bytes - kRingHead) / ring_stage_bytes<FT>(b);
+  return s < kRingMax ? (int)s : kRingMax;
+}
+
+// sum_j c(j) x[j] over a block in the order of band_solve_packed: even and odd j apart
+template <typename FT, typename C>
+__device__ __forceinline__ FT block_dot(C&& c, const FT* x) {
+  constexpr int BS = SolveBlock<FT>::BS, G = LuTile<FT>::G;
+  FT a0 = 0, a1 = 0;
+#pragma unroll
+  for (int j = 0; j < BS; j += G) {
+    const LuVec<FT> v = *(const LuVec<FT>*)(x + j);
+#pragma unroll
+    for (int q = 0; q < G; q += 2) {
+      a0 += c(j + q) * v.v[q];
+      a1 += c(j + q + 1) * v.v[q + 1];
+    }
+  }
+  return a0 + a1;
+}
+
+template <typename FT>
+__device__ __noinline__ bool band_solve_ring(int n, int b, const FT* __restrict__ P, FT* y, unsigned char* ring,
+                                             int stages, int l2d) {
+  constexpr int BS = SolveBlock<FT>::BS;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int cw = ring_warps<FT>(b), nblk = (n + BS - 1) / BS, steps = 2 * nblk;
+  const int64_t PB = packed_block_entries<FT>(b);
+  uint64_t* full = (uint64_t*)ring;
+  uint64_t* empty = full + kRingMax;
+  volatile int* dead = (volatile int*)(empty + kRingMax);
+  if (tid == 0) {
+    for (int q = 0; q < stages; ++q) {
+      tc::mbar_init(full + q, 1);
+      tc::mbar_init(empty + q, cw);
+    }
+    *dead = 0;
+    tc::mbar_init_fence();
+  }
+  for (int a = n + tid; a < nblk * BS; a += blockDim.x) y[a] = (FT)0;
+  // the packed operands and whatever the ring's memory held were written by ordinary stores; the
+  // copies below go through the asynchronous proxy
+  asm volatile("fence.proxy.async;" ::: "memory");
+  __syncthreads();
+  const size_t sb = ring_stage_bytes<FT>(b);
+  if (wid == cw) {
+    if (lane == 0) {
+      const uint32_t dbytes = sizeof(FT) * BS * BS, cbytes = (uint32_t)(sizeof(FT) * BS * b);
+      auto block = [&](int s, const FT*& d, const FT*& c) {  // operands of step s
+        const bool fwd = s < nblk;
+        const FT* Pt = P + (int64_t)(fwd ? s : steps - 1 - s) * PB;
+        d = Pt + (fwd ? 0 : BS * BS);
+        c = Pt + 2 * BS * BS + (fwd ? 0 : (int64_t)b * BS);
+      };
+      int st = 0;
+      uint32_t par = 1;  // parity of the previous use of the stage
+      int issued = 0;
+      for (int s = 0; s < steps; ++s) {
+        if (s >= stages && !tc::mbar_wait(empty + st, par)) {
+          *dead = 1;
+          break;
+        }
+        const FT *d, *c;
+        if (l2d > 0 && s + l2d < steps) {
+          block(s + l2d, d, c);
+          tc::bulk_prefetch_l2(d, dbytes);
+          if (cbytes) tc::bulk_prefetch_l2(c, cbytes);
+        }
+        block(s, d, c);
+        unsigned char* dst = ring + kRingHead + st * sb;
+        tc::mbar_arrive_expect_tx(full + st, dbytes + cbytes);
+        tc::bulk_load(dst, d, dbytes, full + st);
+        if (cbytes) tc::bulk_load(dst + dbytes, c, cbytes, full + st);
+        issued = s + 1;
+        if (++st == stages) {
+          st = 0;
+          par ^= 1;
+        }
+      }
+      if (issued < steps) {  // gave up: see the copies in flight land before the memory is used again
+        for (int s = issued > stages ? issued - stages : 0; s < issued; ++s)
+          tc::mbar_wait(full + s % stages, (uint32_t)(s / stages) & 1u);
+      }
+    }
+    __syncwarp();
+  } else if (wid < cw) {
+    const int r = wid == 0 ? lane % BS : BS + tid - 32;  // coupled row of this thread
+    const bool mine = r < b && (wid > 0 || lane < BS);
+    int st = 0;
+    uint32_t par = 0;
+    bool live = true;
+    for (int s = 0; s < steps; ++s) {
+      const bool fwd = s < nblk;
+      const int k0 = (fwd ? s : steps - 1 - s) * BS;
+      const FT* D = (const FT*)(ring + kRingHead + st * sb);
+      const FT* C = D + BS * BS + r;
+      if (live && !tc::mbar_wait(full + st, par)) {
+        live = false;
+        *dead = 1;
+      }
+      __syncwarp();
+      FT c[BS];
+      if (wid == 0) {
+        // x = (diagonal inverse) y; FP64: the even terms on lanes 0 .. 15, the odd ones on 16 .. 31
+        FT x;
+        if constexpr (BS == 32) {
+          x = block_dot<FT>([&](int j) { return D[j * BS + lane]; }, y + k0);
+        } else {
+          x = 0;
+#pragma unroll
+          for (int j = 0; j < BS; j += 2) x += D[(j + lane / BS) * BS + lane % BS] * y[k0 + j + lane / BS];
+          x += __shfl_xor_sync(0xffffffffu, x, BS);
+        }
+        if (mine) {
+#pragma unroll
+          for (int j = 0; j < BS; ++j) c[j] = C[j * b];
+        }
+        __syncwarp();
+        if (lane < BS && k0 + lane < n) y[k0 + lane] = x;
+      } else if (mine) {
+#pragma unroll
+        for (int j = 0; j < BS; ++j) c[j] = C[j * b];
+      }
+      if (cw > 1) asm volatile("bar.sync 1, %0;" ::"r"(32 * cw) : "memory");
+      else __syncwarp();
+      const int i = fwd ? k0 + BS + r : k0 - 1 - r;
+      if (mine && i >= 0 && i < n) y[i] -= block_dot<FT>([&](int j) { return c[j]; }, y + k0);
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(empty + st);
+      if (++st == stages) {
+        st = 0;
+        par ^= 1;
+      }
+    }
+  }
+  __syncthreads();
+  const bool ok = *dead == 0;
+  __syncthreads();
+  if (tid == 0)
+    for (int q = 0; q < stages; ++q) {
+      tc::mbar_inval(full + q);
+      tc::mbar_inval(empty + q);
+    }
+  return ok;
 }
 
 }  // namespace dev

@@ -17,7 +17,9 @@ struct SubMeta {
   int32_t b;       // half bandwidth of the local matrix over the local unknowns
   int32_t ne;      // elements
   int32_t ncolor;  // element colours (no two elements of one colour share a node)
-  int32_t nrows;   // CSR rows: n (local rows only) or nt (full Neumann rows)
+  int32_t nrows;   // matrix rows: n (local rows only) or nt (full Neumann rows)
+  int32_t slice;   // local rows: rows per slice of the sliced layout (see LocalSet::rowptr); 0: plain CSR
+  int32_t pad;
   int64_t tnode_off, elem_off, color_off, rowptr_off, nnz_off, nnz, factor_off, vec_off, epos_off;
   int64_t dinv_off;  // packed solve operands of the factors: packed_solve_entries(n, b) entries
 };
@@ -38,13 +40,19 @@ struct LocalSet {
   std::vector<int32_t> elem_gid;    // elements, sorted by (colour, id) per subdomain
   std::vector<int32_t> lconn;       // [elem][nen] table node index
   std::vector<int32_t> color_ptr;   // [ncolor + 1] per subdomain, relative element index
-  std::vector<int32_t> rowptr;      // [nrows + 1] per subdomain, relative
+  // Rows of the local matrices.  Neumann rows (the coarse space's): CSR, rowptr [nrows + 1] per
+  // subdomain.  Local rows: slices of `slice` rows (32, or 1), entry k of row a at
+  // base(a / slice) + k height + a % slice, height = the slice's rows, width = its longest row's
+  // entries; rowptr holds {base, width} per slice.  Shorter rows are padded with the row's own column
+  // (and a value that stays zero).  A warp of consecutive rows then reads consecutive entries.
+  std::vector<int32_t> rowptr;      // relative
   std::vector<int32_t> colidx;      // table dof index
-  std::vector<int32_t> epos;        // [elem][(nen*ndof)^2] CSR position (relative), -1 = row not stored
+  std::vector<int32_t> epos;        // [elem][(nen*ndof)^2] value position (relative), -1 = row not stored
   std::vector<uint8_t> owned;       // per local unknown
   std::vector<int32_t> overlap_sorted_elems;  // elements ascending (for inspection)
   std::vector<int64_t> overlap_sorted_off;
-  int64_t total_n = 0, total_nt = 0, total_nnz = 0, total_factor = 0, total_epos = 0, total_dinv = 0;
+  // total_nnz: stored values, padding included; total_entries: entries of the matrices
+  int64_t total_n = 0, total_nt = 0, total_nnz = 0, total_entries = 0, total_factor = 0, total_epos = 0, total_dinv = 0;
   int max_n = 0, max_nt = 0, max_b = 0, max_ne = 0, max_nrows = 0;
 };
 

@@ -41,8 +41,45 @@ struct SubBuild {
   std::vector<int32_t> color_ptr;
   std::vector<int32_t> rowptr, colidx, epos;
   std::vector<uint8_t> owned;
-  int b = 0;
+  int b = 0, nrows = 0, slice = 0;
+  int64_t entries = 0;
 };
+
+// CSR rows into slices (LocalSet::rowptr): of 32 rows unless the padding would exceed one value per
+// row, then of one row, which stores exactly the entries.  The element positions follow.
+void slice_rows(SubBuild& s) {
+  const int n = s.nrows;
+  std::vector<int32_t> table, col;
+  std::vector<int32_t> move(s.colidx.size());
+  for (int h : {32, 1}) {
+    table.clear();
+    int64_t base = 0;
+    for (int a0 = 0; a0 < n; a0 += h) {
+      const int rows = std::min(h, n - a0);
+      int width = 0;
+      for (int a = a0; a < a0 + rows; ++a) width = std::max(width, s.rowptr[a + 1] - s.rowptr[a]);
+      table.push_back((int32_t)base);
+      table.push_back(width);
+      base += (int64_t)width * rows;
+    }
+    if (h > 1 && base > s.entries + n) continue;
+    col.resize(base);
+    for (int a = 0; a < n; ++a) {
+      const int q = a / h, rows = std::min(h, n - q * h), len = s.rowptr[a + 1] - s.rowptr[a];
+      for (int k = 0; k < table[2 * q + 1]; ++k) {
+        const int32_t at = table[2 * q] + k * rows + a % h;
+        col[at] = k < len ? s.colidx[s.rowptr[a] + k] : a;
+        if (k < len) move[s.rowptr[a] + k] = at;
+      }
+    }
+    s.slice = h;
+    break;
+  }
+  for (auto& e : s.epos)
+    if (e >= 0) e = move[e];
+  s.rowptr.swap(table);
+  s.colidx.swap(col);
+}
 
 void build_one(const Context& c, const std::vector<int32_t>& base, int layers, bool neumann, int sub_id,
                Scratch& sc, SubBuild& out) {
@@ -167,6 +204,9 @@ void build_one(const Context& c, const std::vector<int32_t>& base, int layers, b
           }
       }
     }
+  out.nrows = row_nodes * nd;
+  out.entries = (int64_t)out.colidx.size();
+  if (!neumann) slice_rows(out);
   out.owned.assign(out.nV * nd, 0);
   for (int t = 0; t < out.nV; ++t)
     for (int d = 0; d < nd; ++d) out.owned[t * nd + d] = (c.owner[out.tnodes[t]] == sub_id) ? 1 : 0;
@@ -212,7 +252,9 @@ void build_local_set(Context& c, LocalSet& s, int layers, bool neumann_rows, boo
     m.b = p.b;
     m.ne = (int32_t)p.elems.size();
     m.ncolor = (int32_t)p.color_ptr.size() - 1;
-    m.nrows = (int32_t)p.rowptr.size() - 1;
+    m.nrows = p.nrows;
+    m.slice = p.slice;
+    m.pad = 0;
     m.tnode_off = tn;
     m.elem_off = el;
     m.color_off = co;
@@ -226,7 +268,8 @@ void build_local_set(Context& c, LocalSet& s, int layers, bool neumann_rows, boo
     tn += m.nT;
     el += m.ne;
     co += m.ncolor + 1;
-    rp += m.nrows + 1;
+    rp += (int64_t)p.rowptr.size();
+    s.total_entries += p.entries;
     nz += m.nnz;
     fa += (int64_t)m.n * (2 * m.b + 1);
     ve += m.n;

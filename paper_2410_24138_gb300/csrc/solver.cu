@@ -64,7 +64,7 @@ struct LocalArgs {
   void* factor;
   void* dinv;  // packed triangular-solve operands (diagonal-block inverses + couplings)
   double* wbuf;
-  double* work;        // three per-subdomain FP64 vectors (vec_off), `work_stride` apart
+  double* work;        // two per-subdomain FP64 vectors (vec_off), `work_stride` apart
   int64_t work_stride;
   int32_t *its, *status;
   int32_t* chord;  // per subdomain: steps of the last launch taken with the stored factors
@@ -78,6 +78,8 @@ struct LocalArgs {
   double rtol, atol, armijo, ir_rtol;
   int maxit, ls_trials, ir_max;
   int l2_dist;            // L2 prefetch distance of the triangular solves (blocks; 0 = off)
+  int ring;               // tangent application: stages of the operand ring (0: operands in registers)
+  int* err;               // host-mapped: set when a bounded wait gave up
   const double* x;        // evaluation point (global)
   double* out;            // F_x: owned entries receive x - w
   const double* guess;    // optional start states (concatenated local vectors)
@@ -177,15 +179,19 @@ __host__ __device__ inline LocalPlan newton_plan(int max_n, int max_nt, int max_
   return p;
 }
 
+// Tangent application: the table vector (later the refined solution), the reductions, the solve
+// vector and `stages` stages of the ring.
 template <typename FT>
-__host__ __device__ inline LocalPlan apply_plan(int max_n, int max_nt) {
+__host__ __device__ inline LocalPlan apply_plan(int max_n, int max_nt, int max_b, int stages) {
   LocalPlan p;
   size_t o = 0;
   p.xt = o; o += sizeof(double) * max_nt;
   p.racc = 0;
   p.red = o; o += sizeof(double) * 40;
-  p.win = o; o += align_up(sizeof(FT) * max_n, 16);
+  o = align_up(o, 16);
+  p.win = o; o += align_up(sizeof(FT) * align_up(max_n, dev::SolveBlock<FT>::BS), 16);
   p.flag = o;
+  if (stages) o += dev::kRingHead + stages * dev::ring_stage_bytes<FT>(max_b);
   p.total = o;
   return p;
 }
@@ -328,42 +334,75 @@ __device__ void local_jacobian(const LocalArgs& A, const SubMeta& m, const doubl
   }
 }
 
-// s = J^-1 rhs with the band factors, then FP64 iterative refinement against the CSR matrix
-// (columns < n) when the factors are FP32.  `res` is an n-vector of scratch.
+// f(value, column) over the entries of local row a, in ascending column order
+template <typename F>
+__device__ __forceinline__ void for_row(const LocalArgs& A, const SubMeta& m, int a, F&& f) {
+  const int q = m.slice == 32 ? a >> 5 : a, h = m.slice == 32 ? min(32, m.n - (a & ~31)) : 1;
+  const int2 bw = *(const int2*)(A.rowptr + m.rowptr_off + 2 * q);
+  const int64_t first = m.nnz_off + bw.x + (m.slice == 32 ? a & 31 : 0);
+  const double* v = A.csr + first;
+  const int32_t* c = A.colidx + first;
+  for (int k = 0; k < bw.y; k += 6) {
+    double val[6];
+    int32_t col[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const bool in = k + i < bw.y;
+      val[i] = in ? v[(k + i) * h] : 0.0;
+      col[i] = in ? c[(k + i) * h] : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+      if (k + i < bw.y) f(val[i], col[i]);
+  }
+}
+
+// y = (packed operands)^-1 y through the ring where it has two stages and the CTA the threads, else
+// with the operands in registers.  Returns false if a bounded wait gave up.
+struct Ring {
+  unsigned char* mem;
+  int stages;
+};
 template <typename FT, bool PF>
-__device__ int local_solve(const LocalArgs& A, const SubMeta& m, const int32_t* rowptr, const int32_t* colidx,
-                           const double* csr, const FT* Dv, const double* rhs, double rhs_norm, double* s,
-                           double* res, FT* yv, double* red) {
+__device__ bool triangular_solves(const LocalArgs& A, const SubMeta& m, const FT* Dv, FT* yv, const Ring& ring) {
+  if (ring.stages >= 2 && (int)blockDim.x >= dev::ring_threads<FT>(m.b))
+    return dev::band_solve_ring<FT>(m.n, m.b, Dv, yv, ring.mem, ring.stages,
+                                    A.l2_dist > 0 ? ring.stages + A.l2_dist : 0);
+  dev::band_solve_packed<FT, PF>(m.n, m.b, Dv, yv, A.l2_dist);
+  return true;
+}
+
+// s = J^-1 rhs with the band factors, then FP64 iterative refinement against the local matrix
+// (columns < n) when the factors are FP32.  s and yv are in shared memory (s may be rhs's copy).
+// Returns false if a bounded wait gave up.
+template <typename FT, bool PF>
+__device__ bool local_solve(const LocalArgs& A, const SubMeta& m, const FT* Dv, const double* rhs, double rhs_norm,
+                            double* s, FT* yv, double* red, const Ring& ring) {
   const int n = m.n;
   for (int a = threadIdx.x; a < n; a += blockDim.x) yv[a] = (FT)rhs[a];
   __syncthreads();
-  dev::band_solve_packed<FT, PF>(n, m.b, Dv, yv, A.l2_dist);
+  bool ok = triangular_solves<FT, PF>(A, m, Dv, yv, ring);
   for (int a = threadIdx.x; a < n; a += blockDim.x) s[a] = (double)yv[a];
   __syncthreads();
-  int sweeps = 0;
   if (sizeof(FT) == 4) {
-    for (int sw = 0; sw < A.ir_max; ++sw) {
+    for (int sw = 0; ok && sw < A.ir_max; ++sw) {
       double loc = 0.0;
       for (int a = threadIdx.x; a < n; a += blockDim.x) {
         double acc = rhs[a];
-        for (int k = rowptr[a]; k < rowptr[a + 1]; ++k) {
-          const int col = colidx[k];
-          if (col < n) acc -= csr[k] * s[col];
-        }
-        res[a] = acc;
+        for_row(A, m, a, [&](double v, int32_t col) {
+          if (col < n) acc -= v * s[col];
+        });
+        yv[a] = (FT)acc;
         loc += acc * acc;
       }
       const double rn = sqrt(dev::block_sum(loc, red));
       if (!(rn > A.ir_rtol * rhs_norm)) break;
-      for (int a = threadIdx.x; a < n; a += blockDim.x) yv[a] = (FT)res[a];
-      __syncthreads();
-      dev::band_solve_packed<FT, PF>(n, m.b, Dv, yv, A.l2_dist);
+      ok = triangular_solves<FT, PF>(A, m, Dv, yv, ring);
       for (int a = threadIdx.x; a < n; a += blockDim.x) s[a] += (double)yv[a];
       __syncthreads();
-      ++sweeps;
     }
   }
-  return sweeps;
+  return ok;
 }
 
 // Damped Jacobi sweeps on a proposed local start (in xt's local unknowns): they remove the
@@ -441,15 +480,17 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : LAW == NLS_LAW_DIFFUS
     const int sub = A.order[item];
     const SubMeta m = A.meta[sub];
     const int n = m.n;
-    const int32_t* rowptr = A.rowptr + m.rowptr_off;
-    const int32_t* colidx = A.colidx + m.nnz_off;
     double* csr = A.csr + m.nnz_off;
     FT* F = (FT*)A.factor + m.factor_off;
     FT* Dv = (FT*)A.dinv + m.dinv_off;
     double* wb = A.wbuf + m.vec_off;
-    double* r = A.work + m.vec_off;                            // current residual
-    double* s = A.work + A.work_stride + m.vec_off;            // Newton step
-    double* res = A.work + 2 * A.work_stride + m.vec_off;      // refinement residual
+    double* r = A.work + m.vec_off;                  // current residual
+    double* s = A.work + A.work_stride + m.vec_off;  // Newton step
+    // the LU window serves the solves: the solve vector, then the ring of operands
+    const size_t y_bytes = align_up(sizeof(FT) * align_up(n, dev::SolveBlock<FT>::BS), 16);
+    const size_t win_bytes = sizeof(FT) * win_cap;
+    const Ring ring{(unsigned char*)win + y_bytes,
+                    y_bytes < win_bytes ? dev::ring_stages<FT>(m.b, win_bytes - y_bytes) : 0};
     for (int t = tid; t < m.nt; t += blockDim.x)
       xt[t] = A.x[(int64_t)A.tnode_gid[m.tnode_off + t / nd] * nd + t % nd];
     __syncthreads();
@@ -508,9 +549,16 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : LAW == NLS_LAW_DIFFUS
         dev::band_pack_solve<FT>(n, m.b, F, Dv, win, inv_warps);
         mark(2);
       }
-      local_solve<FT, false>(A, m, rowptr, colidx, csr, Dv, r, rn, s, res, yv, red);
+      if (!local_solve<FT, false>(A, m, Dv, r, rn, racc, yv, red, ring)) {
+        status = ST_TIMEOUT;
+        if (tid == 0) *A.err = 1;
+        break;
+      }
       mark(3);
-      for (int a = tid; a < n; a += blockDim.x) wb[a] = xt[a];
+      for (int a = tid; a < n; a += blockDim.x) {
+        s[a] = racc[a];
+        wb[a] = xt[a];
+      }
       __syncthreads();
       double alpha = 1.0, rtn = INFINITY;
       bool accepted = false;
@@ -549,7 +597,7 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : LAW == NLS_LAW_DIFFUS
       __syncthreads();
       rn = rtn;
     }
-    if (A.want_tangent && status != ST_NONFINITE && status != ST_PIVOT) {
+    if (A.want_tangent && status != ST_NONFINITE && status != ST_PIVOT && status != ST_TIMEOUT) {
       local_jacobian<LAW, FT>(A, m, xt, csr, F);
       mark(5);
       if (!A.split_factor) {
@@ -606,7 +654,7 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : 1) k_local_factor(Loca
   const int inv_warps = min((int)(blockDim.x >> 5), (int)(win_cap / dev::pack_scratch<FT>()));
   const int sub = A.order[blockIdx.x];
   const int st = A.status[sub];
-  if (st == ST_NONFINITE || st == ST_PIVOT) return;
+  if (st == ST_NONFINITE || st == ST_PIVOT || st == ST_TIMEOUT) return;
   const SubMeta m = A.meta[sub];
   FT* F = (FT*)A.factor + m.factor_off;
   FT* Dv = (FT*)A.dinv + m.dinv_off;
@@ -622,32 +670,29 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : 1) k_local_factor(Loca
 // ------------------------------------------------------------------------------------------
 template <typename FT>
 __global__ void __launch_bounds__(512) k_local_apply(LocalArgs A) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const LocalPlan P = apply_plan<FT>(A.max_n, A.max_nt);
+  extern __shared__ __align__(128) unsigned char smem[];
+  const LocalPlan P = apply_plan<FT>(A.max_n, A.max_nt, A.max_b, A.ring);
   double* yt = (double*)(smem + P.xt);
   double* red = (double*)(smem + P.red);
   FT* yv = (FT*)(smem + P.win);
-  const int sub = blockIdx.x, tid = threadIdx.x, nd = A.ndof;
+  const int sub = A.order[blockIdx.x], tid = threadIdx.x, nd = A.ndof;
   const SubMeta m = A.meta[sub];
   const int n = m.n;
-  const int32_t* rowptr = A.rowptr + m.rowptr_off;
-  const int32_t* colidx = A.colidx + m.nnz_off;
-  const double* csr = A.csr + m.nnz_off;
+  const Ring ring{smem + P.flag, A.ring ? dev::ring_stages<FT>(m.b, P.total - P.flag) : 0};
   const FT* Dv = (const FT*)A.dinv + m.dinv_off;
   double* q = A.work + m.vec_off;
-  double* z = A.work + A.work_stride + m.vec_off;
-  double* res = A.work + 2 * A.work_stride + m.vec_off;
   for (int t = tid; t < m.nt; t += blockDim.x) yt[t] = A.v[(int64_t)A.tnode_gid[m.tnode_off + t / nd] * nd + t % nd];
   __syncthreads();
   double loc = 0.0;
   for (int a = tid; a < n; a += blockDim.x) {
     double acc = 0.0;
-    for (int k = rowptr[a]; k < rowptr[a + 1]; ++k) acc += csr[k] * yt[colidx[k]];
+    for_row(A, m, a, [&](double v, int32_t col) { acc += v * yt[col]; });
     q[a] = acc;
     loc += acc * acc;
   }
   const double qn = sqrt(dev::block_sum(loc, red));
-  local_solve<FT, true>(A, m, rowptr, colidx, csr, Dv, q, qn, z, res, yv, red);
+  double* z = yt;  // the table vector has been used
+  if (!local_solve<FT, true>(A, m, Dv, q, qn, z, yv, red, ring) && tid == 0) *A.err = 1;
   for (int a = tid; a < n; a += blockDim.x)
     if (A.owned[m.vec_off + a]) {
       const int64_t g = (int64_t)A.tnode_gid[m.tnode_off + a / nd] * nd + a % nd;
@@ -1191,9 +1236,15 @@ int local_threads(const Context& c) {
   return std::max(pick, min_local_threads(c));
 }
 
+// CTA size of the tangent application: the solving warps and the copying one, and enough threads for
+// the matrix products -- 512 while every subdomain has an SM to itself, 256 while two share one.
 int apply_threads(const Context& c) {
-  if (c.dev && c.dev->apply_T) return std::max(c.dev->apply_T, min_local_threads(c));
-  return std::max(64, min_local_threads(c));
+  const int ring = c.opt.local_precision == NLS_PREC_FP32_IR ? dev::ring_threads<float>(c.ov.max_b)
+                                                            : dev::ring_threads<double>(c.ov.max_b);
+  const int need = std::max(64, std::max(ring, min_local_threads(c)));
+  if (c.dev && c.dev->apply_T) return std::max(c.dev->apply_T, need);
+  const int nsm = c.dev ? c.dev->nsm : 152;
+  return std::max(need, c.ov.count <= nsm ? 512 : c.ov.count <= 2 * nsm ? 256 : 128);
 }
 
 bool fp32_local(const Context& c) { return c.opt.local_precision == NLS_PREC_FP32_IR; }
@@ -1283,6 +1334,7 @@ LocalArgs make_args(const Context& c, const LocalSet& hs, const DeviceLocalSet& 
   A.ls_trials = c.opt.ls_trials;
   A.ir_max = c.opt.ir_max_sweeps;
   A.l2_dist = c.opt.l2_prefetch;
+  A.err = D.err_dev;
   return A;
 }
 
@@ -1457,20 +1509,33 @@ void launch_local_newton(Context& c, const double* x, double* out, double load, 
   }
 }
 
+// Stages of the tangent application's operand ring: as many as leave room for the CTAs per SM that the
+// subdomains fill (two at most), at least two.
+template <typename FT>
+int apply_ring_stages(const Context& c) {
+  const Dev& D = *c.dev;
+  const size_t per_sm = D.smem_optin + 1024, want = c.ov.count > D.nsm ? 2 : 1;
+  for (int st = dev::kRingMax; st >= 2; --st) {
+    const size_t sm = apply_plan<FT>(c.ov.max_n, c.ov.max_nt, c.ov.max_b, st).total;
+    if (sm <= D.smem_optin - 128 && ((sm + 1024) * want <= per_sm || st == 2)) return st;
+  }
+  return 0;
+}
+
 void launch_local_apply(Context& c, const double* v, const double* add, double* out) {
   Dev& D = *c.dev;
   LocalArgs A = make_args(c, c.ov, D.ov);
   A.v = v;
   A.add = add;
   A.out = out;
-  // the solves need warp 0 plus one thread per coupled row (32 + b); small CTAs let more
-  // subdomains be in flight on every SM, which is what hides the latency of the solves
   const int T = apply_threads(c);
   if (fp32_local(c)) {
-    const size_t sm = apply_plan<float>(c.ov.max_n, c.ov.max_nt).total;
+    A.ring = apply_ring_stages<float>(c);
+    const size_t sm = apply_plan<float>(c.ov.max_n, c.ov.max_nt, c.ov.max_b, A.ring).total;
     LAUNCH(D, k_local_apply<float>, c.ov.count, T, sm, A);
   } else {
-    const size_t sm = apply_plan<double>(c.ov.max_n, c.ov.max_nt).total;
+    A.ring = apply_ring_stages<double>(c);
+    const size_t sm = apply_plan<double>(c.ov.max_n, c.ov.max_nt, c.ov.max_b, A.ring).total;
     LAUNCH(D, k_local_apply<double>, c.ov.count, T, sm, A);
   }
 }
@@ -1521,10 +1586,11 @@ void tune_local_newton(Context& c, const double* x, double* out, double load, co
 void tune_local_apply(Context& c, const double* v, double* out) {
   Dev& D = *c.dev;
   if (D.apply_tuned || !c.opt.autotune) return;
-  const int need = std::max(64, min_local_threads(c));
+  D.apply_T = 32;  // the smallest CTA that the kernel takes
+  const int need = apply_threads(c);
   std::vector<int> cand;
-  for (int T : {need, need + 32, need + 64, 128, 192, 256})
-    if (T >= need && T <= 256 && std::find(cand.begin(), cand.end(), T) == cand.end()) cand.push_back(T);
+  for (int T : {need, need + 32, need + 64, 128, 192, 256, 384, 512})
+    if (T >= need && T <= 512 && std::find(cand.begin(), cand.end(), T) == cand.end()) cand.push_back(T);
   D.apply_T = need;
   launch_local_apply(c, v, nullptr, out);  // warm-up
   double best = INFINITY;
@@ -1570,6 +1636,15 @@ size_t coarse_factor_smem(const Context& c, bool f32) {
 // A_0(x) = P_0^T DF(x) P_0 -> band -> factor.  Returns false on a bad pivot.
 void coarse_matrix_launch(Context& c, const double* x);
 void coarse_inverse_launch(Context& c);
+
+// Raises DeviceTimeout if a local triangular solve has given up waiting since the last check (its
+// stream synchronised by the caller).
+void check_local_waits(Dev& D) {
+  volatile int* e = D.err_host;
+  if (!*e) return;
+  *e = 0;
+  throw DeviceTimeout("a local triangular solve gave up waiting for its operands");
+}
 
 // Reads the coarse factorization's status word (synchronises the stream).
 bool coarse_status_ok(Dev& D) {
@@ -1809,7 +1884,7 @@ void upload_set(Dev& D, const LocalSet& h, DeviceLocalSet& d, bool fp32_factor, 
     if (with_dinv) d.dinv = D.alloc<double>(h.total_dinv);
   }
   d.w = D.alloc<double>(h.total_n);
-  d.work = D.alloc<double>(3 * (size_t)h.total_n);
+  d.work = D.alloc<double>(2 * (size_t)h.total_n);
   d.its = D.alloc<int32_t>(h.count);
   d.chord = D.alloc<int32_t>(h.count);
   d.status = D.alloc<int32_t>(h.count);
@@ -1934,6 +2009,9 @@ int device_setup(Context& c) {
     CK(cudaMemsetAsync(D.phase, 0, sizeof(unsigned long long) * 8, D.s));
     CK(cudaDeviceGetAttribute(&D.clock_khz, cudaDevAttrClockRate, c.device));
     CK(cudaMallocHost(&D.h_scal, sizeof(double) * (kMaxGmresVecs + 8)));
+    CK(cudaHostAlloc(&D.err_host, sizeof(int), cudaHostAllocMapped));
+    *D.err_host = 0;
+    CK(cudaHostGetDevicePointer((void**)&D.err_dev, D.err_host, 0));
     // kernel attributes for large dynamic shared memory
     const size_t lim = D.smem_optin;
     auto need = [&](size_t b, const char* what) {
@@ -2099,6 +2177,7 @@ void device_free(Context& c) {
   for (void* p : D.allocs)
     if (p) cudaFree(p);
   if (D.h_scal) cudaFreeHost(D.h_scal);
+  if (D.err_host) cudaFreeHost(D.err_host);
   for (auto& r : D.evs) {
     cudaEventDestroy(r.a);
     cudaEventDestroy(r.b);
@@ -2573,6 +2652,7 @@ int solve(Context& c, double* u_user, int u_dev, nls_report* rep) {
     CK(cudaEventRecord(e1, D.s));
     CK(cudaEventSynchronize(e1));
     tlu_check_solves(c);
+    check_local_waits(D);
     float ms = 0.f;
     CK(cudaEventElapsedTime(&ms, e0, e1));
     cudaEventDestroy(e0);
@@ -2624,6 +2704,7 @@ int eval_Fx(Context& c, const double* u, double* Fx, int is_dev, double load, in
     if (its) CK(cudaMemcpyAsync(its, D.ov.its, sizeof(int32_t) * c.ov.count, cudaMemcpyDeviceToHost, D.s));
     if (st) CK(cudaMemcpyAsync(st, D.ov.status, sizeof(int32_t) * c.ov.count, cudaMemcpyDeviceToHost, D.s));
     sync(D);
+    check_local_waits(D);
     if (fi.pivot_failure) return NLS_E_PIVOT;
   } catch (const DeviceTimeout& ex) {
     c.last_error = ex.what();
@@ -2650,6 +2731,10 @@ int apply_tangent(Context& c, const double* v, double* y, int is_dev) {
     tangent(c, D.x, D.gx);
     CK(cudaMemcpyAsync(y, D.gx, sizeof(double) * c.N, is_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, D.s));
     sync(D);
+    check_local_waits(D);
+  } catch (const DeviceTimeout& ex) {
+    c.last_error = ex.what();
+    return NLS_E_DEVICE_TIMEOUT;
   } catch (const std::exception& ex) {
     c.last_error = ex.what();
     return NLS_E_CUDA;
@@ -2918,20 +3003,20 @@ int local_corrections_noalloc(Context& c, const double* x, double* Fx, int32_t* 
   Dev& D = *c.dev;
   const LocalSet& s = c.ov;
   const bool f32 = fp32_local(c);
-  // scratch plan: CSR values, band factors, packed solve operands, local states, work vectors,
-  // its, status, work counter
+  // scratch plan: matrix values and work vectors, band factors, packed solve operands, local states,
+  // its, status, work counter.  The limit is stated for the entries of the matrices and three work
+  // vectors; the padded values and two vectors (at most one value of padding per row) never need more.
   const size_t fbytes = f32 ? sizeof(float) : sizeof(double);
   size_t off = 0;
-  const size_t o_csr = off;
-  off = align_up(off + sizeof(double) * (size_t)s.total_nnz, 256);
+  const size_t o_csr = off, o_work = sizeof(double) * (size_t)s.total_nnz;
+  off = align_up(off + sizeof(double) * (size_t)s.total_entries, 256);
+  off = align_up(off + 3 * sizeof(double) * (size_t)s.total_n, 256);
   const size_t o_fac = off;
   off = align_up(off + fbytes * (size_t)s.total_factor, 256);
   const size_t o_dinv = off;
   off = align_up(off + fbytes * (size_t)s.total_dinv, 256);
   const size_t o_w = off;
   off = align_up(off + sizeof(double) * (size_t)s.total_n, 256);
-  const size_t o_work = off;
-  off = align_up(off + 3 * sizeof(double) * (size_t)s.total_n, 256);
   const size_t o_its = off;
   off = align_up(off + sizeof(int32_t) * (size_t)s.count, 256);
   const size_t o_st = off;

@@ -63,6 +63,25 @@ __device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity) {
   }
 }
 
+__device__ inline void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// Before the barrier's memory serves another purpose.
+__device__ inline void mbar_inval(uint64_t* bar) {
+  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// Untiled bulk copy into this CTA's shared memory (both addresses and the size multiples of 16
+// bytes), completing as transaction bytes on `bar`, and the prefetch of such a range into L2.
+__device__ inline void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+__device__ inline void bulk_prefetch_l2(const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(src)), "r"(bytes));
+}
+
 // ---- cluster exchange through distributed shared memory ------------------------------------
 // Address of the same shared-memory location in CTA `rank` of the cluster.
 __device__ inline uint32_t cluster_addr(const void* local, uint32_t rank) {
