@@ -59,7 +59,11 @@ struct GuessNet {
   int bmax = 0;
   float *X = nullptr, *T = nullptr, *Z1 = nullptr, *A1 = nullptr, *Z2 = nullptr, *A2 = nullptr, *Y = nullptr;
   float *dA = nullptr, *dZ = nullptr, *lossbuf = nullptr;
-  int32_t* idx = nullptr;
+  // training: minibatch indices and partial losses of a chunk of steps, sums of squares of the targets
+  int chunk_batch = 0;
+  int32_t* idx_chunk = nullptr;
+  float* loss_chunk = nullptr;
+  double* sq = nullptr;
   std::vector<void*> allocs;
   template <typename T>
   T* alloc(size_t n) {
@@ -69,6 +73,7 @@ struct GuessNet {
     return (T*)q;
   }
   void ensure_batch(int B);
+  void ensure_chunk(int batch);
 };
 
 // per-context attachment: geometry maps and buffers
@@ -139,111 +144,7 @@ struct SplitMix {
 };
 
 // ------------------------------------------------------------------------------------------
-// GEMM: C[i, j] = beta C[i, j] + sum_k A(i, k) B(k, j), A(i, k) = A[i sai + k sak],
-// B(k, j) = B[k sbk + j sbj]; C row-major with ldc.
-// ------------------------------------------------------------------------------------------
-__device__ inline uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&v);
-}
-
-__global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K, const float* __restrict__ A, int64_t sai,
-                                                   int64_t sak, const float* __restrict__ B, int64_t sbk, int64_t sbj,
-                                                   float* __restrict__ C, int64_t ldc, float beta) {
-  // 64 x 64 tile, 4 warps in 2 x 2, each warp 32 x 32 = 2 x 4 tiles of 16 x 8
-  __shared__ __nv_bfloat16 As[64][16 + 8];
-  __shared__ __nv_bfloat16 Bs[64][16 + 8];  // [n][k]
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int wm = (wid >> 1) * 32, wn = (wid & 1) * 32;
-  const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
-  const int g = lane >> 2, t = lane & 3;
-  float acc[2][4][4];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int e = tid; e < 64 * 16; e += 128) {
-      const int r = e / 16, kk = e % 16;
-      const int i = i0 + r, k = k0 + kk;
-      As[r][kk] = __float2bfloat16_rn((i < M && k < K) ? A[i * sai + k * sak] : 0.f);
-      const int j = j0 + r;
-      Bs[r][kk] = __float2bfloat16_rn((j < N && k < K) ? B[k * sbk + j * sbj] : 0.f);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int mi = 0; mi < 2; ++mi) {
-      const int r = wm + mi * 16;
-      const uint32_t a0 = *reinterpret_cast<const uint32_t*>(&As[r + g][2 * t]);
-      const uint32_t a1 = *reinterpret_cast<const uint32_t*>(&As[r + g + 8][2 * t]);
-      const uint32_t a2 = *reinterpret_cast<const uint32_t*>(&As[r + g][2 * t + 8]);
-      const uint32_t a3 = *reinterpret_cast<const uint32_t*>(&As[r + g + 8][2 * t + 8]);
-#pragma unroll
-      for (int ni = 0; ni < 4; ++ni) {
-        const int cn = wn + ni * 8;
-        const uint32_t b0 = *reinterpret_cast<const uint32_t*>(&Bs[cn + g][2 * t]);
-        const uint32_t b1 = *reinterpret_cast<const uint32_t*>(&Bs[cn + g][2 * t + 8]);
-        asm volatile(
-            "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-            "{%0,%1,%2,%3};\n"
-            : "+f"(acc[mi][ni][0]), "+f"(acc[mi][ni][1]), "+f"(acc[mi][ni][2]), "+f"(acc[mi][ni][3])
-            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int mi = 0; mi < 2; ++mi)
-#pragma unroll
-    for (int ni = 0; ni < 4; ++ni)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int i = i0 + wm + mi * 16 + g + (c >= 2 ? 8 : 0);
-        const int j = j0 + wn + ni * 8 + 2 * t + (c & 1);
-        if (i < M && j < N) {
-          float* cp = C + i * ldc + j;
-          *cp = (beta != 0.f ? beta * *cp : 0.f) + acc[mi][ni][c];
-        }
-      }
-}
-
-__global__ void __launch_bounds__(256) k_gemm_f32(int M, int N, int K, const float* __restrict__ A, int64_t sai,
-                                                  int64_t sak, const float* __restrict__ B, int64_t sbk, int64_t sbj,
-                                                  float* __restrict__ C, int64_t ldc, float beta) {
-  __shared__ float As[16][17], Bs[16][17];
-  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-  const int i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;
-  float acc = 0.f;
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    As[ty][tx] = (blockIdx.y * 16 + ty < M && k0 + tx < K) ? A[(int64_t)(blockIdx.y * 16 + ty) * sai + (k0 + tx) * sak] : 0.f;
-    Bs[ty][tx] = (k0 + ty < K && blockIdx.x * 16 + tx < N) ? B[(int64_t)(k0 + ty) * sbk + (blockIdx.x * 16 + tx) * sbj] : 0.f;
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) acc += As[ty][kk] * Bs[kk][tx];
-    __syncthreads();
-  }
-  if (i < M && j < N) {
-    float* cp = C + (int64_t)i * ldc + j;
-    *cp = (beta != 0.f ? beta * *cp : 0.f) + acc;
-  }
-}
-
-void gemm(cudaStream_t s, bool bf16, int M, int N, int K, const float* A, int64_t sai, int64_t sak, const float* B,
-          int64_t sbk, int64_t sbj, float* C, int64_t ldc, float beta = 0.f) {
-  if (bf16) {
-    dim3 grid((N + 63) / 64, (M + 63) / 64);
-    k_gemm_bf16<<<grid, 128, 0, s>>>(M, N, K, A, sai, sak, B, sbk, sbj, C, ldc, beta);
-  } else {
-    dim3 grid((N + 15) / 16, (M + 15) / 16);
-    k_gemm_f32<<<grid, 256, 0, s>>>(M, N, K, A, sai, sak, B, sbk, sbj, C, ldc, beta);
-  }
-  CK(cudaGetLastError());
-}
-
-// ------------------------------------------------------------------------------------------
-// elementwise pieces
+// GEMM: C(i, j) = sum_k A(i, k) B(k, j), with what follows the product in its epilogue
 // ------------------------------------------------------------------------------------------
 __device__ inline float gelu_f(float z) {
   const float u = 0.7978845608028654f * (z + 0.044715f * z * z * z);
@@ -256,15 +157,199 @@ __device__ inline float gelu_grad_f(float z) {
   return 0.5f * (1.f + th) + 0.5f * z * (1.f - th * th) * du;
 }
 
-// Z += bias (per column); A = gelu(Z) when act != 0
-__global__ void k_bias_act(int B, int n, float* Z, const float* bias, float* A, int act) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)B * n; e += (int64_t)gridDim.x * blockDim.x) {
-    const float z = Z[e] + bias[e % n];
-    Z[e] = z;
-    if (act) A[e] = gelu_f(z);
-  }
+// What a GEMM does with its sums on the way out:
+//   kPlain     C = sum
+//   kBiasAct   z = sum + bias (per column) into C, gelu(z) into `act` (if given)
+//   kGeluBack  C = sum gelu'(z), z read from `z` (same shape)
+enum Epilogue { kPlain, kBiasAct, kGeluBack };
+struct GemmOut {
+  float* C;
+  int64_t ld;
+  Epilogue mode;
+  const float* bias;
+  float* act;
+  const float* z;
+};
+__device__ __forceinline__ void gemm_out(const GemmOut& o, int i, int j, float sum) {
+  const int64_t e = i * o.ld + j;
+  float v = 0.f + sum;
+  if (o.mode == kBiasAct) v += o.bias[j];
+  else if (o.mode == kGeluBack) v *= gelu_grad_f(o.z[e]);
+  o.C[e] = v;
+  if (o.mode == kBiasAct && o.act) o.act[e] = gelu_f(v);
 }
 
+// BF16 GEMM on the tensor cores.  The shapes are a few hundred wide (batch 64 .. 1024): bound by the
+// latency of the chunks of K, so a CTA takes a 32 x 32 tile (64 to 256 of them per product) in chunks
+// of 64 of K, loaded into registers one chunk ahead; AK, BK say which operand is contiguous along K
+// (the loads of a warp follow the contiguous index).  Each warp owns 16 x 16 of the tile and
+// accumulates K in steps of 16 in order, as the 64 x 64 kernel with chunks of 16 did (20 us per
+// product; the same bits).
+template <bool AK, bool BK>
+__global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K, const float* __restrict__ A, int64_t lda,
+                                                   const float* __restrict__ B, int64_t ldb, GemmOut out) {
+  constexpr int KC = 64, LD = KC + 8, Q = 32 * KC / 128;
+  __shared__ __nv_bfloat16 As[2][32][LD], Bs[2][32][LD];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int wm = (wid >> 1) * 16, wn = (wid & 1) * 16;
+  const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
+  const int g = lane >> 2, t = lane & 3;
+  float acc[2][4] = {};
+  float ra[Q], rb[Q];
+  auto at = [&](bool kfast, int q, int& r, int& k) {  // element q of this thread within a 32 x KC chunk
+    const int e = tid + 128 * q;
+    r = kfast ? e / KC : e % 32;
+    k = kfast ? e % KC : e / 32;
+  };
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      int r, k;
+      at(AK, q, r, k);
+      ra[q] = (i0 + r < M && k0 + k < K) ? A[AK ? (i0 + r) * lda + k0 + k : (k0 + k) * lda + i0 + r] : 0.f;
+      at(BK, q, r, k);
+      rb[q] = (j0 + r < N && k0 + k < K) ? B[BK ? (j0 + r) * ldb + k0 + k : (k0 + k) * ldb + j0 + r] : 0.f;
+    }
+  };
+  auto store = [&](int s) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      int r, k;
+      at(AK, q, r, k);
+      As[s][r][k] = __float2bfloat16_rn(ra[q]);
+      at(BK, q, r, k);
+      Bs[s][r][k] = __float2bfloat16_rn(rb[q]);
+    }
+  };
+  fetch(0);
+  store(0);
+  __syncthreads();
+  for (int k0 = 0, s = 0; k0 < K; k0 += KC, s ^= 1) {
+    const bool more = k0 + KC < K;
+    if (more) fetch(k0 + KC);
+    const int steps = min(KC, K - k0 + 15) / 16;
+    for (int kk = 0; kk < steps; ++kk) {
+      const uint32_t* ar0 = reinterpret_cast<const uint32_t*>(&As[s][wm + g][16 * kk + 2 * t]);
+      const uint32_t* ar1 = reinterpret_cast<const uint32_t*>(&As[s][wm + g + 8][16 * kk + 2 * t]);
+#pragma unroll
+      for (int ni = 0; ni < 2; ++ni) {
+        const uint32_t* br = reinterpret_cast<const uint32_t*>(&Bs[s][wn + 8 * ni + g][16 * kk + 2 * t]);
+        asm volatile(
+            "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+            "{%0,%1,%2,%3};\n"
+            : "+f"(acc[ni][0]), "+f"(acc[ni][1]), "+f"(acc[ni][2]), "+f"(acc[ni][3])
+            : "r"(ar0[0]), "r"(ar1[0]), "r"(ar0[4]), "r"(ar1[4]), "r"(br[0]), "r"(br[4]));
+      }
+    }
+    if (more) store(s ^ 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int ni = 0; ni < 2; ++ni)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = i0 + wm + g + (c >= 2 ? 8 : 0), j = j0 + wn + ni * 8 + 2 * t + (c & 1);
+      if (i < M && j < N) gemm_out(out, i, j, acc[ni][c]);
+    }
+}
+
+// FP32 GEMM (inference, the FP32 gradient check): a 16 R x 16 R tile per CTA, R x R sums per thread,
+// chunks of 16 of K loaded one ahead.  Every sum runs over K in order in one accumulator, as in a
+// 16 x 16 tile with one sum per thread (3.8 TFLOP/s over the three products of a batch of 1024).
+template <bool AK, bool BK, int R>
+__global__ void __launch_bounds__(256) k_gemm_f32(int M, int N, int K, const float* __restrict__ A, int64_t lda,
+                                                  const float* __restrict__ B, int64_t ldb, GemmOut out) {
+  constexpr int KC = 16, T = 16 * R, LD = T + 4;
+  __shared__ __align__(16) float As[2][KC][LD], Bs[2][KC][LD];
+  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
+  const int i0 = blockIdx.y * T, j0 = blockIdx.x * T;
+  float acc[R][R] = {}, ra[R], rb[R];
+  auto at = [&](bool kfast, int q, int& r, int& k) {
+    const int e = tid + 256 * q;
+    r = kfast ? e / KC : e % T;
+    k = kfast ? e % KC : e / T;
+  };
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      int r, k;
+      at(AK, q, r, k);
+      ra[q] = (i0 + r < M && k0 + k < K) ? A[AK ? (i0 + r) * lda + k0 + k : (k0 + k) * lda + i0 + r] : 0.f;
+      at(BK, q, r, k);
+      rb[q] = (j0 + r < N && k0 + k < K) ? B[BK ? (j0 + r) * ldb + k0 + k : (k0 + k) * ldb + j0 + r] : 0.f;
+    }
+  };
+  auto store = [&](int s) {
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      int r, k;
+      at(AK, q, r, k);
+      As[s][k][r] = ra[q];
+      at(BK, q, r, k);
+      Bs[s][k][r] = rb[q];
+    }
+  };
+  fetch(0);
+  store(0);
+  __syncthreads();
+  for (int k0 = 0, s = 0; k0 < K; k0 += KC, s ^= 1) {
+    const bool more = k0 + KC < K;
+    if (more) fetch(k0 + KC);
+#pragma unroll
+    for (int kk = 0; kk < KC; ++kk) {
+      float a[R], b[R];
+      if constexpr (R == 4) {
+        *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(&As[s][kk][ty * 4]);
+        *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(&Bs[s][kk][tx * 4]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < R; ++i) a[i] = As[s][kk][ty * R + i], b[i] = Bs[s][kk][tx * R + i];
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) acc[i][j] += a[i] * b[j];
+    }
+    if (more) store(s ^ 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int ii = i0 + ty * R + i, jj = j0 + tx * R + j;
+      if (ii < M && jj < N) gemm_out(out, ii, jj, acc[i][j]);
+    }
+}
+
+template <bool AK, bool BK>
+void gemm_t(cudaStream_t s, bool bf16, int M, int N, int K, const float* A, int64_t lda, const float* B, int64_t ldb,
+            const GemmOut& out) {
+  auto grid = [&](int t) { return dim3((N + t - 1) / t, (M + t - 1) / t); };
+  if (bf16) {
+    k_gemm_bf16<AK, BK><<<grid(32), 128, 0, s>>>(M, N, K, A, lda, B, ldb, out);
+  } else {
+    // 64 x 64 tiles once they give most SMs a CTA (16 x 16 sums per thread read half as much), else 32 x 32
+    const dim3 g = grid(64);
+    if (g.x * g.y >= 100) k_gemm_f32<AK, BK, 4><<<g, 256, 0, s>>>(M, N, K, A, lda, B, ldb, out);
+    else k_gemm_f32<AK, BK, 2><<<grid(32), 256, 0, s>>>(M, N, K, A, lda, B, ldb, out);
+  }
+  CK(cudaGetLastError());
+}
+
+// C(i, j) = sum_k A(i, k) B(k, j).  ak (bk): A (B) is stored with K contiguous, row i (column j) lda
+// (ldb) apart; otherwise with i (j) contiguous, the rows of K lda (ldb) apart.
+void gemm(cudaStream_t s, bool bf16, int M, int N, int K, const float* A, bool ak, int64_t lda, const float* B, bool bk,
+          int64_t ldb, const GemmOut& out) {
+  if (ak && bk) gemm_t<true, true>(s, bf16, M, N, K, A, lda, B, ldb, out);
+  else if (ak) gemm_t<true, false>(s, bf16, M, N, K, A, lda, B, ldb, out);
+  else if (bk) gemm_t<false, true>(s, bf16, M, N, K, A, lda, B, ldb, out);
+  else gemm_t<false, false>(s, bf16, M, N, K, A, lda, B, ldb, out);
+}
+
+// ------------------------------------------------------------------------------------------
+// elementwise pieces
+// ------------------------------------------------------------------------------------------
 // dY = (Y - T) / B; per-block partial losses (fixed order) into part
 __global__ void k_loss_grad(int64_t total, int B, const float* Y, const float* T, float* dY, float* part) {
   __shared__ float red[256];
@@ -283,17 +368,21 @@ __global__ void k_loss_grad(int64_t total, int B, const float* Y, const float* T
   if (threadIdx.x == 0) part[blockIdx.x] = red[0] / (2.f * (float)B);
 }
 
-__global__ void k_gelu_back(int64_t total, const float* Z, float* dAZ) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x)
-    dAZ[e] *= gelu_grad_f(Z[e]);
-}
-
-__global__ void k_colsum(int B, int n, const float* dZ, float* db) {
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    float acc = 0.f;
-    for (int i = 0; i < B; ++i) acc += dZ[(int64_t)i * n + j];
-    db[j] = acc;
+// Column sums over the batch, one thread per column, rows in order, 16 of them in flight.
+__global__ void __launch_bounds__(32) k_colsum(int B, int n, const float* __restrict__ dZ, float* db) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  float acc = 0.f;
+  int i = 0;
+  for (; i + 16 <= B; i += 16) {
+    float v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[q] = dZ[(int64_t)(i + q) * n + j];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) acc += v[q];
   }
+  for (; i < B; ++i) acc += dZ[(int64_t)i * n + j];
+  db[j] = acc;
 }
 
 __global__ void k_adam(int64_t n, float* p, const float* g, float* m, float* v, float lr, float b1, float b2, float eps,
@@ -359,17 +448,20 @@ __global__ void k_feature_stats(int64_t n, int nf, const float* dX, float* mean,
   }
 }
 
-__global__ void k_target_rms(int64_t total, const float* dT, double* out) {
+// Sums of squares of the targets, one per CTA (added on the host in CTA order).
+constexpr int kRmsBlocks = 256;
+__global__ void k_target_squares(int64_t total, const float* dT, double* out) {
   __shared__ double red[256];
   double s = 0.0;
-  for (int64_t e = threadIdx.x; e < total; e += blockDim.x) s += (double)dT[e] * dT[e];
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x)
+    s += (double)dT[e] * dT[e];
   red[threadIdx.x] = s;
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {
     if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) *out = sqrt(red[0] / (double)(total > 0 ? total : 1));
+  if (threadIdx.x == 0) out[blockIdx.x] = red[0];
 }
 
 // ------------------------------------------------------------------------------------------
@@ -511,57 +603,57 @@ void GuessNet::ensure_batch(int B) {
   dA = alloc<float>((size_t)B * std::max(hm, no));
   dZ = alloc<float>((size_t)B * std::max(hm, no));
   lossbuf = alloc<float>(1024);
-  idx = alloc<int32_t>(B);
 }
+
+constexpr int kTrainChunk = 256;  // training steps issued between two reads of their losses
 
 namespace {
 
 // forward pass of B rows of normalised inputs in net.X (or `X` if given) into net.Y
 void net_forward(GuessNet& N, cudaStream_t s, int B, const float* X, bool bf16) {
-  const float* W1 = N.p + N.off[0];
-  const float* b1 = N.p + N.off[1];
-  const float* W2 = N.p + N.off[2];
-  const float* b2 = N.p + N.off[3];
-  const float* W3 = N.p + N.off[4];
-  const float* b3 = N.p + N.off[5];
-  const int grid = 1216;
-  gemm(s, bf16, B, N.h1, N.nf, X, N.nf, 1, W1, 1, N.nf, N.Z1, N.h1);
-  k_bias_act<<<grid, 256, 0, s>>>(B, N.h1, N.Z1, b1, N.A1, 1);
-  gemm(s, bf16, B, N.h2, N.h1, N.A1, N.h1, 1, W2, 1, N.h1, N.Z2, N.h2);
-  k_bias_act<<<grid, 256, 0, s>>>(B, N.h2, N.Z2, b2, N.A2, 1);
-  gemm(s, bf16, B, N.no, N.h2, N.A2, N.h2, 1, W3, 1, N.h2, N.Y, N.no);
-  k_bias_act<<<grid, 256, 0, s>>>(B, N.no, N.Y, b3, nullptr, 0);
+  auto layer = [&](const float* in, int k, int l, int n, float* Z, float* act) {
+    gemm(s, bf16, B, n, k, in, true, k, N.p + N.off[2 * l], true, k, {Z, n, kBiasAct, N.p + N.off[2 * l + 1], act, nullptr});
+  };
+  layer(X, N.nf, 0, N.h1, N.Z1, N.A1);
+  layer(N.A1, N.h1, 1, N.h2, N.Z2, N.A2);
+  layer(N.A2, N.h2, 2, N.no, N.Y, nullptr);
+}
+
+constexpr int kLossParts = 256;
+
+// gradient (into N.g) and partial losses (into `parts`, kLossParts of them) of the batch in N.X / N.T
+void net_gradient(GuessNet& N, cudaStream_t s, int B, bool bf16, float* parts) {
+  net_forward(N, s, B, N.X, bf16);
+  k_loss_grad<<<kLossParts, 256, 0, s>>>((int64_t)B * N.no, B, N.Y, N.T, N.dZ, parts);
+  // layer l from its dZ: dW = dZ^T (inputs), db = column sums, and dZ of the layer below
+  auto layer = [&](int l, const float* dZ, int n, const float* in, int k, float* below, const float* Zbelow) {
+    gemm(s, bf16, n, k, B, dZ, false, n, in, false, k, {N.g + N.off[2 * l], k, kPlain, nullptr, nullptr, nullptr});
+    k_colsum<<<(n + 31) / 32, 32, 0, s>>>(B, n, dZ, N.g + N.off[2 * l + 1]);
+    if (below)
+      gemm(s, bf16, B, k, n, dZ, true, n, N.p + N.off[2 * l], false, k, {below, k, kGeluBack, nullptr, nullptr, Zbelow});
+  };
+  layer(2, N.dZ, N.no, N.A2, N.h2, N.dA, N.Z2);
+  layer(1, N.dA, N.h2, N.A1, N.h1, N.dZ, N.Z1);
+  layer(0, N.dZ, N.h1, N.X, N.nf, nullptr, nullptr);
   CK(cudaGetLastError());
 }
 
-// loss and gradient (into N.g) of the batch in N.X / N.T
-float net_gradient(GuessNet& N, cudaStream_t s, int B, bool bf16) {
-  net_forward(N, s, B, N.X, bf16);
-  const float* W2 = N.p + N.off[2];
-  const float* W3 = N.p + N.off[4];
-  const int nb = 256;
-  k_loss_grad<<<nb, 256, 0, s>>>((int64_t)B * N.no, B, N.Y, N.T, N.dZ, N.lossbuf);
-  // layer 3: dW3 = dY^T A2, db3 = colsum dY, dA2 = dY W3
-  gemm(s, bf16, N.no, N.h2, B, N.dZ, 1, N.no, N.A2, N.h2, 1, N.g + N.off[4], N.h2);
-  k_colsum<<<(N.no + 255) / 256, 256, 0, s>>>(B, N.no, N.dZ, N.g + N.off[5]);
-  gemm(s, bf16, B, N.h2, N.no, N.dZ, N.no, 1, W3, N.h2, 1, N.dA, N.h2);
-  k_gelu_back<<<1216, 256, 0, s>>>((int64_t)B * N.h2, N.Z2, N.dA);
-  // layer 2 (dZ2 in dA)
-  gemm(s, bf16, N.h2, N.h1, B, N.dA, 1, N.h2, N.A1, N.h1, 1, N.g + N.off[2], N.h1);
-  k_colsum<<<(N.h2 + 255) / 256, 256, 0, s>>>(B, N.h2, N.dA, N.g + N.off[3]);
-  gemm(s, bf16, B, N.h1, N.h2, N.dA, N.h2, 1, W2, N.h1, 1, N.dZ, N.h1);
-  k_gelu_back<<<1216, 256, 0, s>>>((int64_t)B * N.h1, N.Z1, N.dZ);
-  // layer 1 (dZ1 in dZ)
-  gemm(s, bf16, N.h1, N.nf, B, N.dZ, 1, N.h1, N.X, N.nf, 1, N.g + N.off[0], N.nf);
-  k_colsum<<<(N.h1 + 255) / 256, 256, 0, s>>>(B, N.h1, N.dZ, N.g + N.off[1]);
-  CK(cudaGetLastError());
-  std::vector<float> part(nb);
-  CK(cudaMemcpyAsync(part.data(), N.lossbuf, nb * sizeof(float), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+float loss_of(const float* parts) {
   double L = 0.0;
-  for (float v : part) L += v;
+  for (int q = 0; q < kLossParts; ++q) L += parts[q];
   return (float)L;
 }
+
+}  // namespace
+
+void GuessNet::ensure_chunk(int batch) {
+  if (!loss_chunk) loss_chunk = alloc<float>((size_t)kTrainChunk * kLossParts);
+  if (batch <= chunk_batch) return;
+  chunk_batch = batch;
+  idx_chunk = alloc<int32_t>((size_t)kTrainChunk * batch);
+}
+
+namespace {
 
 // ------------------------------------------------------------------------------------------
 // host geometry of the attachment (structured P1 or Q1 meshes of the unit square)
@@ -789,7 +881,7 @@ GuessProposal guess_propose(Context& c, const double* x, double load) {
   LAUNCH(D, k_guess_features, G->nsub, 128, 0, a, G->nsub);
   LAUNCH(D, k_normalise, 1216, 256, 0, G->nsub, N.nf, G->raw, N.mean, N.scale, G->xin);
   net_forward(N, D.s, G->nsub, G->xin, false);
-  D.launches += 6;
+  D.launches += 3;
   LAUNCH(D, k_guess_decode, G->nsub, 128, 0, a, G->nsub, N.Y, N.tscale, G->guess);
   CK(cudaMemsetAsync(G->accepted, 0, sizeof(int32_t) * G->nsub, D.s));
   G->proposed_total += G->nsub;
@@ -1054,9 +1146,11 @@ int nls_guess_gradient(nls_guess_net* w, int32_t B, const float* X, const float*
     N.ensure_batch(B);
     CK(cudaMemcpy(N.X, X, (size_t)B * N.nf * sizeof(float), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(N.T, T, (size_t)B * N.no * sizeof(float), cudaMemcpyHostToDevice));
-    const float L = nls::net_gradient(N, 0, B, precision == 1);
+    nls::net_gradient(N, 0, B, precision == 1, N.lossbuf);
     CK(cudaMemcpy(grad, N.g, N.nparam * sizeof(float), cudaMemcpyDeviceToHost));
-    if (loss) *loss = L;
+    float parts[nls::kLossParts];
+    CK(cudaMemcpy(parts, N.lossbuf, sizeof(parts), cudaMemcpyDeviceToHost));
+    if (loss) *loss = nls::loss_of(parts);
   } catch (const std::exception&) {
     return NLS_E_CUDA;
   }
@@ -1087,26 +1181,39 @@ int nls_guess_train(nls_guess_net* w, int32_t steps, int32_t batch, double lr, u
     N.ensure_batch(batch);
     // normalisation from the harvested pairs (inputs per feature, targets by their rms)
     nls::k_feature_stats<<<N.nf, 256>>>(N.npairs, N.nf, N.dX, N.mean, N.scale);
-    double* rms = nullptr;
-    CK(cudaMalloc(&rms, sizeof(double)));
-    nls::k_target_rms<<<1, 256>>>(N.npairs * N.no, N.dT, rms);
-    double hr = 1.0;
-    CK(cudaMemcpy(&hr, rms, sizeof(double), cudaMemcpyDeviceToHost));
-    cudaFree(rms);
+    if (!N.sq) N.sq = N.alloc<double>(nls::kRmsBlocks);
+    nls::k_target_squares<<<nls::kRmsBlocks, 256>>>(N.npairs * N.no, N.dT, N.sq);
+    std::vector<double> sq(nls::kRmsBlocks);
+    CK(cudaMemcpy(sq.data(), N.sq, sizeof(double) * sq.size(), cudaMemcpyDeviceToHost));
+    double sum = 0.0;
+    for (double v : sq) sum += v;
+    const double hr = std::sqrt(sum / (double)std::max<int64_t>(N.npairs * N.no, 1));
     N.tscale = (float)(hr > 1e-30 ? hr : 1.0);
+    // The steps go out without waiting for one another: the minibatches of up to kTrainChunk steps are
+    // drawn and copied ahead, their partial losses stay on the device until the chunk is done.
     nls::SplitMix rng{seed};
-    std::vector<int32_t> idx(batch);
-    for (int st = 0; st < steps; ++st) {
-      for (int r = 0; r < batch; ++r) idx[r] = (int32_t)(rng.next() % (uint64_t)N.npairs);
-      CK(cudaMemcpy(N.idx, idx.data(), batch * sizeof(int32_t), cudaMemcpyHostToDevice));
-      nls::k_gather_batch<<<1216, 256>>>(batch, N.nf, N.no, N.idx, N.dX, N.dT, N.mean, N.scale, N.tscale, N.X, N.T);
-      const float L = nls::net_gradient(N, 0, batch, true);
-      N.adam_t += 1;
-      const float b1 = 0.9f, b2 = 0.999f;
-      nls::k_adam<<<1216, 256>>>(N.nparam, N.p, N.g, N.m, N.v, (float)lr, b1, b2, 1e-8f,
-                                 1.f - std::pow(b1, (float)N.adam_t), 1.f - std::pow(b2, (float)N.adam_t));
-      CK(cudaGetLastError());
-      if (loss_out) loss_out[st] = L;
+    N.ensure_chunk(batch);
+    std::vector<int32_t> idx;
+    std::vector<float> parts;
+    for (int s0 = 0; s0 < steps; s0 += nls::kTrainChunk) {
+      const int ns = std::min(nls::kTrainChunk, steps - s0);
+      idx.resize((size_t)ns * batch);
+      for (auto& r : idx) r = (int32_t)(rng.next() % (uint64_t)N.npairs);
+      CK(cudaMemcpy(N.idx_chunk, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+      for (int st = 0; st < ns; ++st) {
+        nls::k_gather_batch<<<1216, 256>>>(batch, N.nf, N.no, N.idx_chunk + (size_t)st * batch, N.dX, N.dT, N.mean, N.scale,
+                                           N.tscale, N.X, N.T);
+        nls::net_gradient(N, 0, batch, true, N.loss_chunk + (size_t)st * nls::kLossParts);
+        N.adam_t += 1;
+        const float b1 = 0.9f, b2 = 0.999f;
+        nls::k_adam<<<1216, 256>>>(N.nparam, N.p, N.g, N.m, N.v, (float)lr, b1, b2, 1e-8f,
+                                   1.f - std::pow(b1, (float)N.adam_t), 1.f - std::pow(b2, (float)N.adam_t));
+        CK(cudaGetLastError());
+      }
+      parts.resize((size_t)ns * nls::kLossParts);
+      CK(cudaMemcpy(parts.data(), N.loss_chunk, parts.size() * sizeof(float), cudaMemcpyDeviceToHost));
+      if (loss_out)
+        for (int st = 0; st < ns; ++st) loss_out[s0 + st] = nls::loss_of(&parts[(size_t)st * nls::kLossParts]);
     }
     CK(cudaDeviceSynchronize());
   } catch (const std::exception&) {
