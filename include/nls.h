@@ -115,10 +115,10 @@ typedef struct nls_options {
                                  fastest (nls_get_tuning).  The choice changes the order of
                                  floating-point reductions only.  0 (default): the library's
                                  fixed choice or threads_per_block. */
-  int32_t l2_prefetch;        /* the triangular solves with the packed factors (local Newton
-                                 steps, tangent applications, coarse solves) prefetch the
-                                 operands of the 32-row block this many blocks ahead into L2;
-                                 0 = off, at most 64 (default 4).  Changes no result. */
+  int32_t l2_prefetch;        /* triangular solves that keep their operands in registers (those whose
+                                 operand ring does not fit in shared memory) prefetch the operands of
+                                 the 32-row block this many blocks ahead into L2; 0 = off, at most 64
+                                 (default 4).  Changes no result. */
   int32_t outer_backtrack;    /* 1: the outer Newton step u <- u - alpha du takes the first of
                                  alpha = 1, 1/2, ... (at most min(ls_trials, 5)) with ||F(u')|| <
                                  outer_atol or ||F_x(u')|| <= (1 - armijo alpha) ||F_x(u)||, the last

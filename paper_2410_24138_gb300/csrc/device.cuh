@@ -20,6 +20,13 @@ namespace dev {
 
 constexpr int kWarp = 32;
 
+// The dynamic shared memory of the kernel.  The large routines below are real calls (their code would
+// otherwise be in every kernel twice, and their registers with it); they take their arrays as offsets
+// into it, because through a pointer argument the compiler could only use generic loads, which take
+// about twice as long as shared-memory ones.
+extern __shared__ __align__(128) unsigned char dyn_smem[];
+__device__ __forceinline__ uint32_t dyn_offset(const void* p) { return tc::smem_u32(p) - tc::smem_u32(dyn_smem); }
+
 // ------------------------------------------------------------------------------------------
 // reductions (deterministic for a fixed block size)
 // ------------------------------------------------------------------------------------------
@@ -458,10 +465,28 @@ __host__ __device__ constexpr int band_limit_stride(int b) {
   return w;
 }
 
+// 1 / p.  FP64: from the FP32 reciprocal (relative error e < 2^-23) by r (1 + e + e^2), three FP64
+// instructions at about 70 cycles each instead of a division; the next term of the series is below
+// 2^-69, so the result is within one ulp.
 template <typename FT>
 __device__ inline FT recip(FT p) {
-  if constexpr (sizeof(FT) == 4) return __frcp_rn(p);
-  else return (FT)1 / p;
+  if constexpr (sizeof(FT) == 4) {
+    return __frcp_rn(p);
+  } else {
+    const unsigned e = ((unsigned)__double2hiint(p) >> 20) & 0x7ff;
+    if (e - 923u >= 200u) return (FT)1 / p;  // outside [2^-100, 2^100): no FP32 value to start from
+    const double r = (double)__frcp_rn((float)p), err = fma(-p, r, 1.0);
+    return fma(r, fma(err, err, err), r);
+  }
+}
+// Zero, infinite or NaN, without floating-point instructions.
+__device__ inline bool bad_pivot(float p) {
+  const unsigned u = __float_as_uint(p) & 0x7fffffffu;
+  return u == 0 || u >= 0x7f800000u;
+}
+__device__ inline bool bad_pivot(double p) {
+  const unsigned h = (unsigned)__double2hiint(p) & 0x7fffffffu;
+  return (h | (unsigned)__double2loint(p)) == 0 || h >= 0x7ff00000u;
 }
 
 // f(integral_constant<int, I>) for I = I0 .. N - 1: a loop whose index is a constant in its body
@@ -483,7 +508,10 @@ struct alignas(16) LuVec {
 // band_lu_window<FT>(b, 0) entries, 16-byte aligned, win_cap of them usable.  blockDim.x: a
 // multiple of 32, at least 64.
 template <typename FT>
-__device__ __noinline__ int band_lu_inplace(int n, int b, FT* __restrict__ F, FT* win, size_t win_cap, int* flag) {
+__device__ __noinline__ int band_lu_at(int n, int b, FT* __restrict__ F, uint32_t win_off, size_t win_cap,
+                                        uint32_t flag_off) {
+  FT* const win = (FT*)(dyn_smem + win_off);
+  int* const flag = (int*)(dyn_smem + flag_off);
   constexpr int G = LuTile<FT>::G, NB = LuTile<FT>::NB, TE = LuTile<FT>::TE;
   constexpr int RH = 32 / NB;       // tile rows a warp covers with one entry per lane
   constexpr int C = NB * NB / 32;   // entries per lane of a tile spread over a warp
@@ -559,7 +587,7 @@ __device__ __noinline__ int band_lu_inplace(int n, int b, FT* __restrict__ F, FT
 #pragma unroll
       for (int j = j0; j < C; ++j) u[j] = __shfl_sync(0xffffffffu, a[j], k + NB * h);
       const FT rp = recip<FT>(p);
-      bad |= !(p != (FT)0) || !(p - p == (FT)0);  // zero, infinite or NaN
+      bad |= bad_pivot(p);
       const FT l = x * rp;
 #pragma unroll
       for (int j = j0; j < C; ++j) {
@@ -592,11 +620,12 @@ __device__ __noinline__ int band_lu_inplace(int n, int b, FT* __restrict__ F, FT
     FT* D = tile(sK, sK);
     const int s1 = wrap(sK + 1);
     // A: L tiles (I, K) row by row, U tiles (K, J) column by column
-    for (int idx = tid; idx < 2 * tb * NB; idx += T) {
-      const bool lower = idx < tb * NB;
-      const int q = lower ? idx : idx - tb * NB;
+    const int half = (tb * NB + 31) & ~31;  // a warp takes rows or columns, not both
+    for (int idx = tid; idx < 2 * half; idx += T) {
+      const bool lower = idx < half;
+      const int q = lower ? idx : idx - half;
       const int o = q / NB, x = q % NB;  // tile K + 1 + o, row or column x
-      if (K + 1 + o >= NP) continue;
+      if (o >= tb || K + 1 + o >= NP) continue;
       const int so = wrap(s1 + o);
       FT a[NB];
       if (lower) {
@@ -734,6 +763,10 @@ __device__ __noinline__ int band_lu_inplace(int n, int b, FT* __restrict__ F, FT
   }
   return *flag;
 }
+template <typename FT>
+__device__ __forceinline__ int band_lu_inplace(int n, int b, FT* F, FT* win, size_t win_cap, int* flag) {
+  return band_lu_at<FT>(n, b, F, dyn_offset(win), win_cap, dyn_offset(flag));
+}
 
 // ------------------------------------------------------------------------------------------
 // Triangular solves with the band factors, in place on y[0..n) (shared memory).
@@ -858,14 +891,19 @@ __device__ void band_solve(int n, int b, const FT* __restrict__ F, FT* y) {
 
 // ------------------------------------------------------------------------------------------
 // Packed solve operands.  After a factorization the operands of the two triangular solves are
-// copied, block by block (BS rows), into a layout in which every warp-wide load of the solve
-// reads BS consecutive values:
+// copied, block by block (BS rows), into rows of BS entries = 128 bytes, one per row that the block
+// solves or couples to:
 //
 //   block t (rows k0 = t BS .. k0 + bs - 1), PB = 2 BS^2 + 2 b BS entries:
-//     [0, BS^2)               inv(L_tt), column-major: entry (r, j) at j BS + r (identity padded)
-//     [BS^2, 2 BS^2)          inv(U_tt), column-major (U's diagonal is stored inverted)
-//     [2 BS^2, + b BS)        CL: entry (j, r) at j b + r = L[k0 + BS + r][k0 + j]
-//     [2 BS^2 + b BS, + b BS) CU: entry (j, r) at j b + r = U[k0 - 1 - r][k0 + j]
+//     [0, BS^2)               inv(L_tt): row r holds inv(L_tt)[r][j], j < BS (identity padded)
+//     [BS^2, 2 BS^2)          inv(U_tt) likewise (U's diagonal is stored inverted)
+//     [2 BS^2, + b BS)        CL: row r holds L[k0 + BS + r][k0 + j]
+//     [2 BS^2 + b BS, + b BS) CU: row r holds U[k0 - 1 - r][k0 + j]
+//
+// The thread that owns a row reads it as eight 16-byte groups; group g of row r is stored at position
+// g ^ (r mod 8), so that eight threads reading their rows from shared memory touch all banks.  (With
+// the rows along the threads instead, one 4-byte load per term, a solve step issued 64 loads on its
+// critical warp, and packing had to transpose everything.)
 //
 // The explicit diagonal-block inverses replace the BS-step dependent shuffle chain of a
 // diagonal block by one short dot product per row.  One warp per block; `tmp` (16-byte aligned)
@@ -875,8 +913,13 @@ template <typename FT>
 __host__ __device__ constexpr int64_t packed_block_entries(int b) {
   return 2 * (int64_t)SolveBlock<FT>::BS * SolveBlock<FT>::BS + 2 * (int64_t)b * SolveBlock<FT>::BS;
 }
+// Position of entry j of row r within the row.
+template <typename FT>
+__host__ __device__ constexpr int packed_at(int r, int j) {
+  return (((j / LuTile<FT>::G) ^ (r & 7)) * LuTile<FT>::G) + j % LuTile<FT>::G;
+}
 
-// Rows of the scratch: padded to whole 16-byte groups, with the column reads of a warp spread over
+// Rows of the scratch: padded to whole 16-byte groups, with the column writes of a warp spread over
 // the banks.
 template <typename FT>
 __host__ __device__ constexpr int pack_stride() {
@@ -900,34 +943,20 @@ __device__ void band_pack_solve_range(int n, int b, const FT* __restrict__ F, FT
   if (wid < nwarps) {
     FT* M = tmp + wid * BS * LD;
     const int hi = lane / BS, lo = lane % BS;  // a warp covers H rows of BS entries at once
-    // the inverses go out through the scratch: the column a lane holds becomes a row of the operands
-    auto store = [&](const FT (&x)[BS], FT* dst) {
-      __syncwarp();
-      if (lane < BS) {
-#pragma unroll
-        for (int i = 0; i < BS; ++i) M[lane * LD + i] = x[i];
-      }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < E; ++q) dst[q * 32 + lane] = M[(q * H + hi) * LD + lo];
-      __syncwarp();
-    };
     for (int t = first + wid; t < nblk; t += stride) {
       const int k0 = t * BS, bs = min(BS, n - k0);
       FT* out = P + (int64_t)t * PB;
-      FT vl[E], vu[E];  // L_tt and U_tt (its diagonal stored inverted), entry (i, j) = (q H + hi, lo)
+      FT vu[E];  // U_tt (its diagonal stored inverted), entry (i, j) = (q H + hi, lo)
 #pragma unroll
       for (int q = 0; q < E; ++q) {
         const int i = q * H + hi, j = lo;
         const bool in = i < bs && j < bs && i - j <= b && j - i <= b;
         const FT v = in ? F[(int64_t)(k0 + i) * W + (j - i + b)] : (i == j) ? (FT)1 : (FT)0;
-        vl[q] = (j < i) ? v : (FT)0;
+        M[lo * LD + i] = (j < i) ? v : (FT)0;  // L_tt, transposed
         vu[q] = (j < i) ? (FT)0 : v;
       }
-      FT x[BS];
-#pragma unroll
-      for (int q = 0; q < E; ++q) M[lo * LD + q * H + hi] = vl[q];  // transposed
       __syncwarp();
+      FT x[BS];
       // column `lane` of inv(L) (lanes past BS repeat one): forward substitution with e_lane, each
       // unknown taken out of all later rows at once
 #pragma unroll
@@ -941,7 +970,11 @@ __device__ void band_pack_solve_range(int n, int b, const FT* __restrict__ F, FT
           for (int i = 0; i < G; ++i)
             if (g + i > j) x[g + i] -= v.v[i] * x[j];
         }
-      store(x, out);
+      __syncwarp();
+      if (lane < BS) {
+#pragma unroll
+        for (int i = 0; i < BS; ++i) out[i * BS + packed_at<FT>(i, lane)] = x[i];
+      }
 #pragma unroll
       for (int q = 0; q < E; ++q) M[(q * H + hi) * LD + lo] = vu[q];
       __syncwarp();
@@ -960,31 +993,31 @@ __device__ void band_pack_solve_range(int n, int b, const FT* __restrict__ F, FT
         }
         x[i] = acc * diag;
       }
-      store(x, out + BS * BS);
-      // couplings, BS coupled rows at a time through the scratch: the band is read along its rows and
-      // the operands are written along the coupled rows, both coalesced
+      __syncwarp();
+      if (lane < BS) {
+#pragma unroll
+        for (int i = 0; i < BS; ++i) out[BS * BS + i * BS + packed_at<FT>(i, lane)] = x[i];
+      }
+      // couplings: rows of the band become rows of the operands
       FT* cl = out + 2 * BS * BS;
       FT* cu = cl + (int64_t)b * BS;
-      for (int r0 = 0; r0 < b; r0 += BS) {
+      const bool jn = lo < bs;
+      for (int r0 = 0; r0 < b; r0 += 8 * H) {
+        FT vl[8], vc[8];
 #pragma unroll
-        for (int q = 0; q < E; ++q) {
+        for (int q = 0; q < 8; ++q) {
           const int r = r0 + q * H + hi, j = lo;
           const int il = k0 + BS + r, dl = j - BS - r + b, iu = k0 - 1 - r, du = j + 1 + r + b;
-          const bool in = r < b && j < bs;
-          vl[q] = (in && il < n && dl >= 0) ? F[(int64_t)il * W + dl] : (FT)0;
-          vu[q] = (in && iu >= 0 && du <= 2 * b) ? F[(int64_t)iu * W + du] : (FT)0;
+          vl[q] = (jn && r < b && il < n && dl >= 0) ? F[(int64_t)il * W + dl] : (FT)0;
+          vc[q] = (jn && r < b && iu >= 0 && du <= 2 * b) ? F[(int64_t)iu * W + du] : (FT)0;
         }
 #pragma unroll
-        for (int up = 0; up < 2; ++up) {
-#pragma unroll
-          for (int q = 0; q < E; ++q) M[(q * H + hi) * LD + lo] = up ? vu[q] : vl[q];
-          __syncwarp();
-          FT* dst = up ? cu : cl;
-          if (r0 + lo < b) {
-#pragma unroll
-            for (int q = 0; q < E; ++q) dst[(int64_t)(q * H + hi) * b + r0 + lo] = M[lo * LD + q * H + hi];
+        for (int q = 0; q < 8; ++q) {
+          const int r = r0 + q * H + hi;
+          if (r < b) {
+            cl[(int64_t)r * BS + packed_at<FT>(r, lo)] = vl[q];
+            cu[(int64_t)r * BS + packed_at<FT>(r, lo)] = vc[q];
           }
-          __syncwarp();
         }
       }
     }
@@ -993,8 +1026,13 @@ __device__ void band_pack_solve_range(int n, int b, const FT* __restrict__ F, FT
 }
 
 template <typename FT>
-__device__ __noinline__ void band_pack_solve(int n, int b, const FT* __restrict__ F, FT* __restrict__ P, FT* tmp, int nwarps) {
-  band_pack_solve_range<FT>(n, b, F, P, tmp, nwarps, 0, nwarps);
+__device__ __noinline__ void band_pack_at(int n, int b, const FT* __restrict__ F, FT* __restrict__ P, uint32_t tmp_off,
+                                          int nwarps) {
+  band_pack_solve_range<FT>(n, b, F, P, (FT*)(dyn_smem + tmp_off), nwarps, 0, nwarps);
+}
+template <typename FT>
+__device__ __forceinline__ void band_pack_solve(int n, int b, const FT* F, FT* P, FT* tmp, int nwarps) {
+  band_pack_at<FT>(n, b, F, P, dyn_offset(tmp), nwarps);
 }
 
 // Triangular solves with the packed operands, in place on y[0..n) (shared memory): warp 0
@@ -1006,10 +1044,10 @@ __device__ __noinline__ void band_pack_solve(int n, int b, const FT* __restrict_
 // for kernels that keep enough CTAs resident).  With l2d > 0 the operands of the block l2d steps
 // ahead are prefetched into L2 (one 128-byte line per thread: the diagonal-block inverse by the
 // first BS^2 sizeof(FT) / 128 threads, the b coupling lines by the coupling threads), so that
-// the register loads of the current and next block wait for L2 rather than HBM.  The forward
-// sweep starts at block t0: y must vanish in the rows before it.  Needs blockDim.x >= 32 + b.
+// the register loads of the current and next block wait for L2 rather than HBM.  Needs blockDim.x >=
+// 32 + b.
 template <typename FT, bool PF>
-__device__ void band_solve_packed(int n, int b, const FT* __restrict__ P, FT* y, int l2d = 0, int t0 = 0) {
+__device__ void band_solve_packed(int n, int b, const FT* __restrict__ P, FT* y, int l2d = 0) {
   constexpr int BS = SolveBlock<FT>::BS;
   constexpr int NB = PF ? 2 : 1;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -1022,12 +1060,15 @@ __device__ void band_solve_packed(int n, int b, const FT* __restrict__ P, FT* y,
   FT buf[NB][BS];
   auto load = [&](int t, int which, int64_t od, int64_t oc) {
     const FT* Pt = P + (int64_t)t * PB;
-    if (diag) {
+    if (diag || offd) {
+      const int row = diag ? lane : r;
+      const FT* R = Pt + (diag ? od : oc) + (int64_t)row * BS;
 #pragma unroll
-      for (int j = 0; j < BS; ++j) buf[which][j] = Pt[od + j * BS + lane];
-    } else if (offd) {
+      for (int j = 0; j < BS; j += LuTile<FT>::G) {
+        const LuVec<FT> v = *(const LuVec<FT>*)(R + packed_at<FT>(row, j));
 #pragma unroll
-      for (int j = 0; j < BS; ++j) buf[which][j] = Pt[oc + j * b + r];
+        for (int i = 0; i < LuTile<FT>::G; ++i) buf[which][j + i] = v.v[i];
+      }
     }
   };
   constexpr int LINE = 128 / (int)sizeof(FT);            // entries per 128-byte line
@@ -1040,9 +1081,9 @@ __device__ void band_solve_packed(int n, int b, const FT* __restrict__ P, FT* y,
     if (a) asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(a)));
   };
   // forward: diag lanes read inv(L_tt), coupling threads read CL
-  if (PF && t0 < nblk) load(t0, 0, oL, oCL);
-  for (int q = t0 + 1; q < t0 + l2d && q < nblk; ++q) l2pf(q, oL, oCL);
-  for (int t = t0; t < nblk; ++t) {
+  if (PF && nblk > 0) load(0, 0, oL, oCL);
+  for (int q = 1; q < l2d && q < nblk; ++q) l2pf(q, oL, oCL);
+  for (int t = 0; t < nblk; ++t) {
     const int k0 = t * BS, kb = min(BS, n - k0);
     if (l2d > 0 && t + l2d < nblk) l2pf(t + l2d, oL, oCL);
     if (PF) {
@@ -1131,24 +1172,31 @@ __device__ void band_solve_packed(int n, int b, const FT* __restrict__ P, FT* y,
 // The same triangular solves with the operands streamed through shared memory.
 //
 // What bounds them: 2 ceil(n / BS) dependent block steps, each reading BS (BS + b) operand entries
-// once (15 KB in FP32 at b = 85).  With the operands in registers one step ahead, a step waited for
-// L2 (about 1400 cycles a step with one CTA per SM); here one thread of an extra warp keeps `stages`
-// blocks in flight by bulk copies (cp.async.bulk on mbarriers), and the chain of a step is warp 0's
-// alone: it applies the diagonal inverse, takes the coupling to the next block's rows itself and goes
-// on, while the other warps add the coupling to the rows beyond; one named barrier of the solving
-// warps per step keeps the order of the additions to every row, so the results are bit for bit those
-// of band_solve_packed.
+// once (15 KB in FP32 at b = 85).  One thread of an extra warp keeps `stages` blocks in flight by bulk
+// copies (cp.async.bulk on mbarriers), and the chain of a step is warp 0's alone: it applies the
+// diagonal inverse, takes the coupling to the next block's rows itself and goes on, while the other
+// warps add the coupling to the rows beyond; one named barrier of the solving warps per step keeps
+// the order of the additions to every row, so the results are bit for bit those of
+// band_solve_packed.  Every warp reads its operands of the next step into registers as soon as the
+// current ones are used, so that only the exchange of the solved block is on the chain.  FP64: two
+// lanes per row, the even and the odd terms, because a warp's FP64 instruction takes 64 cycles.
 //
 // Ring in shared memory (16-byte aligned): 128 bytes of mbarriers and a flag, then the stages, each
 // the diagonal inverse and the coupling of one block and direction.  y: nblk BS entries, 16-byte
 // aligned.  Needs ring_threads(b) threads and two stages; every thread of the CTA calls it, after a
-// barrier that follows the writes of y and P.  Returns false if a bounded wait gave up.
+// barrier that follows the writes of y and P.  The forward sweep starts at block t0: y must vanish in
+// the rows before it.  Returns false if a bounded wait gave up.
 // ------------------------------------------------------------------------------------------
 constexpr int kRingMax = 6;
 constexpr int kRingHead = 128;
+// Lanes per row (SP), and the warps that solve: warp 0 and those of the rows past the next block.
 template <typename FT>
-__host__ __device__ constexpr int ring_warps(int b) {  // warps that solve: warp 0 and the rows past the next block
-  return 1 + (b > SolveBlock<FT>::BS ? (b - SolveBlock<FT>::BS + 31) / 32 : 0);
+__host__ __device__ constexpr int ring_split() {
+  return 32 / SolveBlock<FT>::BS;
+}
+template <typename FT>
+__host__ __device__ constexpr int ring_warps(int b) {
+  return 1 + (b > SolveBlock<FT>::BS ? (ring_split<FT>() * (b - SolveBlock<FT>::BS) + 31) / 32 : 0);
 }
 template <typename FT>
 __host__ __device__ constexpr int ring_threads(int b) {
@@ -1164,29 +1212,38 @@ __host__ __device__ constexpr int ring_stages(int b, size_t bytes) {
   return s < kRingMax ? (int)s : kRingMax;
 }
 
-// sum_j c(j) x[j] over a block in the order of band_solve_packed: even and odd j apart
-template <typename FT, typename C>
-__device__ __forceinline__ FT block_dot(C&& c, const FT* x) {
+// sum_j c[j] x[j] over a block in the order of band_solve_packed (even and odd j apart): one lane per
+// row, or two lanes 16 apart that hold the even (lane < 16) and the odd terms.
+template <typename FT>
+__device__ __forceinline__ FT block_dot(const FT (&c)[SolveBlock<FT>::BS / ring_split<FT>()], const FT* x) {
   constexpr int BS = SolveBlock<FT>::BS, G = LuTile<FT>::G;
-  FT a0 = 0, a1 = 0;
+  if constexpr (ring_split<FT>() == 1) {
+    FT a0 = 0, a1 = 0;
 #pragma unroll
-  for (int j = 0; j < BS; j += G) {
-    const LuVec<FT> v = *(const LuVec<FT>*)(x + j);
+    for (int j = 0; j < BS; j += G) {
+      const LuVec<FT> v = *(const LuVec<FT>*)(x + j);
 #pragma unroll
-    for (int q = 0; q < G; q += 2) {
-      a0 += c(j + q) * v.v[q];
-      a1 += c(j + q + 1) * v.v[q + 1];
+      for (int q = 0; q < G; q += 2) {
+        a0 += c[j + q] * v.v[q];
+        a1 += c[j + q + 1] * v.v[q + 1];
+      }
     }
+    return a0 + a1;
+  } else {
+    const int h = (threadIdx.x & 31) >> 4;
+    FT a = 0;
+#pragma unroll
+    for (int j = 0; j < BS / 2; ++j) a += c[j] * x[2 * j + h];
+    return a + __shfl_xor_sync(0xffffffffu, a, 16);
   }
-  return a0 + a1;
 }
 
 template <typename FT>
-__device__ __noinline__ bool band_solve_ring(int n, int b, const FT* __restrict__ P, FT* y, unsigned char* ring,
-                                             int stages, int l2d) {
+__device__ __forceinline__ bool band_solve_ring(int n, int b, const FT* __restrict__ P, FT* y, unsigned char* ring,
+                                                int stages, int t0 = 0) {
   constexpr int BS = SolveBlock<FT>::BS;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int cw = ring_warps<FT>(b), nblk = (n + BS - 1) / BS, steps = 2 * nblk;
+  const int cw = ring_warps<FT>(b), nblk = (n + BS - 1) / BS, nf = nblk - t0, steps = nf + nblk;
   const int64_t PB = packed_block_entries<FT>(b);
   uint64_t* full = (uint64_t*)ring;
   uint64_t* empty = full + kRingMax;
@@ -1208,12 +1265,6 @@ __device__ __noinline__ bool band_solve_ring(int n, int b, const FT* __restrict_
   if (wid == cw) {
     if (lane == 0) {
       const uint32_t dbytes = sizeof(FT) * BS * BS, cbytes = (uint32_t)(sizeof(FT) * BS * b);
-      auto block = [&](int s, const FT*& d, const FT*& c) {  // operands of step s
-        const bool fwd = s < nblk;
-        const FT* Pt = P + (int64_t)(fwd ? s : steps - 1 - s) * PB;
-        d = Pt + (fwd ? 0 : BS * BS);
-        c = Pt + 2 * BS * BS + (fwd ? 0 : (int64_t)b * BS);
-      };
       int st = 0;
       uint32_t par = 1;  // parity of the previous use of the stage
       int issued = 0;
@@ -1222,13 +1273,10 @@ __device__ __noinline__ bool band_solve_ring(int n, int b, const FT* __restrict_
           *dead = 1;
           break;
         }
-        const FT *d, *c;
-        if (l2d > 0 && s + l2d < steps) {
-          block(s + l2d, d, c);
-          tc::bulk_prefetch_l2(d, dbytes);
-          if (cbytes) tc::bulk_prefetch_l2(c, cbytes);
-        }
-        block(s, d, c);
+        const bool fwd = s < nf;
+        const FT* Pt = P + (int64_t)(fwd ? t0 + s : steps - 1 - s) * PB;
+        const FT* d = Pt + (fwd ? 0 : BS * BS);
+        const FT* c = Pt + 2 * BS * BS + (fwd ? 0 : (int64_t)b * BS);
         unsigned char* dst = ring + kRingHead + st * sb;
         tc::mbar_arrive_expect_tx(full + st, dbytes + cbytes);
         tc::bulk_load(dst, d, dbytes, full + st);
@@ -1246,52 +1294,72 @@ __device__ __noinline__ bool band_solve_ring(int n, int b, const FT* __restrict_
     }
     __syncwarp();
   } else if (wid < cw) {
-    const int r = wid == 0 ? lane % BS : BS + tid - 32;  // coupled row of this thread
-    const bool mine = r < b && (wid > 0 || lane < BS);
-    int st = 0;
+    constexpr int SP = ring_split<FT>(), J = BS / SP;  // lanes per row, terms per lane
+    const int h = SP == 1 ? 0 : lane >> 4, rl = lane % BS;
+    const int r = wid == 0 ? rl : BS + (wid - 1) * BS + rl;  // coupled row of this lane
+    const bool mine = r < b;
+    FT d[J], c[J];  // this lane's terms of the diagonal inverse (warp 0) and of the coupling
+    int st = 0;      // stage and parity of the next operands
     uint32_t par = 0;
     bool live = true;
-    for (int s = 0; s < steps; ++s) {
-      const bool fwd = s < nblk;
-      const int k0 = (fwd ? s : steps - 1 - s) * BS;
-      const FT* D = (const FT*)(ring + kRingHead + st * sb);
-      const FT* C = D + BS * BS + r;
-      if (live && !tc::mbar_wait(full + st, par)) {
+    auto arrived = [&] { return tc::mbar_test(full + st, par); };
+    auto settle = [&](bool there) {  // the next operands are there, or the wait has given up
+      if (!there && live && !tc::mbar_wait(full + st, par)) {
         live = false;
         *dead = 1;
       }
       __syncwarp();
-      FT c[BS];
-      if (wid == 0) {
-        // x = (diagonal inverse) y; FP64: the even terms on lanes 0 .. 15, the odd ones on 16 .. 31
-        FT x;
-        if constexpr (BS == 32) {
-          x = block_dot<FT>([&](int j) { return D[j * BS + lane]; }, y + k0);
-        } else {
-          x = 0;
+    };
+    auto load = [&](FT (&v)[J], int row, const FT* rows) {
+      constexpr int G = LuTile<FT>::G;
+      const FT* R = rows + row * BS;
+      if constexpr (SP == 1) {
 #pragma unroll
-          for (int j = 0; j < BS; j += 2) x += D[(j + lane / BS) * BS + lane % BS] * y[k0 + j + lane / BS];
-          x += __shfl_xor_sync(0xffffffffu, x, BS);
+        for (int j = 0; j < BS; j += G) {
+          const LuVec<FT> w = *(const LuVec<FT>*)(R + packed_at<FT>(row, j));
+#pragma unroll
+          for (int i = 0; i < G; ++i) v[j + i] = w.v[i];
         }
-        if (mine) {
+      } else {
 #pragma unroll
-          for (int j = 0; j < BS; ++j) c[j] = C[j * b];
-        }
-        __syncwarp();
-        if (lane < BS && k0 + lane < n) y[k0 + lane] = x;
-      } else if (mine) {
-#pragma unroll
-        for (int j = 0; j < BS; ++j) c[j] = C[j * b];
+        for (int j = 0; j < J; ++j) v[j] = R[packed_at<FT>(row, SP * j + h)];
       }
-      if (cw > 1) asm volatile("bar.sync 1, %0;" ::"r"(32 * cw) : "memory");
-      else __syncwarp();
-      const int i = fwd ? k0 + BS + r : k0 - 1 - r;
-      if (mine && i >= 0 && i < n) y[i] -= block_dot<FT>([&](int j) { return c[j]; }, y + k0);
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(empty + st);
+    };
+    auto load_d = [&] { load(d, rl, (const FT*)(ring + kRingHead + st * sb)); };
+    auto load_c = [&] {
+      if (mine) load(c, r, (const FT*)(ring + kRingHead + st * sb) + BS * BS);
+    };
+#pragma unroll
+    for (int j = 0; j < J; ++j) c[j] = (FT)0;
+    settle(arrived());
+    if (wid == 0) load_d();
+    load_c();
+    for (int s = 0; s < steps; ++s) {
+      const bool fwd = s < nf, more = s + 1 < steps;
+      const int k0 = (fwd ? t0 + s : steps - 1 - s) * BS, i = fwd ? k0 + BS + r : k0 - 1 - r;
+      const bool add = mine && i >= 0 && i < n;
+      const int used = st;
       if (++st == stages) {
         st = 0;
         par ^= 1;
+      }
+      const bool there = more && arrived();  // asked for early, used after the diagonal block
+      if (wid == 0) {
+        const FT x = block_dot<FT>(d, y + k0);
+        __syncwarp();
+        if (h == 0 && k0 + rl < n) y[k0 + rl] = x;
+      }
+      if (cw > 1) asm volatile("bar.sync 1, %0;" ::"r"(32 * cw) : "memory");
+      else __syncwarp();
+      const FT yi = add ? y[i] : (FT)0;
+      const FT t = block_dot<FT>(c, y + k0);
+      if (add && h == 0) y[i] = yi - t;
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(empty + used);
+      if (more) {
+        settle(there);
+        if (wid == 0) load_d();
+        load_c();
       }
     }
   }

@@ -189,7 +189,8 @@ __host__ __device__ inline LocalPlan apply_plan(int max_n, int max_nt, int max_b
   p.racc = 0;
   p.red = o; o += sizeof(double) * 40;
   o = align_up(o, 16);
-  p.win = o; o += align_up(sizeof(FT) * align_up(max_n, dev::SolveBlock<FT>::BS), 16);
+  p.win = o; o += sizeof(FT) * align_up(max_n, dev::SolveBlock<FT>::BS);
+  if (stages) o = align_up(o, 128);  // the bulk copies write whole 128-byte lines
   p.flag = o;
   if (stages) o += dev::kRingHead + stages * dev::ring_stage_bytes<FT>(max_b);
   p.total = o;
@@ -342,19 +343,16 @@ __device__ __forceinline__ void for_row(const LocalArgs& A, const SubMeta& m, in
   const int64_t first = m.nnz_off + bw.x + (m.slice == 32 ? a & 31 : 0);
   const double* v = A.csr + first;
   const int32_t* c = A.colidx + first;
-  for (int k = 0; k < bw.y; k += 6) {
+  int k = 0;
+  for (; k + 6 <= bw.y; k += 6) {  // six entries in flight
     double val[6];
     int32_t col[6];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      const bool in = k + i < bw.y;
-      val[i] = in ? v[(k + i) * h] : 0.0;
-      col[i] = in ? c[(k + i) * h] : -1;
-    }
+    for (int i = 0; i < 6; ++i) val[i] = v[(k + i) * h], col[i] = c[(k + i) * h];
 #pragma unroll
-    for (int i = 0; i < 6; ++i)
-      if (k + i < bw.y) f(val[i], col[i]);
+    for (int i = 0; i < 6; ++i) f(val[i], col[i]);
   }
+  for (; k < bw.y; ++k) f(v[k * h], c[k * h]);
 }
 
 // y = (packed operands)^-1 y through the ring where it has two stages and the CTA the threads, else
@@ -366,8 +364,7 @@ struct Ring {
 template <typename FT, bool PF>
 __device__ bool triangular_solves(const LocalArgs& A, const SubMeta& m, const FT* Dv, FT* yv, const Ring& ring) {
   if (ring.stages >= 2 && (int)blockDim.x >= dev::ring_threads<FT>(m.b))
-    return dev::band_solve_ring<FT>(m.n, m.b, Dv, yv, ring.mem, ring.stages,
-                                    A.l2_dist > 0 ? ring.stages + A.l2_dist : 0);
+    return dev::band_solve_ring<FT>(m.n, m.b, Dv, yv, ring.mem, ring.stages);
   dev::band_solve_packed<FT, PF>(m.n, m.b, Dv, yv, A.l2_dist);
   return true;
 }
@@ -376,33 +373,28 @@ __device__ bool triangular_solves(const LocalArgs& A, const SubMeta& m, const FT
 // (columns < n) when the factors are FP32.  s and yv are in shared memory (s may be rhs's copy).
 // Returns false if a bounded wait gave up.
 template <typename FT, bool PF>
-__device__ bool local_solve(const LocalArgs& A, const SubMeta& m, const FT* Dv, const double* rhs, double rhs_norm,
-                            double* s, FT* yv, double* red, const Ring& ring) {
+__device__ __forceinline__ bool local_solve(const LocalArgs& A, const SubMeta& m, const FT* Dv, const double* rhs,
+                                            double rhs_norm, double* s, FT* yv, double* red, const Ring& ring) {
   const int n = m.n;
   for (int a = threadIdx.x; a < n; a += blockDim.x) yv[a] = (FT)rhs[a];
   __syncthreads();
-  bool ok = triangular_solves<FT, PF>(A, m, Dv, yv, ring);
-  for (int a = threadIdx.x; a < n; a += blockDim.x) s[a] = (double)yv[a];
-  __syncthreads();
-  if (sizeof(FT) == 4) {
-    for (int sw = 0; ok && sw < A.ir_max; ++sw) {
-      double loc = 0.0;
-      for (int a = threadIdx.x; a < n; a += blockDim.x) {
-        double acc = rhs[a];
-        for_row(A, m, a, [&](double v, int32_t col) {
-          if (col < n) acc -= v * s[col];
-        });
-        yv[a] = (FT)acc;
-        loc += acc * acc;
-      }
-      const double rn = sqrt(dev::block_sum(loc, red));
-      if (!(rn > A.ir_rtol * rhs_norm)) break;
-      ok = triangular_solves<FT, PF>(A, m, Dv, yv, ring);
-      for (int a = threadIdx.x; a < n; a += blockDim.x) s[a] += (double)yv[a];
-      __syncthreads();
+  for (int sw = 0;; ++sw) {
+    if (!triangular_solves<FT, PF>(A, m, Dv, yv, ring)) return false;
+    for (int a = threadIdx.x; a < n; a += blockDim.x) s[a] = (sw ? s[a] : 0.0) + (double)yv[a];
+    __syncthreads();
+    if (sizeof(FT) == 8 || sw >= A.ir_max) return true;
+    double loc = 0.0;
+    for (int a = threadIdx.x; a < n; a += blockDim.x) {
+      double acc = rhs[a];
+      for_row(A, m, a, [&](double v, int32_t col) {
+        if (col < n) acc -= v * s[col];
+      });
+      yv[a] = (FT)acc;
+      loc += acc * acc;
     }
+    const double rn = sqrt(dev::block_sum(loc, red));
+    if (!(rn > A.ir_rtol * rhs_norm)) return true;
   }
-  return ok;
 }
 
 // Damped Jacobi sweeps on a proposed local start (in xt's local unknowns): they remove the
@@ -427,7 +419,7 @@ __device__ bool smooth_proposal(const LocalArgs& A, const SubMeta& m, double* xt
 // one CTA per subdomain, into A.out (concatenated local vectors).
 template <int LAW>
 __global__ void __launch_bounds__(256) k_guess_smooth(LocalArgs A) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   double* xt = (double*)smem;
   double* racc = xt + A.max_nt;
   const int sub = blockIdx.x, nd = A.ndof;
@@ -450,7 +442,7 @@ __global__ void __launch_bounds__(256) k_guess_smooth(LocalArgs A) {
 template <int LAW, typename FT, int MAXT>
 __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : LAW == NLS_LAW_DIFFUSION ? 2 : 1))
     k_local_newton(LocalArgs A) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   const LocalPlan P = newton_plan<FT>(A.max_n, A.max_nt, A.max_b);
   double* xt = (double*)(smem + P.xt);
   double* racc = (double*)(smem + P.racc);  // residual being assembled
@@ -487,10 +479,8 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : LAW == NLS_LAW_DIFFUS
     double* r = A.work + m.vec_off;                  // current residual
     double* s = A.work + A.work_stride + m.vec_off;  // Newton step
     // the LU window serves the solves: the solve vector, then the ring of operands
-    const size_t y_bytes = align_up(sizeof(FT) * align_up(n, dev::SolveBlock<FT>::BS), 16);
-    const size_t win_bytes = sizeof(FT) * win_cap;
-    const Ring ring{(unsigned char*)win + y_bytes,
-                    y_bytes < win_bytes ? dev::ring_stages<FT>(m.b, win_bytes - y_bytes) : 0};
+    const size_t ring_at = align_up(P.win + sizeof(FT) * align_up(n, dev::SolveBlock<FT>::BS), 128);
+    const Ring ring{smem + ring_at, ring_at < P.flag ? dev::ring_stages<FT>(m.b, P.flag - ring_at) : 0};
     for (int t = tid; t < m.nt; t += blockDim.x)
       xt[t] = A.x[(int64_t)A.tnode_gid[m.tnode_off + t / nd] * nd + t % nd];
     __syncthreads();
@@ -646,7 +636,7 @@ __host__ __device__ inline LocalPlan factor_plan(int max_b) {
 // MAXT = 256: three CTAs per SM; MAXT = 512: one, for at most one subdomain per SM.
 template <typename FT, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : 1) k_local_factor(LocalArgs A) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   const LocalPlan P = factor_plan<FT>(A.max_b);
   FT* win = (FT*)(smem + P.win);
   int* flag = (int*)(smem + P.flag);
@@ -668,8 +658,9 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : 1) k_local_factor(Loca
 // ------------------------------------------------------------------------------------------
 // k_local_apply: out[owned] = (R_i DF(v_i) P_i)^-1 R_i DF(v_i) v  (+ add[owned])
 // ------------------------------------------------------------------------------------------
-template <typename FT>
-__global__ void __launch_bounds__(512) k_local_apply(LocalArgs A) {
+// MAXT = 256: the whole register budget; 128: three CTAs per SM.
+template <typename FT, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT <= 128 ? 3 : 1) k_local_apply(LocalArgs A) {
   extern __shared__ __align__(128) unsigned char smem[];
   const LocalPlan P = apply_plan<FT>(A.max_n, A.max_nt, A.max_b, A.ring);
   double* yt = (double*)(smem + P.xt);
@@ -705,7 +696,7 @@ __global__ void __launch_bounds__(512) k_local_apply(LocalArgs A) {
 // ------------------------------------------------------------------------------------------
 template <int LAW>
 __global__ void __launch_bounds__(256) k_harmonic(LocalArgs A) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   const SmemPlan P = harmonic_plan(A.max_n, A.max_nt, A.max_b);
   double* xt = (double*)(smem + P.xt);
   double* yv = (double*)(smem + P.yv);
@@ -749,7 +740,7 @@ __global__ void __launch_bounds__(256) k_harmonic(LocalArgs A) {
 
 template <int LAW>
 __global__ void __launch_bounds__(256, 2) k_galerkin(LocalArgs A) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   const SmemPlan P = smem_plan<double>(A.max_n, A.max_nt);
   double* xt = (double*)(smem + P.xt);
   const int j = blockIdx.x, tid = threadIdx.x, nd = A.ndof;
@@ -811,7 +802,7 @@ __host__ __device__ constexpr size_t coarse_window(int b0) {
 }
 template <typename FT>
 __global__ void __launch_bounds__(1024) k_coarse_factor(int N0, int b0, const double* A0, FT* F, FT* Dinv, int* status) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   FT* win = (FT*)smem;
   int* flag = (int*)(smem + align_up(sizeof(FT) * coarse_window<FT>(b0), 16));
   const int64_t total = (int64_t)N0 * (2 * b0 + 1);
@@ -828,23 +819,164 @@ __global__ void __launch_bounds__(1024) k_coarse_factor(int N0, int b0, const do
   if (threadIdx.x == 0) *status = bad ? ST_PIVOT : ST_OK;
 }
 
-// Columns of A_0^-1 from the band factors (one CTA per column, the solve vector in shared
-// memory): one solve A_0 z = e_col in the factors' precision (the forward sweep starts at the
-// block of `col`, above which e_col and z vanish), stored in that precision and transposed
-// (AinvT[col][row]) so that the GEMV below reads it coalesced.  FP32 columns are refined where
-// they are applied (coarse_solve): the FP64 residual of one vector costs N0 (2 b0 + 1)
-// multiply-adds, that of every column of the inverse N0 times as many.
+// Bytes of the solve vector before the operand ring.
 template <typename FT>
-__global__ void __launch_bounds__(512) k_coarse_inverse(int N0, int b0, const FT* Dinv, FT* AinvT, int l2d) {
-  extern __shared__ __align__(16) unsigned char smem[];
+__host__ __device__ constexpr size_t coarse_solve_vector(int N0) {
+  return (sizeof(FT) * (size_t)((N0 + dev::SolveBlock<FT>::BS - 1) / dev::SolveBlock<FT>::BS * dev::SolveBlock<FT>::BS) + 127) /
+         128 * 128;
+}
+
+// Columns of A_0^-1 from the band factors: the solves A_0 z = e_col in the factors' precision, stored in
+// that precision and transposed (AinvT[col][row]) so that the GEMV below reads it coalesced.  FP32
+// columns are refined where they are applied (coarse_solve): the FP64 residual of one vector costs
+// N0 (2 b0 + 1) multiply-adds, that of every column of the inverse N0 times as many.  The forward
+// sweep starts at the block of the column, above which e_col and z vanish.
+//
+// k_coarse_inverse: one CTA per column, through the operand ring.
+template <typename FT>
+__global__ void __launch_bounds__(256) k_coarse_inverse(int N0, int b0, const FT* Dinv, FT* AinvT, int stages, int* err) {
+  extern __shared__ __align__(128) unsigned char smem[];
   FT* y = (FT*)smem;
-  constexpr int BS = dev::SolveBlock<FT>::BS;
   for (int col = blockIdx.x; col < N0; col += gridDim.x) {
     for (int a = threadIdx.x; a < N0; a += blockDim.x) y[a] = (a == col) ? (FT)1 : (FT)0;
     __syncthreads();
-    dev::band_solve_packed<FT, false>(N0, b0, Dinv, y, l2d, col / BS);
+    if (!dev::band_solve_ring<FT>(N0, b0, Dinv, y, smem + coarse_solve_vector<FT>(N0), stages,
+                                  col / dev::SolveBlock<FT>::BS) &&
+        threadIdx.x == 0)
+      *err = 1;
     for (int a = threadIdx.x; a < N0; a += blockDim.x) AinvT[(int64_t)col * N0 + a] = y[a];
     __syncthreads();
+  }
+}
+
+// k_coarse_inverse_blocks: 32 columns per CTA.  With one column per CTA every column streams all packed
+// operands from L2 (N_0 = 5235, b_0 = 197: 38 GB, 3.5 ms).  Here a step's operands are staged once in
+// shared memory for 32 columns (lane = column): each warp holds the block of its columns in registers
+// and takes rows of the operands, read as broadcast 16-byte groups (2.4 ms, bound by those reads).
+// The rows that a block couples to are kept in a window of shared memory; the forward result of a
+// block goes through AinvT.  A column's sums are those of band_solve_packed: even and odd terms
+// apart, blocks in order.
+template <typename FT>
+__host__ __device__ constexpr int inverse_blocks(int b0) {  // blocks of the window
+  constexpr int BS = dev::SolveBlock<FT>::BS;
+  return 1 + (b0 + BS - 1) / BS;
+}
+template <typename FT>
+__host__ __device__ constexpr size_t inverse_smem(int b0, int buffers) {
+  constexpr size_t BS = dev::SolveBlock<FT>::BS;
+  return sizeof(FT) * (buffers * BS * (BS + (b0 + 3) / 4 * 4) + inverse_blocks<FT>(b0) * BS * 33);
+}
+// R consecutive rows of the operands, from row r, times the block held in v
+template <int R, typename FT>
+__device__ __forceinline__ void inverse_dots(const FT* rows, int r, const FT* v, FT* out) {
+  constexpr int BS = dev::SolveBlock<FT>::BS, G = dev::LuTile<FT>::G;
+  using Vec = dev::LuVec<FT>;
+  FT a0[R], a1[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) a0[i] = a1[i] = 0;
+#pragma unroll
+  for (int j = 0; j < BS; j += G) {
+    Vec w[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) w[i] = *(const Vec*)(rows + (r + i) * BS + dev::packed_at<FT>(r + i, j));
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int q = 0; q < G; q += 2) {
+        a0[i] += w[i].v[q] * v[j + q];
+        a1[i] += w[i].v[q + 1] * v[j + q + 1];
+      }
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i) out[i] = a0[i] + a1[i];
+}
+template <typename FT>
+__global__ void __launch_bounds__(256) k_coarse_inverse_blocks(int N0, int b0, const FT* __restrict__ Dinv,
+                                                                FT* AinvT, int buffers) {
+  constexpr int BS = dev::SolveBlock<FT>::BS, G = dev::LuTile<FT>::G, LD = 33;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int SE = BS * (BS + b0), SP = BS * (BS + (b0 + 3) / 4 * 4);  // operands of one step, and their room
+  FT* ops = (FT*)smem;
+  FT* win = ops + buffers * SP;  // row i of the matrix at (i mod WR) LD, a column per lane
+  const int WB = inverse_blocks<FT>(b0), WR = WB * BS;
+  const int nblk = (N0 + BS - 1) / BS, c0 = blockIdx.x * 32, t0 = c0 / BS;
+  const int64_t PB = dev::packed_block_entries<FT>(b0);
+  const int steps = (nblk - t0) + nblk;
+  auto block_of = [&](int s) { return s < nblk - t0 ? t0 + s : steps - 1 - s; };
+  auto stage = [&](int s, FT* dst) {  // operands of step s
+    if (s < steps) {
+      const bool fwd = s < nblk - t0;
+      const FT* P = Dinv + (int64_t)block_of(s) * PB;
+      const FT *d = P + (fwd ? 0 : BS * BS), *c = P + 2 * BS * BS + (fwd ? 0 : (int64_t)b0 * BS);
+      for (int e = tid; e < SE / G; e += blockDim.x) {
+        const FT* src = e < BS * BS / G ? d + e * G : c + (e - BS * BS / G) * G;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(tc::smem_u32(dst + e * G)), "l"(src)
+                     : "memory");
+      }
+    }
+    dev::cp_async_commit();
+  };
+  // the rows of block u enter the window: unit columns (forward) or the forward result
+  auto enter = [&](int u, bool fwd) {
+    if (u < 0 || u >= nblk) return;
+    FT* w = win + (u % WB) * BS * LD;
+#pragma unroll
+    for (int q = 0; q < BS * 32 / 256; ++q) {
+      const int e = tid + 256 * q, r = e % BS, c = e / BS, i = u * BS + r, col = c0 + c;
+      FT v = 0;
+      if (fwd) v = (i == col && i < N0) ? (FT)1 : (FT)0;
+      else if (u >= t0 && i < N0 && col < N0) v = AinvT[(int64_t)col * N0 + i];
+      w[r * LD + c] = v;
+    }
+  };
+  stage(0, ops);
+  for (int q = 0; q < WB; ++q) enter(t0 + q, true);
+  for (int s = 0; s < steps; ++s) {
+    const bool fwd = s < nblk - t0;
+    const int t = block_of(s), k0 = t * BS;
+    if (s == nblk - t0) {  // turn: the last blocks, all written out by this CTA
+      __syncthreads();
+      for (int q = 0; q < WB; ++q) enter(nblk - 1 - q, false);
+    }
+    FT* cur = ops + (buffers > 1 ? (s & 1) * SP : 0);
+    if (buffers == 1 && s > 0) stage(s, ops);
+    dev::cp_async_wait<0>();
+    __syncthreads();
+    if (buffers > 1) stage(s + 1, ops + ((s + 1) & 1) * SP);
+    constexpr int RW = BS / 8;  // rows of the diagonal block per warp (eight warps)
+    const int slot = (t % WB) * BS;
+    FT v[BS], x[RW], y[4];
+    FT* blk = win + slot * LD + lane;
+#pragma unroll
+    for (int j = 0; j < BS; ++j) v[j] = blk[j * LD];
+    inverse_dots<RW, FT>(cur, wid * RW, v, x);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < RW; ++i) blk[(wid * RW + i) * LD] = (k0 + wid * RW + i < N0) ? x[i] : (FT)0;
+    __syncthreads();
+    // the solved block to global memory, rows along the lanes
+#pragma unroll
+    for (int q = 0; q < BS * 32 / 256; ++q) {
+      const int r = (tid + 256 * q) % BS, c = (tid + 256 * q) / BS;
+      if (k0 + r < N0 && c0 + c < N0) AinvT[(int64_t)(c0 + c) * N0 + k0 + r] = win[(slot + r) * LD + c];
+    }
+#pragma unroll
+    for (int j = 0; j < BS; ++j) v[j] = blk[j * LD];
+    for (int r = wid * 4; r < b0; r += 32) {
+      inverse_dots<4, FT>(cur + BS * BS, r, v, y);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int row = fwd ? k0 + BS + r + i : k0 - 1 - r - i;
+        int at = fwd ? slot + BS + r + i : slot - 1 - r - i;  // row mod WR
+        at = at >= WR ? at - WR : at < 0 ? at + WR : at;
+        if (r + i < b0 && row >= 0 && row < N0) win[at * LD + lane] -= y[i];
+      }
+    }
+    __syncthreads();
+    // block t leaves the window; the block beyond it on the other side takes its place
+    if (fwd) enter(t + WB, true);
+    else enter(t - WB, false);
   }
 }
 
@@ -857,6 +989,7 @@ constexpr int kGemvChunks = 16;
 // Largest coarse dimension with an explicit inverse (N0^2 entries in the factors' precision:
 // 1 GB in FP32 at the limit); larger coarse problems use the one-CTA band solve.
 constexpr int kMaxInverseN0 = 16384;
+constexpr int kInverseColumns = 2048;  // coarse dofs up to which the inverse is formed column by column
 template <typename FT>
 __global__ void __launch_bounds__(256) k_dense_gemv_t(int N0, const FT* AinvT, const double* g, double* part,
                                                        const int* skip) {
@@ -945,18 +1078,24 @@ __global__ void __launch_bounds__(256) k_coarse_residual(int N0, int b0, const d
 // One coarse solve with the packed band factors in one CTA (the solve vector in shared memory):
 // z = (accumulate ? z : 0) + A_0^-1 rhs in the factors' precision.  With *skip set (a refinement
 // that has converged) the kernel does nothing; `reset`, if given, is cleared (the refinement flag
-// of the solve that starts here).  Needs blockDim.x >= 32 + b0.
+// of the solve that starts here).  Needs blockDim.x >= 32 + b0.  `stages`: stages of the operand ring
+// behind the solve vector (at least two, and ring_threads threads), or 0: operands in registers.
 template <typename FT>
 __global__ void __launch_bounds__(512) k_coarse_band_solve(int N0, int b0, const FT* Dinv, const double* rhs,
                                                              double* z, int accumulate, const int* skip, int* reset,
-                                                             int l2d) {
+                                                             int l2d, int stages, int* err) {
   if (skip && *skip) return;
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   FT* y = (FT*)smem;
   if (reset && threadIdx.x == 0) *reset = 0;
   for (int a = threadIdx.x; a < N0; a += blockDim.x) y[a] = (FT)rhs[a];
   __syncthreads();
-  dev::band_solve_packed<FT, true>(N0, b0, Dinv, y, l2d);
+  if (stages) {
+    if (!dev::band_solve_ring<FT>(N0, b0, Dinv, y, smem + coarse_solve_vector<FT>(N0), stages) && threadIdx.x == 0)
+      *err = 1;
+  } else {
+    dev::band_solve_packed<FT, true>(N0, b0, Dinv, y, l2d);
+  }
   for (int a = threadIdx.x; a < N0; a += blockDim.x) z[a] = (accumulate ? z[a] : 0.0) + (double)y[a];
 }
 
@@ -1237,14 +1376,16 @@ int local_threads(const Context& c) {
 }
 
 // CTA size of the tangent application: the solving warps and the copying one, and enough threads for
-// the matrix products -- 512 while every subdomain has an SM to itself, 256 while two share one.
+// the matrix products -- 256 while every subdomain has an SM to itself, else 128, three CTAs of which
+// share an SM.  (A kernel for 512 threads is held to 128 registers, and a solve step took 1900 cycles
+// instead of 750.)
 int apply_threads(const Context& c) {
   const int ring = c.opt.local_precision == NLS_PREC_FP32_IR ? dev::ring_threads<float>(c.ov.max_b)
                                                             : dev::ring_threads<double>(c.ov.max_b);
   const int need = std::max(64, std::max(ring, min_local_threads(c)));
   if (c.dev && c.dev->apply_T) return std::max(c.dev->apply_T, need);
   const int nsm = c.dev ? c.dev->nsm : 152;
-  return std::max(need, c.ov.count <= nsm ? 512 : c.ov.count <= 2 * nsm ? 256 : 128);
+  return std::max(need, c.ov.count <= nsm ? 256 : 128);
 }
 
 bool fp32_local(const Context& c) { return c.opt.local_precision == NLS_PREC_FP32_IR; }
@@ -1510,11 +1651,12 @@ void launch_local_newton(Context& c, const double* x, double* out, double load, 
 }
 
 // Stages of the tangent application's operand ring: as many as leave room for the CTAs per SM that the
-// subdomains fill (two at most), at least two.
+// subdomains fill (three at most), at least two.  (4096 solves of n = 3120, b = 83 in one launch are
+// bound by HBM with three stages at three CTAs per SM or six at one.)
 template <typename FT>
 int apply_ring_stages(const Context& c) {
   const Dev& D = *c.dev;
-  const size_t per_sm = D.smem_optin + 1024, want = c.ov.count > D.nsm ? 2 : 1;
+  const size_t per_sm = D.smem_optin + 1024, want = std::min(3, (c.ov.count + D.nsm - 1) / D.nsm);
   for (int st = dev::kRingMax; st >= 2; --st) {
     const size_t sm = apply_plan<FT>(c.ov.max_n, c.ov.max_nt, c.ov.max_b, st).total;
     if (sm <= D.smem_optin - 128 && ((sm + 1024) * want <= per_sm || st == 2)) return st;
@@ -1522,22 +1664,23 @@ int apply_ring_stages(const Context& c) {
   return 0;
 }
 
-void launch_local_apply(Context& c, const double* v, const double* add, double* out) {
+template <typename FT>
+void launch_apply_t(Context& c, LocalArgs& A, int T) {
   Dev& D = *c.dev;
-  LocalArgs A = make_args(c, c.ov, D.ov);
+  A.ring = apply_ring_stages<FT>(c);
+  const size_t sm = apply_plan<FT>(c.ov.max_n, c.ov.max_nt, c.ov.max_b, A.ring).total;
+  const char* name = sizeof(FT) == 4 ? "k_local_apply<float>" : "k_local_apply<double>";
+  if (T <= 128) LAUNCH_NAMED(D, name, (k_local_apply<FT, 128>), c.ov.count, T, sm, A);
+  else LAUNCH_NAMED(D, name, (k_local_apply<FT, 256>), c.ov.count, T, sm, A);
+}
+
+void launch_local_apply(Context& c, const double* v, const double* add, double* out) {
+  LocalArgs A = make_args(c, c.ov, c.dev->ov);
   A.v = v;
   A.add = add;
   A.out = out;
-  const int T = apply_threads(c);
-  if (fp32_local(c)) {
-    A.ring = apply_ring_stages<float>(c);
-    const size_t sm = apply_plan<float>(c.ov.max_n, c.ov.max_nt, c.ov.max_b, A.ring).total;
-    LAUNCH(D, k_local_apply<float>, c.ov.count, T, sm, A);
-  } else {
-    A.ring = apply_ring_stages<double>(c);
-    const size_t sm = apply_plan<double>(c.ov.max_n, c.ov.max_nt, c.ov.max_b, A.ring).total;
-    LAUNCH(D, k_local_apply<double>, c.ov.count, T, sm, A);
-  }
+  if (fp32_local(c)) launch_apply_t<float>(c, A, apply_threads(c));
+  else launch_apply_t<double>(c, A, apply_threads(c));
 }
 
 // ---- autotuner (nls_options.autotune) -------------------------------------------------------
@@ -1589,8 +1732,8 @@ void tune_local_apply(Context& c, const double* v, double* out) {
   D.apply_T = 32;  // the smallest CTA that the kernel takes
   const int need = apply_threads(c);
   std::vector<int> cand;
-  for (int T : {need, need + 32, need + 64, 128, 192, 256, 384, 512})
-    if (T >= need && T <= 512 && std::find(cand.begin(), cand.end(), T) == cand.end()) cand.push_back(T);
+  for (int T : {need, need + 32, need + 64, 128, 192, 256})
+    if (T >= need && T <= 256 && std::find(cand.begin(), cand.end(), T) == cand.end()) cand.push_back(T);
   D.apply_T = need;
   launch_local_apply(c, v, nullptr, out);  // warm-up
   double best = INFINITY;
@@ -1643,7 +1786,7 @@ void check_local_waits(Dev& D) {
   volatile int* e = D.err_host;
   if (!*e) return;
   *e = 0;
-  throw DeviceTimeout("a local triangular solve gave up waiting for its operands");
+  throw DeviceTimeout("a triangular solve gave up waiting for its operands");
 }
 
 // Reads the coarse factorization's status word (synchronises the stream).
@@ -1748,15 +1891,28 @@ void coarse_solve(Context& c, const double* g, double* z) {
   // as above, the steps after convergence returning at once
   const int N0 = c.cs.N0;
   const bool f32 = fp32_coarse(c);
-  const int T = coarse_solve_threads(c);
+  const int b0 = c.cs.b0;
+  const int T = std::max(coarse_solve_threads(c), std::min(512, f32 ? dev::ring_threads<float>(b0) : dev::ring_threads<double>(b0)));
+  // the operand ring behind the solve vector, where two stages of it fit (15 against 18 us per solve at
+  // N_0 = 699, b_0 = 77)
+  auto ring = [&](size_t vec, size_t stage, int threads) {
+    const size_t room = D.smem_optin - 128;
+    if (T < threads || vec + dev::kRingHead + 2 * stage > room) return 0;
+    return (int)std::min<size_t>(dev::kRingMax, (room - vec - dev::kRingHead) / stage);
+  };
   auto band_solve = [&](const double* rhs, int accumulate, const int* skip, int* reset) {
     if (tlu_solve(c, rhs, z, accumulate, skip, reset)) return;  // tiled factors: the cluster solve
-    if (f32)
-      LAUNCH(D, k_coarse_band_solve<float>, 1, T, sizeof(float) * N0, N0, c.cs.b0, (const float*)D.A0dinv, rhs, z,
-             accumulate, skip, reset, c.opt.l2_prefetch);
-    else
-      LAUNCH(D, k_coarse_band_solve<double>, 1, T, sizeof(double) * N0, N0, c.cs.b0, (const double*)D.A0dinv, rhs, z,
-             accumulate, skip, reset, c.opt.l2_prefetch);
+    if (f32) {
+      const size_t vec = coarse_solve_vector<float>(N0), stage = dev::ring_stage_bytes<float>(b0);
+      const int st = ring(vec, stage, dev::ring_threads<float>(b0));
+      LAUNCH(D, k_coarse_band_solve<float>, 1, T, st ? vec + dev::kRingHead + st * stage : sizeof(float) * N0, N0, b0,
+             (const float*)D.A0dinv, rhs, z, accumulate, skip, reset, c.opt.l2_prefetch, st, D.err_dev);
+    } else {
+      const size_t vec = coarse_solve_vector<double>(N0), stage = dev::ring_stage_bytes<double>(b0);
+      const int st = ring(vec, stage, dev::ring_threads<double>(b0));
+      LAUNCH(D, k_coarse_band_solve<double>, 1, T, st ? vec + dev::kRingHead + st * stage : sizeof(double) * N0, N0, b0,
+             (const double*)D.A0dinv, rhs, z, accumulate, skip, reset, c.opt.l2_prefetch, st, D.err_dev);
+    }
   };
   band_solve(g, 0, nullptr, D.cflag);
   const int sweeps = f32 ? c.opt.ir_max_sweeps : 0;
@@ -1863,6 +2019,13 @@ CoarseResult coarse_newton(Context& c, const double* u, double load) {
 // setup on the device
 // ------------------------------------------------------------------------------------------
 namespace {
+
+// The flag that a kernel whose bounded wait gave up sets (host memory, mapped).
+void alloc_err(Dev& D) {
+  CK(cudaHostAlloc(&D.err_host, sizeof(int), cudaHostAllocMapped));
+  *D.err_host = 0;
+  CK(cudaHostGetDevicePointer((void**)&D.err_dev, D.err_host, 0));
+}
 
 void upload_set(Dev& D, const LocalSet& h, DeviceLocalSet& d, bool fp32_factor, bool with_dinv = true) {
   d.count = h.count;
@@ -2009,9 +2172,7 @@ int device_setup(Context& c) {
     CK(cudaMemsetAsync(D.phase, 0, sizeof(unsigned long long) * 8, D.s));
     CK(cudaDeviceGetAttribute(&D.clock_khz, cudaDevAttrClockRate, c.device));
     CK(cudaMallocHost(&D.h_scal, sizeof(double) * (kMaxGmresVecs + 8)));
-    CK(cudaHostAlloc(&D.err_host, sizeof(int), cudaHostAllocMapped));
-    *D.err_host = 0;
-    CK(cudaHostGetDevicePointer((void**)&D.err_dev, D.err_host, 0));
+    alloc_err(D);
     // kernel attributes for large dynamic shared memory
     const size_t lim = D.smem_optin;
     auto need = [&](size_t b, const char* what) {
@@ -2038,14 +2199,16 @@ int device_setup(Context& c) {
     set_smem(k_local_newton<NLS_LAW_DIFFUSION, double, 256>, lim);
     set_smem(k_local_newton<NLS_LAW_NEOHOOKE, float, 256>, lim);
     set_smem(k_local_newton<NLS_LAW_NEOHOOKE, double, 256>, lim);
-    set_smem(k_local_apply<float>, lim);
+    set_smem(k_local_apply<float, 128>, lim);
+    set_smem(k_local_apply<float, 256>, lim);
+    set_smem(k_local_apply<double, 128>, lim);
+    set_smem(k_local_apply<double, 256>, lim);
     set_smem(k_local_factor<float, 256>, lim);
     set_smem(k_local_factor<double, 256>, lim);
     set_smem(k_local_factor<float, 512>, lim);
     set_smem(k_local_factor<double, 512>, lim);
     set_smem(k_guess_smooth<NLS_LAW_DIFFUSION>, lim);
     set_smem(k_guess_smooth<NLS_LAW_NEOHOOKE>, lim);
-    set_smem(k_local_apply<double>, lim);
     set_smem(k_harmonic<NLS_LAW_DIFFUSION>, lim);
     set_smem(k_harmonic<NLS_LAW_NEOHOOKE>, lim);
     set_smem(k_galerkin<NLS_LAW_DIFFUSION>, lim);
@@ -2089,6 +2252,8 @@ int device_setup(Context& c) {
         D.gpart = D.alloc<double>((size_t)cs.N0 * kGemvChunks);
         set_smem(k_coarse_inverse<float>, lim);
         set_smem(k_coarse_inverse<double>, lim);
+        set_smem(k_coarse_inverse_blocks<float>, lim);
+        set_smem(k_coarse_inverse_blocks<double>, lim);
       }
       D.p0_rowptr = D.upload(cs.p0_rowptr);
       D.p0_col = D.upload(cs.p0_col);
@@ -2209,14 +2374,28 @@ void coarse_inverse_launch(Context& c) {
   Dev& D = *c.dev;
   if (!D.ainv) return;
   const int N0 = c.cs.N0;
-  const int T = std::max(64, (32 + c.cs.b0 + 31) / 32 * 32);
-  const int grid = std::min(N0, D.nsm * 8);
+  const int b0 = c.cs.b0;
+  // one CTA per column while that is bound by the latency of a column's steps: up to kInverseColumns
+  // columns and the half bandwidth of a 256-thread CTA (N_0 = 699, b_0 = 77: 158 us with 32 columns per
+  // CTA), then 32 columns per CTA, which read the operands 32 times less often
+  auto run = [&](auto columns, auto blocks, const char* name, int threads, size_t vec, size_t stage, size_t two,
+                 size_t one, auto* Dinv, auto* Ainv) {
+    const size_t ring = vec + dev::kRingHead + 3 * stage;
+    if (N0 <= kInverseColumns && threads <= 256 && ring <= D.smem_optin - 128) {
+      LAUNCH_NAMED(D, name, columns, std::min(N0, D.nsm * 16), threads, ring, N0, b0, Dinv, Ainv, 3, D.err_dev);
+    } else {
+      const int buffers = two <= D.smem_optin ? 2 : 1;  // half bandwidths past about 400 in FP64: one
+      LAUNCH_NAMED(D, name, blocks, (N0 + 31) / 32, 256, buffers == 2 ? two : one, N0, b0, Dinv, Ainv, buffers);
+    }
+  };
   if (fp32_coarse(c))
-    LAUNCH(D, k_coarse_inverse<float>, grid, T, sizeof(float) * N0, N0, c.cs.b0, (const float*)D.A0dinv,
-           (float*)D.ainv, c.opt.l2_prefetch);
+    run(k_coarse_inverse<float>, k_coarse_inverse_blocks<float>, "k_coarse_inverse<float>", dev::ring_threads<float>(b0),
+        coarse_solve_vector<float>(N0), dev::ring_stage_bytes<float>(b0), inverse_smem<float>(b0, 2),
+        inverse_smem<float>(b0, 1), (const float*)D.A0dinv, (float*)D.ainv);
   else
-    LAUNCH(D, k_coarse_inverse<double>, grid, T, sizeof(double) * N0, N0, c.cs.b0, (const double*)D.A0dinv,
-           (double*)D.ainv, c.opt.l2_prefetch);
+    run(k_coarse_inverse<double>, k_coarse_inverse_blocks<double>, "k_coarse_inverse<double>",
+        dev::ring_threads<double>(b0), coarse_solve_vector<double>(N0), dev::ring_stage_bytes<double>(b0),
+        inverse_smem<double>(b0, 2), inverse_smem<double>(b0, 1), (const double*)D.A0dinv, (double*)D.ainv);
 }
 
 // The tangent phase's coarse work at u_0, first part (issued on D.s): DF(u_0) for the coarse term
@@ -2899,6 +3078,7 @@ int band_solve(int device, int32_t n, int32_t b, const double* band, const doubl
       device_free(c);
       return NLS_E_UNSUPPORTED;  // the one-CTA window or the solve vector exceeds shared memory
     }
+    alloc_err(D);
     const size_t nw = (size_t)n * (2 * b + 1);
     D.A0 = D.alloc<double>(nw);
     CK(cudaMemcpyAsync(D.A0, band, sizeof(double) * nw, cudaMemcpyHostToDevice, D.s));
@@ -2940,6 +3120,7 @@ int band_solve(int device, int32_t n, int32_t b, const double* band, const doubl
     }
     sync(D);
     tlu_check_solves(c);
+    check_local_waits(D);
   } catch (const DeviceTimeout&) {
     status = NLS_E_DEVICE_TIMEOUT;
   } catch (const CudaFailure&) {
