@@ -1202,6 +1202,14 @@ __global__ void k_mask(int64_t n, const uint8_t* free_dof, double* x) {
     if (!free_dof[i]) x[i] = 0.0;
 }
 
+// x = v on the free dofs, 0 elsewhere; y = 0 (y may be v's memory)
+__global__ void k_masked_copy(int64_t n, const uint8_t* free_dof, const double* v, double* x, double* y) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    x[i] = free_dof[i] ? v[i] : 0.0;
+    y[i] = 0.0;
+  }
+}
+
 __global__ void k_set_dirichlet(int64_t n, const uint8_t* free_dof, const double* ubc, double* x) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     if (!free_dof[i]) x[i] = ubc[i];
@@ -2862,9 +2870,13 @@ int solve(Context& c, double* u_user, int u_dev, nls_report* rep) {
 int eval_F(Context& c, const double* u, double* F, int is_dev, double load) {
   Dev& D = *c.dev;
   try {
-    CK(cudaMemcpyAsync(D.x, u, sizeof(double) * c.N, is_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, D.s));
-    global_residual(c, D.x, D.F, load);
-    CK(cudaMemcpyAsync(F, D.F, sizeof(double) * c.N, is_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, D.s));
+    if (is_dev) {  // read and written in place: the element pass has read u before F is written
+      global_residual(c, u, F, load);
+    } else {
+      CK(cudaMemcpyAsync(D.x, u, sizeof(double) * c.N, cudaMemcpyHostToDevice, D.s));
+      global_residual(c, D.x, D.F, load);
+      CK(cudaMemcpyAsync(F, D.F, sizeof(double) * c.N, cudaMemcpyDeviceToHost, D.s));
+    }
     sync(D);
   } catch (const std::exception& ex) {
     c.last_error = ex.what();
@@ -2903,12 +2915,11 @@ int apply_tangent(Context& c, const double* v, double* y, int is_dev) {
   }
   D.prof = c.opt.profile_kernels != 0;
   try {
-    CK(cudaMemcpyAsync(D.t1, v, sizeof(double) * c.N, is_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, D.s));
-    LAUNCH(D, k_mask, grid_for(c.N), 256, 0, c.N, D.free_dof, D.t1);
-    CK(cudaMemcpyAsync(D.x, D.t1, sizeof(double) * c.N, cudaMemcpyDeviceToDevice, D.s));
-    CK(cudaMemsetAsync(D.gx, 0, sizeof(double) * c.N, D.s));
-    tangent(c, D.x, D.gx);
-    CK(cudaMemcpyAsync(y, D.gx, sizeof(double) * c.N, is_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, D.s));
+    if (!is_dev) CK(cudaMemcpyAsync(D.t1, v, sizeof(double) * c.N, cudaMemcpyHostToDevice, D.s));
+    double* out = is_dev ? y : D.gx;
+    LAUNCH(D, k_masked_copy, grid_for(c.N), 256, 0, c.N, D.free_dof, is_dev ? v : D.t1, D.x, out);
+    tangent(c, D.x, out);
+    if (!is_dev) CK(cudaMemcpyAsync(y, D.gx, sizeof(double) * c.N, cudaMemcpyDeviceToHost, D.s));
     sync(D);
     check_local_waits(D);
   } catch (const DeviceTimeout& ex) {

@@ -345,7 +345,7 @@ class Solver:
         return out
 
     def eval_F(self, u, load: float = 1.0):
-        F = np.zeros_like(u) if isinstance(u, np.ndarray) else u.new_zeros(u.shape)
+        F = np.zeros_like(u) if isinstance(u, np.ndarray) else u.new_empty(u.shape)  # every entry is written
         self._check(self.lib.nls_eval_F(self.h, _ptr(u), _ptr(F), _is_device(u), load), "nls_eval_F")
         return F
 
@@ -358,7 +358,7 @@ class Solver:
         return Fx, its, st
 
     def apply_tangent(self, v):
-        y = np.zeros_like(v) if isinstance(v, np.ndarray) else v.new_zeros(v.shape)
+        y = np.zeros_like(v) if isinstance(v, np.ndarray) else v.new_empty(v.shape)  # every entry is written
         self._check(self.lib.nls_apply_tangent(self.h, _ptr(v), _ptr(y), _is_device(v)), "nls_apply_tangent")
         return y
 
