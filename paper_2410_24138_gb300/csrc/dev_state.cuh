@@ -125,6 +125,7 @@ struct Dev {
   double *c = nullptr, *ct = nullptr, *dc = nullptr, *g = nullptr, *gt = nullptr, *cres = nullptr, *tg = nullptr;
   void* cy = nullptr;
   double *V = nullptr, *partial = nullptr, *scal = nullptr, *coef = nullptr;
+  unsigned* ticket = nullptr;  // CTAs done in the tiled vector kernels (0 between launches)
   // GMRES least-squares state on the device: R (m x m), rotations, rotated right-hand side, state
   double *gR = nullptr, *gcs = nullptr, *gsn = nullptr, *gg = nullptr;
   GmresState* gst = nullptr;
