@@ -107,22 +107,6 @@ struct SmemPlan {
   size_t xt, r, rt, s, red, yv, win, rp, flag, total;
 };
 
-template <typename FT>
-__host__ __device__ inline SmemPlan smem_plan(int max_n, int max_nt) {
-  SmemPlan p;
-  size_t o = 0;
-  p.xt = o; o += sizeof(double) * max_nt;
-  p.r = o; o += sizeof(double) * max_n;
-  p.rt = o; o += sizeof(double) * max_n;
-  p.s = o; o += sizeof(double) * max_n;
-  p.red = o; o += sizeof(double) * 40;
-  p.yv = o; o += align_up(sizeof(FT) * max_n, 16);
-  p.win = p.rp = o;
-  p.flag = o; o += 16;
-  p.total = o;
-  return p;
-}
-
 // Shared memory of the batched local kernels.  Only what the inner loops hit per entry stays in
 // shared memory -- the table state (gathered by every element), the residual being assembled,
 // the band-LU window and the solve vector (which lives in the window once the factors are
@@ -736,11 +720,16 @@ __global__ void __launch_bounds__(256) k_harmonic(LocalArgs A) {
   }
 }
 
+// Rows of Phi_j and K^(j) Phi_j that the Galerkin kernel keeps in shared memory at a time.
+constexpr int kGalRows = 32;
+size_t galerkin_smem(int max_nt, int max_nc) {
+  return sizeof(double) * std::max((size_t)max_nt, (size_t)2 * kGalRows * max_nc);
+}
+
 template <int LAW>
 __global__ void __launch_bounds__(256, 2) k_galerkin(LocalArgs A) {
   extern __shared__ __align__(128) unsigned char smem[];
-  const SmemPlan P = smem_plan<double>(A.max_n, A.max_nt);
-  double* xt = (double*)(smem + P.xt);
+  double* xt = (double*)smem;
   const int j = blockIdx.x, tid = threadIdx.x, nd = A.ndof;
   const SubMeta m = A.meta[j];
   const int nc = A.cj_ptr[j + 1] - A.cj_ptr[j];
@@ -761,15 +750,42 @@ __global__ void __launch_bounds__(256, 2) k_galerkin(LocalArgs A) {
     Y[idx] = acc;
   }
   __syncthreads();
-  // block = Phi_j^T Y, one warp per entry, fixed-order lane sums
-  const int lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+  // block = Phi_j^T Y: rows of Phi and Y through shared memory, kGalRows at a time, one thread per entry
+  // (a warp per entry read both arrays 8 bytes at a time, nc entries apart).  Eq. 2's tangent is
+  // symmetric: the entries c <= d are formed, and mirrored.
+  double* ps = xt;  // the table vector has been used; kGalRows x nc of Phi, then of Y
+  double* ys = ps + kGalRows * nc;
   double* blk = A.blk + A.blk_off[j];
-  for (int e = wid; e < nc * nc; e += nw) {
-    const int c = e / nc, d = e % nc;
+  const bool sym = LAW == NLS_LAW_NEOHOOKE;
+  const int pairs = sym ? nc * (nc + 1) / 2 : nc * nc;
+  for (int e0 = 0; e0 < pairs; e0 += blockDim.x) {
+    const int e = e0 + tid;
+    int c = 0, d = 0;
+    if (sym) {  // e-th pair of the rows 0 .. c of the lower triangle
+      c = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+      while ((c + 1) * (c + 2) / 2 <= e) ++c;
+      while (c * (c + 1) / 2 > e) --c;
+      d = e - c * (c + 1) / 2;
+    } else {
+      c = e / nc;
+      d = e % nc;
+    }
     double acc = 0.0;
-    for (int t = lane; t < m.nt; t += 32) acc += phi[(int64_t)t * nc + c] * Y[(int64_t)t * nc + d];
-    acc = dev::warp_sum(acc);
-    if (lane == 0) blk[e] = acc;
+    for (int t0 = 0; t0 < m.nt; t0 += kGalRows) {
+      const int rows = min(kGalRows, m.nt - t0);
+      __syncthreads();
+      for (int q = tid; q < rows * nc; q += blockDim.x) {
+        ps[q] = phi[(int64_t)t0 * nc + q];
+        ys[q] = Y[(int64_t)t0 * nc + q];
+      }
+      __syncthreads();
+      if (e < pairs)
+        for (int t = 0; t < rows; ++t) acc += ps[t * nc + d] * ys[t * nc + c];
+    }
+    if (e < pairs) {
+      if (sym) blk[c * nc + d] = blk[d * nc + c] = acc;
+      else blk[d * nc + c] = acc;
+    }
   }
 }
 
@@ -1951,7 +1967,7 @@ void coarse_assemble_launch(Context& c, const double* x) {
   LocalArgs A = coarse_args(c);
   A.x = x;
   const int T = 256;
-  const size_t sm = smem_plan<double>(c.nov.max_n, c.nov.max_nt).total;
+  const size_t sm = galerkin_smem(c.nov.max_nt, c.cs.max_nc);
   if (c.law == NLS_LAW_DIFFUSION) LAUNCH(D, (k_galerkin<NLS_LAW_DIFFUSION>), c.nov.count, T, sm, A);
   else LAUNCH(D, (k_galerkin<NLS_LAW_NEOHOOKE>), c.nov.count, T, sm, A);
   const int64_t ne = (int64_t)c.cs.N0 * (2 * c.cs.b0 + 1);
@@ -2570,16 +2586,12 @@ FxInfo evaluate_Fx(Context& c, const double* u, double load, double* t_inner, do
   }
   sync(D);
   auto t1 = std::chrono::steady_clock::now();
-  // The tangent phase's coarse work depends on u_0 only: it goes on a second stream of the
-  // highest priority, issued before the batched local solves, so that it runs beside them.  The
-  // persistent local Newton grid fills every SM, so how it shares them depends on its occupancy:
-  // - several CTAs per SM: DF(u_0) and A_0(u_0) (many CTAs) go first on this stream, and the
-  //   single-CTA factorization of A_0 is dispatched together with the local solves, beside
-  //   some of their CTAs (the kernel pulls subdomains from a work counter, so a CTA of it that
-  //   starts late only takes fewer of them);
-  // - one CTA per SM (none can share an SM with the factorization): the whole chain goes on
-  //   the second stream, its assembly overlapping the start of the local solves, and the local
-  //   Newton grid leaves one SM to the factorization.
+  // The tangent phase's coarse work depends on u_0 only.  DF(u_0) and A_0(u_0) (many CTAs, FP64) go
+  // first on this stream; the single-CTA factorization of A_0 and the explicit inverse go on a second
+  // stream of the highest priority, beside the batched local solves, whose persistent grid leaves them
+  // one SM where it holds one CTA per SM (it pulls subdomains from a work counter: a CTA less, or one
+  // that starts late, only takes fewer of them).  Beside a local grid that fills the registers of every
+  // SM the assembly itself starved: 4.8 instead of 1.2 ms a launch for Eq. 2's Galerkin blocks (384^2 cells).
   // The tiled factorization spreads every step over many CTAs: it cannot live in the corner of the
   // machine the local grid leaves, so it runs alone on the main stream, before the local solves.
   const bool two_level = cp != NLS_COUPLING_ONE;
@@ -2589,7 +2601,7 @@ FxInfo evaluate_Fx(Context& c, const double* u, double load, double* t_inner, do
     tangent_coarse_assemble(c);
     tangent_coarse_factor(c);
   } else if (two_level) {
-    if (!spare_sm) tangent_coarse_assemble(c);
+    tangent_coarse_assemble(c);
     if (!D.s2) {
       int least = 0, greatest = 0;
       CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
@@ -2601,7 +2613,6 @@ FxInfo evaluate_Fx(Context& c, const double* u, double load, double* t_inner, do
     CK(cudaStreamWaitEvent(D.s2, D.ev_u0, 0));
     std::swap(D.s, D.s2);
     try {
-      if (spare_sm) tangent_coarse_assemble(c);
       tangent_coarse_factor(c);
     } catch (...) {
       std::swap(D.s, D.s2);
