@@ -100,7 +100,8 @@ struct Dev {
       }
   }
   // mesh
-  int32_t *conn = nullptr, *g_elem = nullptr, *g_rowptr = nullptr, *g_col = nullptr, *g_epos = nullptr;
+  int32_t *conn = nullptr, *g_elem = nullptr, *g_col = nullptr, *g_epos = nullptr;
+  int64_t *g_slice = nullptr, *p0_slice = nullptr;
   int64_t* star_ptr = nullptr;  // node stars (ascending element ids) for the global residual's node sums
   int32_t* star_ref = nullptr;  // e nen + a per star entry
   double* Re = nullptr;         // element residuals [e][a][dof]
@@ -109,7 +110,7 @@ struct Dev {
   uint8_t* free_dof = nullptr;
   DeviceLocalSet ov, nov;
   // coarse
-  int32_t *p0_rowptr = nullptr, *p0_col = nullptr, *p0t_rowptr = nullptr, *p0t_col = nullptr, *p0t_src = nullptr;
+  int32_t *p0_col = nullptr, *p0t_rowptr = nullptr, *p0t_col = nullptr, *p0t_src = nullptr;
   int64_t* p0_src = nullptr;
   double *p0_val = nullptr, *p0t_val = nullptr, *phi = nullptr, *Y = nullptr, *blk = nullptr, *A0 = nullptr;
   int64_t *phi_off = nullptr, *blk_off = nullptr, *a0_src = nullptr;

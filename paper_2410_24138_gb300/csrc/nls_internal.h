@@ -77,9 +77,10 @@ struct Coarse {
   int N0 = 0;                      // coarse dofs
   int b0 = 0;                      // half bandwidth of A_0
   std::vector<int32_t> first_node; // smallest global node id per coarse node
-  // P_0 as CSR over global dofs (values filled on the device)
-  std::vector<int32_t> p0_rowptr, p0_col;
-  std::vector<int64_t> p0_src;     // index into the concatenated Phi blocks
+  // P_0 over global dofs in slices of 32 rows (as Context::g_slice; values filled on the device)
+  std::vector<int64_t> p0_slice;
+  std::vector<int32_t> p0_col;
+  std::vector<int64_t> p0_src;     // index into the concatenated Phi blocks, -1 for padding
   std::vector<int32_t> p0t_rowptr, p0t_col;  // transpose: rows = coarse dofs, col = global dof
   std::vector<int32_t> p0t_src;    // index into p0 values
   // per non-overlapping subdomain j: columns C_j and dense Phi_j [nt_j x nc_j] (row-major)
@@ -128,7 +129,10 @@ struct Context {
   LocalSet nov;     // non-overlapping subdomains (coarse space)
   Coarse cs;
   std::vector<int32_t> g_color_ptr, g_elem;  // global element colouring
-  std::vector<int32_t> g_rowptr, g_col;      // global CSR pattern
+  // global matrix DF in slices of 32 rows: entry k of row i at g_slice[i / 32] + 32 k + i % 32; shorter
+  // rows (and rows past N) are padded with column 0 and a value that stays zero
+  std::vector<int64_t> g_slice;
+  std::vector<int32_t> g_col;
   std::vector<int32_t> g_epos;               // [elem][(nen*ndof)^2], element order = conn order
   std::vector<double> geom;                  // per element geometry
   int geom_stride = 0;

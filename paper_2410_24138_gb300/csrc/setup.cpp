@@ -304,7 +304,33 @@ void build_local_set(Context& c, LocalSet& s, int layers, bool neumann_rows, boo
 
 namespace {
 
-// ---- global structures: colouring, CSR pattern, geometry, external load -------------------
+// ---- global structures: colouring, matrix pattern, geometry, external load -------------------
+
+// CSR rows into slices of 32 rows (Context::g_slice): `col` is replaced, padded by `fill(row)`, and
+// at[k] is the new position of entry k.
+template <typename Fill>
+void slice_matrix(const std::vector<int32_t>& rowptr, std::vector<int32_t>& col, std::vector<int64_t>& slice,
+                  std::vector<int64_t>& at, Fill&& fill) {
+  const int64_t n = (int64_t)rowptr.size() - 1, ns = (n + 31) / 32;
+  slice.assign(ns + 1, 0);
+  for (int64_t q = 0; q < ns; ++q) {
+    int32_t width = 0;
+    for (int64_t i = 32 * q; i < std::min(n, 32 * q + 32); ++i) width = std::max(width, rowptr[i + 1] - rowptr[i]);
+    slice[q + 1] = slice[q] + 32 * (int64_t)width;
+  }
+  std::vector<int32_t> padded(slice[ns]);
+  at.resize(col.size());
+  for (int64_t i = 0; i < 32 * ns; ++i) {
+    const int64_t first = slice[i >> 5] + (i & 31), end = slice[(i >> 5) + 1];
+    const int32_t k0 = i < n ? rowptr[i] : 0, len = i < n ? rowptr[i + 1] - k0 : 0;
+    int32_t k = 0;
+    for (int64_t p = first; p < end; p += 32, ++k) {
+      padded[p] = k < len ? col[k0 + k] : fill(i);
+      if (k < len) at[k0 + k] = p;
+    }
+  }
+  col.swap(padded);
+}
 
 void build_global(Context& c) {
   const int nen = c.nen, nd = c.ndof, ned = nen * nd;
@@ -330,8 +356,8 @@ void build_global(Context& c) {
     std::vector<int32_t> fill(c.g_color_ptr.begin(), c.g_color_ptr.end() - 1);
     for (int64_t e = 0; e < c.n_elems; ++e) c.g_elem[fill[color[e]]++] = (int32_t)e;
   }
-  // global CSR pattern of DF (all dofs)
-  c.g_rowptr.assign(c.N + 1, 0);
+  // global pattern of DF (all dofs), first as CSR
+  std::vector<int32_t> rowptr(c.N + 1, 0);
   c.g_col.clear();
   std::vector<int32_t> nb;
   for (int64_t v = 0; v < c.n_nodes; ++v) {
@@ -343,7 +369,7 @@ void build_global(Context& c) {
     for (int da = 0; da < nd; ++da) {
       for (int32_t s : nb)
         for (int db = 0; db < nd; ++db) c.g_col.push_back(s * nd + db);
-      c.g_rowptr[v * nd + da + 1] = (int32_t)c.g_col.size();
+      rowptr[v * nd + da + 1] = (int32_t)c.g_col.size();
     }
   }
   if (c.g_col.size() > (size_t)INT32_MAX) throw std::runtime_error("global Jacobian too large for 32-bit positions");
@@ -352,8 +378,8 @@ void build_global(Context& c) {
     for (int a = 0; a < nen; ++a)
       for (int da = 0; da < nd; ++da) {
         int64_t row = (int64_t)c.conn[e * nen + a] * nd + da;
-        const int32_t* b0 = c.g_col.data() + c.g_rowptr[row];
-        const int32_t* b1 = c.g_col.data() + c.g_rowptr[row + 1];
+        const int32_t* b0 = c.g_col.data() + rowptr[row];
+        const int32_t* b1 = c.g_col.data() + rowptr[row + 1];
         for (int bb = 0; bb < nen; ++bb)
           for (int db = 0; db < nd; ++db) {
             int32_t col = c.conn[e * nen + bb] * nd + db;
@@ -361,6 +387,11 @@ void build_global(Context& c) {
                 (int32_t)(std::lower_bound(b0, b1, col) - c.g_col.data());
           }
       }
+  std::vector<int64_t> at;
+  slice_matrix(rowptr, c.g_col, c.g_slice, at, [&](int64_t i) { return (int32_t)std::min<int64_t>(i, c.N - 1); });
+  // positions are kept as 32-bit words, read as unsigned: room for the padding
+  if (c.g_col.size() > (size_t)UINT32_MAX) throw std::runtime_error("global Jacobian too large for 32-bit positions");
+  for (auto& e : c.g_epos) e = (int32_t)(uint32_t)at[e];
   // element geometry
   if (c.elem_type == NLS_P1_TRI) {
     c.geom_stride = 8;  // G (3 x 2), area, pad
@@ -608,7 +639,7 @@ void build_coarse(Context& c) {
       }
     }
   }
-  cs.p0_rowptr.assign(c.N + 1, 0);
+  std::vector<int32_t> rowptr(c.N + 1, 0);
   for (int64_t v = 0; v < c.n_nodes; ++v)
     for (int d = 0; d < nd; ++d) {
       int64_t g = v * nd + d;
@@ -632,9 +663,9 @@ void build_coarse(Context& c) {
           }
         }
       }
-      cs.p0_rowptr[g + 1] = (int32_t)cs.p0_col.size();
+      rowptr[g + 1] = (int32_t)cs.p0_col.size();
     }
-  // transpose
+  // transpose (CSR), with the positions of the sliced P_0
   std::vector<int32_t> cnt(cs.N0 + 1, 0);
   for (int32_t col : cs.p0_col) cnt[col + 1] += 1;
   for (int k = 0; k < cs.N0; ++k) cnt[k + 1] += cnt[k];
@@ -642,12 +673,18 @@ void build_coarse(Context& c) {
   cs.p0t_col.assign(cs.p0_col.size(), 0);
   cs.p0t_src.assign(cs.p0_col.size(), 0);
   {
+    const std::vector<int32_t> csr_col = cs.p0_col;
+    const std::vector<int64_t> csr_src = cs.p0_src;
+    std::vector<int64_t> at;
+    slice_matrix(rowptr, cs.p0_col, cs.p0_slice, at, [](int64_t) { return 0; });
+    cs.p0_src.assign(cs.p0_col.size(), -1);
     std::vector<int32_t> fill(cnt.begin(), cnt.end() - 1);
     for (int64_t g = 0; g < c.N; ++g)
-      for (int32_t k = cs.p0_rowptr[g]; k < cs.p0_rowptr[g + 1]; ++k) {
-        int32_t pos = fill[cs.p0_col[k]]++;
+      for (int32_t k = rowptr[g]; k < rowptr[g + 1]; ++k) {
+        cs.p0_src[at[k]] = csr_src[k];
+        int32_t pos = fill[csr_col[k]]++;
         cs.p0t_col[pos] = (int32_t)g;
-        cs.p0t_src[pos] = k;
+        cs.p0t_src[pos] = (int32_t)at[k];
       }
   }
   // A_0 band structure and the per-subdomain block contributions
