@@ -12,6 +12,7 @@
 #include <numeric>
 #include <set>
 #include <stdexcept>
+#include <system_error>
 #include <thread>
 
 #include "nls_internal.h"
@@ -306,30 +307,39 @@ namespace {
 
 // ---- global structures: colouring, matrix pattern, geometry, external load -------------------
 
-// CSR rows into slices of 32 rows (Context::g_slice): `col` is replaced, padded by `fill(row)`, and
-// at[k] is the new position of entry k.
-template <typename Fill>
-void slice_matrix(const std::vector<int32_t>& rowptr, std::vector<int32_t>& col, std::vector<int64_t>& slice,
-                  std::vector<int64_t>& at, Fill&& fill) {
+// f(begin, end) over [0, n) in ranges, one per host thread (f does not throw); a range whose thread
+// cannot be started runs here.
+template <typename F>
+void in_ranges(int64_t n, F&& f) {
+  const int64_t parts = std::max<int64_t>(1, std::min<int64_t>(std::min(16u, std::thread::hardware_concurrency()), n / 4096));
+  std::vector<std::thread> pool;
+  pool.reserve(parts);
+  for (int64_t t = 1; t < parts; ++t) {
+    const int64_t b = n * t / parts, e = n * (t + 1) / parts;
+    try {
+      pool.emplace_back([&f, b, e] { f(b, e); });
+    } catch (const std::system_error&) {
+      f(b, e);
+    }
+  }
+  f((int64_t)0, n / parts);
+  for (auto& th : pool) th.join();
+}
+
+// First positions of the slices of 32 rows of a CSR matrix (Context::g_slice): entry k of row i moves
+// to slice[i / 32] + 32 k + i % 32.
+std::vector<int64_t> slice_starts(const std::vector<int32_t>& rowptr) {
   const int64_t n = (int64_t)rowptr.size() - 1, ns = (n + 31) / 32;
-  slice.assign(ns + 1, 0);
+  std::vector<int64_t> slice(ns + 1, 0);
   for (int64_t q = 0; q < ns; ++q) {
     int32_t width = 0;
     for (int64_t i = 32 * q; i < std::min(n, 32 * q + 32); ++i) width = std::max(width, rowptr[i + 1] - rowptr[i]);
     slice[q + 1] = slice[q] + 32 * (int64_t)width;
   }
-  std::vector<int32_t> padded(slice[ns]);
-  at.resize(col.size());
-  for (int64_t i = 0; i < 32 * ns; ++i) {
-    const int64_t first = slice[i >> 5] + (i & 31), end = slice[(i >> 5) + 1];
-    const int32_t k0 = i < n ? rowptr[i] : 0, len = i < n ? rowptr[i + 1] - k0 : 0;
-    int32_t k = 0;
-    for (int64_t p = first; p < end; p += 32, ++k) {
-      padded[p] = k < len ? col[k0 + k] : fill(i);
-      if (k < len) at[k0 + k] = p;
-    }
-  }
-  col.swap(padded);
+  return slice;
+}
+inline int64_t sliced(const std::vector<int64_t>& slice, int64_t row, int64_t k) {
+  return slice[row >> 5] + 32 * k + (row & 31);
 }
 
 void build_global(Context& c) {
@@ -373,25 +383,37 @@ void build_global(Context& c) {
     }
   }
   if (c.g_col.size() > (size_t)INT32_MAX) throw std::runtime_error("global Jacobian too large for 32-bit positions");
-  c.g_epos.assign((size_t)c.n_elems * ned * ned, 0);
-  for (int64_t e = 0; e < c.n_elems; ++e)
-    for (int a = 0; a < nen; ++a)
-      for (int da = 0; da < nd; ++da) {
-        int64_t row = (int64_t)c.conn[e * nen + a] * nd + da;
-        const int32_t* b0 = c.g_col.data() + rowptr[row];
-        const int32_t* b1 = c.g_col.data() + rowptr[row + 1];
-        for (int bb = 0; bb < nen; ++bb)
-          for (int db = 0; db < nd; ++db) {
-            int32_t col = c.conn[e * nen + bb] * nd + db;
-            c.g_epos[(size_t)e * ned * ned + (a * nd + da) * ned + bb * nd + db] =
-                (int32_t)(std::lower_bound(b0, b1, col) - c.g_col.data());
-          }
-      }
-  std::vector<int64_t> at;
-  slice_matrix(rowptr, c.g_col, c.g_slice, at, [&](int64_t i) { return (int32_t)std::min<int64_t>(i, c.N - 1); });
+  c.g_slice = slice_starts(rowptr);
   // positions are kept as 32-bit words, read as unsigned: room for the padding
-  if (c.g_col.size() > (size_t)UINT32_MAX) throw std::runtime_error("global Jacobian too large for 32-bit positions");
-  for (auto& e : c.g_epos) e = (int32_t)(uint32_t)at[e];
+  if (c.g_slice.back() > (int64_t)UINT32_MAX) throw std::runtime_error("global Jacobian too large for 32-bit positions");
+  c.g_epos.assign((size_t)c.n_elems * ned * ned, 0);
+  in_ranges(c.n_elems, [&](int64_t e0, int64_t e1) {
+    for (int64_t e = e0; e < e1; ++e)
+      for (int a = 0; a < nen; ++a)
+        for (int da = 0; da < nd; ++da) {
+          int64_t row = (int64_t)c.conn[e * nen + a] * nd + da;
+          const int32_t* b0 = c.g_col.data() + rowptr[row];
+          const int32_t* b1 = c.g_col.data() + rowptr[row + 1];
+          for (int bb = 0; bb < nen; ++bb)
+            for (int db = 0; db < nd; ++db) {
+              int32_t col = c.conn[e * nen + bb] * nd + db;
+              c.g_epos[(size_t)e * ned * ned + (a * nd + da) * ned + bb * nd + db] =
+                  (int32_t)(uint32_t)sliced(c.g_slice, row, std::lower_bound(b0, b1, col) - b0);
+            }
+        }
+  });
+  {
+    std::vector<int32_t> padded(c.g_slice.back());
+    in_ranges((int64_t)c.g_slice.size() - 1, [&](int64_t q0, int64_t q1) {
+      for (int64_t q = q0; q < q1; ++q)
+        for (int64_t k = 0; 32 * k < c.g_slice[q + 1] - c.g_slice[q]; ++k)
+          for (int64_t i = 32 * q; i < 32 * q + 32; ++i) {
+            const bool in = i < c.N && k < rowptr[i + 1] - rowptr[i];
+            padded[sliced(c.g_slice, i, k)] = in ? c.g_col[rowptr[i] + k] : (int32_t)std::min<int64_t>(i, c.N - 1);
+          }
+    });
+    c.g_col.swap(padded);
+  }
   // element geometry
   if (c.elem_type == NLS_P1_TRI) {
     c.geom_stride = 8;  // G (3 x 2), area, pad
@@ -673,19 +695,21 @@ void build_coarse(Context& c) {
   cs.p0t_col.assign(cs.p0_col.size(), 0);
   cs.p0t_src.assign(cs.p0_col.size(), 0);
   {
-    const std::vector<int32_t> csr_col = cs.p0_col;
-    const std::vector<int64_t> csr_src = cs.p0_src;
-    std::vector<int64_t> at;
-    slice_matrix(rowptr, cs.p0_col, cs.p0_slice, at, [](int64_t) { return 0; });
-    cs.p0_src.assign(cs.p0_col.size(), -1);
+    cs.p0_slice = slice_starts(rowptr);
+    std::vector<int32_t> col(cs.p0_slice.back(), 0);
+    std::vector<int64_t> src(cs.p0_slice.back(), -1);
     std::vector<int32_t> fill(cnt.begin(), cnt.end() - 1);
     for (int64_t g = 0; g < c.N; ++g)
       for (int32_t k = rowptr[g]; k < rowptr[g + 1]; ++k) {
-        cs.p0_src[at[k]] = csr_src[k];
-        int32_t pos = fill[csr_col[k]]++;
+        const int64_t at = sliced(cs.p0_slice, g, k - rowptr[g]);
+        col[at] = cs.p0_col[k];
+        src[at] = cs.p0_src[k];
+        int32_t pos = fill[cs.p0_col[k]]++;
         cs.p0t_col[pos] = (int32_t)g;
-        cs.p0t_src[pos] = (int32_t)at[k];
+        cs.p0t_src[pos] = (int32_t)at;
       }
+    cs.p0_col.swap(col);
+    cs.p0_src.swap(src);
   }
   // A_0 band structure and the per-subdomain block contributions
   int b0 = 0;
