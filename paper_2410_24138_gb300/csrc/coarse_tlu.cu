@@ -7,8 +7,8 @@
 // is cut into square tiles and factored without pivoting, right-looking, one tile column per
 // step, across many CTAs:
 //
-//   step k:  A_kk = L_kk U_kk                      (every panel CTA, in registers, blocked by
-//                                                   32-column groups)
+//   step k:  A_kk = L_kk U_kk                      (every panel CTA, in shared memory, blocked by 16
+//                                                   or 8 columns)
 //            L_ik = A_ik U_kk^-1,  U_kj = L_kk^-1 A_kj   (i, j = k+1 .. k+TB; row slabs per CTA)
 //            A_ij -= L_ik U_kj                     (i, j = k+1 .. k+TB; one CTA per tile)
 //
@@ -109,180 +109,216 @@ __global__ void k_tlu_init(int N0, int b0, int NT, int TB, const double* __restr
 // stores it in DG[k] and flags a zero or non-finite pivot.  Panel p < TB is the L tile
 // (k+1+p, k): X := X U_kk^-1 on rows of the tile; panel p >= TB is the U tile (k, k+1+p-TB),
 // stored transposed: X := X L_kk^-T on rows of the stored transpose.  Both are X := X M^-1 with
-// M upper triangular.  The diagonal tile's LU and the slab's solve are both blocked by 32-column
-// groups: one barrier per column inside a group, a rank-32 update of the rest after it.  With LT
-// given, an L tile is also written transposed there (the B operand of M_tk for the solves).
-template <typename FT>
-__device__ inline FT rcp(FT x) {
-  if constexpr (sizeof(FT) == 4) return __frcp_rn(x);
-  else return (FT)1 / x;
+// M upper triangular.  With LT given, an L tile is also written transposed there (the B operand of
+// M_tk for the solves).
+//
+// What bounds it is the chain of TS pivots and then TS columns.  One step per pivot with a CTA barrier
+// took 860 cycles (108 us per launch at TS = 128, b_0 = 197; now 35 us).  Both are blocked by NB = 16
+// (FP32) or 8 (FP64): warp 0 factors a diagonal block in registers, one thread per row or column
+// finishes the block's L rows and U columns (the slab's rows), and all warps take the NB rank-1 updates
+// of the rest with one load and one store per entry.  Every entry keeps the order of its updates, so
+// the FP32 factors are the same bits.
+template <typename FT, int TS>
+constexpr int panel_ld() {  // row stride in shared memory: whole 16-byte groups, rows on different banks
+  return TS + dev::LuTile<FT>::G;
+}
+
+// O -= L U on a 2D range of NB x NB blocks: rows r0 + NB i (i < nr), columns c0 + NB j (j < nc) of O (row
+// stride LD), L the rows' NB multipliers at column k0 of `Ls`, U the NB rows k0 .. of `Us`.  A warp takes
+// one block row by two block columns, a lane G x G entries.
+template <typename FT, int LD>
+__device__ __forceinline__ void panel_update(FT* O, const FT* Ls, const FT* Us, int k0, int r0, int nr, int c0, int nc) {
+  constexpr int G = dev::LuTile<FT>::G, NB = dev::LuTile<FT>::NB;
+  using Vec = dev::LuVec<FT>;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, pairs = (nc + 1) / 2;
+  for (int u = wid; u < nr * pairs; u += nw) {
+    const int j = 2 * (u % pairs) + ((lane & 7) >> 2);
+    if (j >= nc) continue;
+    const int r = r0 + NB * (u / pairs) + (lane >> 3) * G, c = c0 + NB * j + (lane & 3) * G;
+    Vec acc[G];
+#pragma unroll
+    for (int i = 0; i < G; ++i) acc[i] = *(const Vec*)(O + (r + i) * LD + c);
+#pragma unroll
+    for (int k = 0; k < NB; k += G) {
+      Vec l[G], v[G];
+#pragma unroll
+      for (int i = 0; i < G; ++i) l[i] = *(const Vec*)(Ls + (r + i) * LD + k0 + k);
+#pragma unroll
+      for (int i = 0; i < G; ++i) v[i] = *(const Vec*)(Us + (k0 + k + i) * LD + c);
+#pragma unroll
+      for (int q = 0; q < G; ++q)
+#pragma unroll
+        for (int i = 0; i < G; ++i)
+#pragma unroll
+          for (int e = 0; e < G; ++e) acc[i].v[e] -= l[i].v[q] * v[q].v[e];
+    }
+#pragma unroll
+    for (int i = 0; i < G; ++i) *(Vec*)(O + (r + i) * LD + c) = acc[i];
+  }
+}
+
+// One row of NB values times the inverse of the upper triangular block M (row stride LD, reciprocal
+// diagonal rd, or 1 where rd is null): x_t = a_t rd_t, a_j -= x_t M_tj for j > t.
+template <typename FT, int LD>
+__device__ __forceinline__ void panel_row(FT* row, const FT* M, const FT* rd) {
+  constexpr int G = dev::LuTile<FT>::G, NB = dev::LuTile<FT>::NB;
+  using Vec = dev::LuVec<FT>;
+  FT a[NB];
+#pragma unroll
+  for (int g = 0; g < NB; g += G) {
+    const Vec v = *(const Vec*)(row + g);
+#pragma unroll
+    for (int i = 0; i < G; ++i) a[g + i] = v.v[i];
+  }
+#pragma unroll
+  for (int k = 0; k < NB; ++k) {
+    if (rd) a[k] *= rd[k];
+#pragma unroll
+    for (int g = (k + 1) / G * G; g < NB; g += G) {
+      const Vec v = *(const Vec*)(M + k * LD + g);
+#pragma unroll
+      for (int i = 0; i < G; ++i)
+        if (g + i > k) a[g + i] -= a[k] * v.v[i];
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < NB; g += G) {
+    Vec v;
+#pragma unroll
+    for (int i = 0; i < G; ++i) v.v[i] = a[g + i];
+    *(Vec*)(row + g) = v;
+  }
 }
 
 template <typename FT, int TS, int NS>
 __global__ void __launch_bounds__(512) k_tlu_panel(int k, int NT, int TB, FT* __restrict__ T, FT* __restrict__ DG,
                                                    FT* __restrict__ LT, int32_t* status) {
-  // 512 threads as 16 x 32: thread (ty, tx) keeps the entries (ty + 16 a, tx + 32 b) of the tile
-  // in registers (RA x CB of them); one elimination step only passes the pivot row and column
-  // through shared memory (double-buffered by the step's parity: one barrier per step).
-  constexpr int SLAB = TS / NS, LD = TS + 1, RA = TS / 16, CB = TS / 32, SA = SLAB / 16;
-  static_assert(SLAB % 16 == 0 && TS % 32 == 0, "panel tiling");
+  constexpr int SLAB = TS / NS, LD = panel_ld<FT, TS>(), G = dev::LuTile<FT>::G, NB = dev::LuTile<FT>::NB;
+  constexpr int NK = TS / NB, C = NB * NB / 32, RV = TS / G;  // blocks; entries per lane of a block; groups per row
+  using Vec = dev::LuVec<FT>;
+  static_assert(TS % (2 * NB) == 0 && SLAB % NB == 0, "panel tiling");
   extern __shared__ __align__(16) unsigned char smem[];
-  FT* Dg = (FT*)smem;           // TS x LD: the factored diagonal tile (for the slab solve)
-  FT* rpiv = Dg + TS * LD;      // TS reciprocal pivots
-  FT* rowbuf = rpiv + TS;       // 2 x TS
-  FT* colbuf = rowbuf + 2 * TS; // 2 x TS
+  FT* Dg = (FT*)smem;        // TS x LD: the diagonal tile, then its factors
+  FT* Mb = Dg + TS * LD;     // TS x LD: M of the slab's solve (right of the diagonal)
+  FT* Xs = Mb + TS * LD;     // SLAB x LD: the slab
+  FT* rpiv = Xs + SLAB * LD;  // TS reciprocal pivots
+  FT* dt = rpiv + TS;        // NB x NB: transposed multipliers of the current block
   __shared__ int s_bad;
-  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
   const int p = blockIdx.x / NS, q = blockIdx.x % NS;
   const bool lower = p < TB;
   const int other = k + 1 + (lower ? p : p - TB);  // the panel's tile row (L) or column (U)
   const bool has_panel = other < NT;
   if (!has_panel && blockIdx.x != 0) return;
   const FT* Akk = T + tile_slot(k, k, TB) * TS * TS;
-  FT R[RA][CB];
-#pragma unroll
-  for (int a = 0; a < RA; ++a)
-#pragma unroll
-    for (int b = 0; b < CB; ++b) R[a][b] = Akk[(ty + 16 * a) * TS + tx + 32 * b];
+  FT* P = has_panel ? T + (lower ? tile_slot(other, k, TB) : tile_slot(k, other, TB)) * TS * TS + (int64_t)q * SLAB * TS
+                    : nullptr;
+  for (int e = tid; e < TS * RV; e += nt) *(Vec*)(Dg + e / RV * LD + e % RV * G) = *(const Vec*)(Akk + e * G);
+  if (has_panel)
+    for (int e = tid; e < SLAB * RV; e += nt) *(Vec*)(Xs + e / RV * LD + e % RV * G) = *(const Vec*)(P + e * G);
   if (tid == 0) s_bad = 0;
-  // Blocked right-looking LU over the 32-column panels j of the tile.  Row r = ty + 16 a is the
-  // same in a whole warp and column c = tx + 32 b is lane tx of column group b, so panel j is the
-  // register column R[.][j] and its 32 pivot rows are a = 2j, 2j + 1.  For each pivot t of the
-  // panel: rows below t update their panel column and, inside the panel's own 32 rows, also the
-  // columns right of the panel (which makes those rows U12 = L11^-1 A12); then the rows below the
-  // panel take the rank-32 product A22 -= L21 U12 at once, L21 from warp shuffles (row r's
-  // multipliers sit in the lanes of its warp) and U12 through shared memory.
-#pragma unroll
-  for (int j = 0; j < CB; ++j) {
-    for (int t = 32 * j; t < 32 * j + 32; ++t) {
-      FT* rb = rowbuf + (t & 1) * TS;
-      FT* cb = colbuf + (t & 1) * TS;
-#pragma unroll
-      for (int a = 0; a < RA; ++a)
-        if (ty + 16 * a == t) {
-#pragma unroll
-          for (int b = j; b < CB; ++b) rb[tx + 32 * b] = R[a][b];
-        }
-      if (tx == t - 32 * j) {
-#pragma unroll
-        for (int a = 0; a < RA; ++a) cb[ty + 16 * a] = R[a][j];
-      }
-      __syncthreads();
-      const FT piv = rb[t];
-      const FT rp = rcp<FT>(piv);
-      if (tid == 0) {
-        rpiv[t] = rp;
-        if (!(piv != (FT)0) || !isfinite((double)piv)) s_bad = 1;
-      }
-#pragma unroll
-      for (int a = 0; a < RA; ++a) {
-        const int r = ty + 16 * a;
-        if (r > t) {  // warp-uniform
-          const FT l = cb[r] * rp;
-          const int c = tx + 32 * j;
-          if (c > t) R[a][j] -= l * rb[c];
-          else if (c == t) R[a][j] = l;  // the multiplier of L
-          if (a == 2 * j || a == 2 * j + 1) {  // the panel's own rows: U12
-#pragma unroll
-            for (int b = j + 1; b < CB; ++b) R[a][b] -= l * rb[tx + 32 * b];
-          }
-        }
-      }
-    }
-    if (j + 1 < CB) {
-      // U12 (rows 32 j .. 32 j + 31, columns right of the panel) into shared memory (Dg serves as
-      // scratch until the end), then A22 -= L21 U12 on the rows below the panel
-#pragma unroll
-      for (int a = 2 * j; a < 2 * j + 2; ++a)
-#pragma unroll
-        for (int b = j + 1; b < CB; ++b) Dg[(ty + 16 * (a - 2 * j)) * LD + tx + 32 * b] = R[a][b];
-      __syncthreads();
-      for (int kk = 0; kk < 32; ++kk) {
-        FT l[RA];
-#pragma unroll
-        for (int a = 2 * j + 2; a < RA; ++a) l[a] = __shfl_sync(0xffffffffu, R[a][j], kk);
-#pragma unroll
-        for (int b = j + 1; b < CB; ++b) {
-          const FT u = Dg[kk * LD + tx + 32 * b];
-#pragma unroll
-          for (int a = 2 * j + 2; a < RA; ++a) R[a][b] -= l[a] * u;
-        }
-      }
-      __syncthreads();  // U12 read by every warp before the next panel's rows overwrite the scratch
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < RA; ++a)
-#pragma unroll
-    for (int b = 0; b < CB; ++b) Dg[(ty + 16 * a) * LD + tx + 32 * b] = R[a][b];
   __syncthreads();
+  for (int J = 0; J < NK; ++J) {
+    const int j0 = J * NB;
+    FT* D = Dg + j0 * LD + j0;
+    if (wid == 0) {
+      // the diagonal block: lane (r, h) holds row r, columns h C .. h C + C - 1
+      const int r = lane % NB, h = lane / NB;
+      FT a[C];
+#pragma unroll
+      for (int g = 0; g < C; g += G) {
+        const Vec v = *(const Vec*)(D + r * LD + h * C + g);
+#pragma unroll
+        for (int i = 0; i < G; ++i) a[g + i] = v.v[i];
+      }
+      bool bad = false;
+      dev::static_for<0, NB>([&](auto tc_) {
+        constexpr int t = decltype(tc_)::value, ht = t / C, kt = t % C, f0 = ht == NB / C - 1 ? kt + 1 : 0;
+        const FT piv = __shfl_sync(0xffffffffu, a[kt], t + NB * ht);
+        const FT x = __shfl_sync(0xffffffffu, a[kt], r + NB * ht);
+        FT u[C];
+#pragma unroll
+        for (int f = f0; f < C; ++f) u[f] = __shfl_sync(0xffffffffu, a[f], t + NB * h);
+        const FT rp = dev::recip<FT>(piv);
+        bad |= dev::bad_pivot(piv);
+        if (lane == t) rpiv[j0 + t] = rp;
+        const FT l = x * rp;
+#pragma unroll
+        for (int f = f0; f < C; ++f) {
+          const FT y = a[f] - l * u[f];
+          a[f] = (r > t && h * C + f > t) ? y : a[f];
+        }
+        if (h == ht) a[kt] = r > t ? l : a[kt];
+      });
+#pragma unroll
+      for (int g = 0; g < C; g += G) {
+        Vec v;
+#pragma unroll
+        for (int i = 0; i < G; ++i) v.v[i] = a[g + i];
+        *(Vec*)(D + r * LD + h * C + g) = v;
+      }
+#pragma unroll
+      for (int f = 0; f < C; ++f) dt[(h * C + f) * NB + r] = a[f];
+      if (bad && lane == 0) s_bad = 1;
+    }
+    __syncthreads();
+    const int rest = TS - j0 - NB, half = (rest + 31) & ~31;  // a warp takes rows or columns, not both
+    for (int e = tid; e < 2 * half; e += nt) {
+      const int i = e < half ? e : e - half;
+      if (i >= rest) continue;
+      const int x = j0 + NB + i;
+      if (e < half) {
+        panel_row<FT, LD>(Dg + x * LD + j0, D, rpiv + j0);
+      } else {
+        FT a[NB];
+#pragma unroll
+        for (int t = 0; t < NB; ++t) a[t] = Dg[(j0 + t) * LD + x];
+#pragma unroll
+        for (int t = 0; t < NB; ++t)
+#pragma unroll
+          for (int g = (t + 1) / G * G; g < NB; g += G) {
+            const Vec v = *(const Vec*)(dt + t * NB + g);
+#pragma unroll
+            for (int f = 0; f < G; ++f)
+              if (g + f > t) a[g + f] -= v.v[f] * a[t];
+          }
+#pragma unroll
+        for (int t = 1; t < NB; ++t) Dg[(j0 + t) * LD + x] = a[t];
+      }
+    }
+    __syncthreads();
+    panel_update<FT, LD>(Dg, Dg, Dg, j0, j0 + NB, NK - 1 - J, j0 + NB, NK - 1 - J);
+    __syncthreads();
+  }
   if (blockIdx.x == 0) {
     FT* out = DG + (int64_t)k * TS * TS;
-#pragma unroll
-    for (int a = 0; a < RA; ++a)
-#pragma unroll
-      for (int b = 0; b < CB; ++b) out[(ty + 16 * a) * TS + tx + 32 * b] = R[a][b];
+    for (int e = tid; e < TS * RV; e += nt) *(Vec*)(out + e * G) = *(const Vec*)(Dg + e / RV * LD + e % RV * G);
     if (tid == 0 && s_bad) atomicExch(status, (int32_t)ST_PIVOT);
   }
   if (!has_panel) return;
   // X := X M^-1 on the slab's rows, M = U_kk (lower panel) or L_kk^T (upper panel, unit diagonal)
-  FT* P = T + (lower ? tile_slot(other, k, TB) : tile_slot(k, other, TB)) * TS * TS + (int64_t)q * SLAB * TS;
-  FT X[SA][CB];
-  {
-#pragma unroll
-    for (int a = 0; a < SA; ++a)
-#pragma unroll
-      for (int b = 0; b < CB; ++b) X[a][b] = P[(ty + 16 * a) * TS + tx + 32 * b];
-    // blocked over the 32-column groups j: column by column inside the group (one barrier per
-    // column, only the group's register column X[.][j] changes), then the columns right of the
-    // group take X[:, right] -= X[:, group] M[group, right] at once (the row's group values from
-    // warp shuffles, M from the factored tile)
-#pragma unroll
-    for (int j = 0; j < CB; ++j) {
-      for (int t = 32 * j; t < 32 * j + 32; ++t) {
-        FT* cb = colbuf + (t & 1) * TS;
-        const FT rt = lower ? rpiv[t] : (FT)1;
-        if (tx == t - 32 * j) {
-#pragma unroll
-          for (int a = 0; a < SA; ++a) cb[ty + 16 * a] = X[a][j] * rt;
-        }
-        const int c = tx + 32 * j;
-        const FT m = (c > t) ? (lower ? Dg[t * LD + c] : Dg[c * LD + t]) : (FT)0;
-        __syncthreads();
-#pragma unroll
-        for (int a = 0; a < SA; ++a) {
-          const FT x = cb[ty + 16 * a];
-          if (c > t) X[a][j] -= x * m;
-          else if (c == t) X[a][j] = x;  // final value of column t
-        }
-      }
-      if (j + 1 < CB) {
-        for (int kk = 0; kk < 32; ++kk) {
-          FT xv[SA];
-#pragma unroll
-          for (int a = 0; a < SA; ++a) xv[a] = __shfl_sync(0xffffffffu, X[a][j], kk);
-          const int k = 32 * j + kk;
-#pragma unroll
-          for (int b = j + 1; b < CB; ++b) {
-            const int c = tx + 32 * b;
-            const FT m = lower ? Dg[k * LD + c] : Dg[c * LD + k];
-#pragma unroll
-            for (int a = 0; a < SA; ++a) X[a][b] -= xv[a] * m;
-          }
-        }
-      }
+  const FT* M = Dg;
+  if (!lower) {
+    for (int e = tid; e < TS * TS; e += nt) {
+      const int c = e / TS, t = e % TS;  // consecutive threads read a row of L
+      if (t < c) Mb[t * LD + c] = Dg[c * LD + t];
+    }
+    M = Mb;
+    __syncthreads();
+  }
+  for (int J = 0; J < NK; ++J) {
+    const int j0 = J * NB;
+    if (tid < SLAB) panel_row<FT, LD>(Xs + tid * LD + j0, M + j0 * LD + j0, lower ? rpiv + j0 : nullptr);
+    __syncthreads();
+    if (J + 1 < NK) {
+      panel_update<FT, LD>(Xs, Xs, M, j0, 0, SLAB / NB, j0 + NB, NK - 1 - J);
+      __syncthreads();
     }
   }
-#pragma unroll
-  for (int a = 0; a < SA; ++a)
-#pragma unroll
-    for (int b = 0; b < CB; ++b) P[(ty + 16 * a) * TS + tx + 32 * b] = X[a][b];
+  for (int e = tid; e < SLAB * RV; e += nt) *(Vec*)(P + e * G) = *(const Vec*)(Xs + e / RV * LD + e % RV * G);
   if (lower && LT) {  // (L_other,k)^T: entry [c][r] = L[r][c]
     FT* out = LT + ((int64_t)other * TB + (other - k - 1)) * TS * TS;
-#pragma unroll
-    for (int a = 0; a < SA; ++a)
-#pragma unroll
-      for (int b = 0; b < CB; ++b) out[(int64_t)(tx + 32 * b) * TS + q * SLAB + ty + 16 * a] = X[a][b];
+    for (int e = tid; e < SLAB * TS; e += nt) out[(int64_t)(e / SLAB) * TS + q * SLAB + e % SLAB] = Xs[e % SLAB * LD + e / SLAB];
   }
 }
 
@@ -748,7 +784,8 @@ inline int grid_for_n(int64_t n, int threads = 256) {
 
 template <typename FT, int TS, int NS>
 size_t panel_smem() {
-  return sizeof(FT) * ((size_t)TS * (TS + 1) + 5 * (size_t)TS);
+  constexpr size_t NB = dev::LuTile<FT>::NB;
+  return sizeof(FT) * ((2 * (size_t)TS + TS / NS) * panel_ld<FT, TS>() + TS + NB * NB);
 }
 template <typename FT, int TS, int NS>
 size_t update_simt_smem() {
