@@ -866,9 +866,10 @@ __global__ void __launch_bounds__(256) k_coarse_inverse(int N0, int b0, const FT
 
 // k_coarse_inverse_blocks: 32 columns per CTA.  With one column per CTA every column streams all packed
 // operands from L2 (N_0 = 5235, b_0 = 197: 38 GB, 3.5 ms).  Here a step's operands are staged once in
-// shared memory for 32 columns (lane = column): each warp holds the block of its columns in registers
-// and takes rows of the operands, read as broadcast 16-byte groups (2.4 ms, bound by those reads).
-// The rows that a block couples to are kept in a window of shared memory; the forward result of a
+// shared memory for 32 columns.  Rows of the operands as broadcast 16-byte groups against one column per
+// lane took a shared-memory word per multiply-add (2.4 ms); a warp now takes 32 rows (FP64: 16) by 32
+// columns, a lane 8 x 4 (4 x 4) of them, for 12 words per 32 multiply-adds (1.4 ms).  The rows that
+// a block couples to are kept in a window of shared memory; the forward result of a
 // block goes through AinvT.  A column's sums are those of band_solve_packed: even and odd terms
 // apart, blocks in order.
 template <typename FT>
@@ -904,6 +905,46 @@ __device__ __forceinline__ void inverse_dots(const FT* rows, int r, const FT* v,
   }
 #pragma unroll
   for (int i = 0; i < R; ++i) out[i] = a0[i] + a1[i];
+}
+// Rows r0 + TR (lane / 8) + i (i < TR; rows past `rows` read the last one) of the operands times columns
+// lane % 8 + 8 c of the BS x 32 block `v`, even and odd terms apart as above.
+template <int TR, typename FT>
+__device__ __forceinline__ void inverse_tile(const FT* ops, int r0, int rows, const FT* v, int ld, FT (&out)[TR][4]) {
+  constexpr int BS = dev::SolveBlock<FT>::BS, G = dev::LuTile<FT>::G;
+  using Vec = dev::LuVec<FT>;
+  const int lane = threadIdx.x & 31;
+  int r[TR];
+#pragma unroll
+  for (int i = 0; i < TR; ++i) r[i] = min(r0 + TR * (lane >> 3) + i, rows - 1);
+  v += lane & 7;
+  FT odd[TR][4];
+#pragma unroll
+  for (int i = 0; i < TR; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) out[i][c] = odd[i][c] = 0;
+#pragma unroll 2
+  for (int j = 0; j < BS; j += G) {
+    Vec w[TR];
+#pragma unroll
+    for (int i = 0; i < TR; ++i) w[i] = *(const Vec*)(ops + r[i] * BS + dev::packed_at<FT>(r[i], j));
+#pragma unroll
+    for (int q = 0; q < G; q += 2) {
+      FT a[4], b[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) a[c] = v[(j + q) * ld + 8 * c], b[c] = v[(j + q + 1) * ld + 8 * c];
+#pragma unroll
+      for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          out[i][c] += w[i].v[q] * a[c];
+          odd[i][c] += w[i].v[q + 1] * b[c];
+        }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < TR; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) out[i][c] += odd[i][c];
 }
 template <typename FT>
 __global__ void __launch_bounds__(256) k_coarse_inverse_blocks(int N0, int b0, const FT* __restrict__ Dinv,
@@ -961,7 +1002,7 @@ __global__ void __launch_bounds__(256) k_coarse_inverse_blocks(int N0, int b0, c
     if (buffers > 1) stage(s + 1, ops + ((s + 1) & 1) * SP);
     constexpr int RW = BS / 8;  // rows of the diagonal block per warp (eight warps)
     const int slot = (t % WB) * BS;
-    FT v[BS], x[RW], y[4];
+    FT v[BS], x[RW];
     FT* blk = win + slot * LD + lane;
 #pragma unroll
     for (int j = 0; j < BS; ++j) v[j] = blk[j * LD];
@@ -976,16 +1017,20 @@ __global__ void __launch_bounds__(256) k_coarse_inverse_blocks(int N0, int b0, c
       const int r = (tid + 256 * q) % BS, c = (tid + 256 * q) / BS;
       if (k0 + r < N0 && c0 + c < N0) AinvT[(int64_t)(c0 + c) * N0 + k0 + r] = win[(slot + r) * LD + c];
     }
+    constexpr int TR = 2 * G;  // rows per lane
+    for (int r0 = wid * 4 * TR; r0 < b0; r0 += 32 * TR) {
+      FT y[TR][4];
+      inverse_tile<TR, FT>(cur + BS * BS, r0, b0, win + slot * LD, LD, y);
+      const int r = r0 + TR * (lane >> 3);
 #pragma unroll
-    for (int j = 0; j < BS; ++j) v[j] = blk[j * LD];
-    for (int r = wid * 4; r < b0; r += 32) {
-      inverse_dots<4, FT>(cur + BS * BS, r, v, y);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < TR; ++i) {
         const int row = fwd ? k0 + BS + r + i : k0 - 1 - r - i;
         int at = fwd ? slot + BS + r + i : slot - 1 - r - i;  // row mod WR
         at = at >= WR ? at - WR : at < 0 ? at + WR : at;
-        if (r + i < b0 && row >= 0 && row < N0) win[at * LD + lane] -= y[i];
+        if (r + i < b0 && row >= 0 && row < N0) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) win[at * LD + (lane & 7) + 8 * c] -= y[i][c];
+        }
       }
     }
     __syncthreads();
@@ -1000,11 +1045,45 @@ __global__ void __launch_bounds__(256) k_coarse_inverse_blocks(int N0, int b0, c
 // AinvT), warp partials are summed in shared memory in warp order, chunk partials go to
 // `part` and k_gemv_finish adds them in chunk order (no atomics: the result is reproducible).
 // With `skip` set (a refinement that has converged) both kernels return at once.
+//
+// What bounds it is the FP64 unit: N_0^2 multiply-adds, and as long again for widening FP32 entries with
+// the conversion instruction, which runs there too (N_0 = 5235: 115 us, of which the 110 MB take 17).  So
+// an entry is widened with integer instructions (59 us), which is exact but for zeros, subnormal numbers,
+// infinities and NaN: a warp lane that meets one among its next entries converts those the usual way.
 constexpr int kGemvChunks = 16;
 // Largest coarse dimension with an explicit inverse (N0^2 entries in the factors' precision:
 // 1 GB in FP32 at the limit); larger coarse problems use the one-CTA band solve.
 constexpr int kMaxInverseN0 = 16384;
 constexpr int kInverseColumns = 2048;  // coarse dofs up to which the inverse is formed column by column
+// acc += sum_i AinvT[i * stride] * g[8 i], i < U, in order
+template <int U>
+__device__ __forceinline__ double gemv_terms(const float* A, int64_t stride, const double* g, double acc) {
+  float a[U];
+  double b[U];
+  bool special = false;
+#pragma unroll
+  for (int i = 0; i < U; ++i) a[i] = A[i * stride], b[i] = g[8 * i];
+#pragma unroll
+  for (int i = 0; i < U; ++i) special |= (__float_as_uint(a[i]) << 1) - 0x01000000u >= 0xfe000000u;
+  if (!special) {
+    // sign, exponent re-biased by 1023 - 127, 23 bits of mantissa on top of the 52
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const int q = __float_as_int(a[i]);
+      acc += __hiloint2double(((q >> 3) & (int)0x8fffffff) + (896 << 20), q << 29) * b[i];
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < U; ++i) acc += (double)a[i] * b[i];
+  }
+  return acc;
+}
+template <int U>
+__device__ __forceinline__ double gemv_terms(const double* A, int64_t stride, const double* g, double acc) {
+#pragma unroll
+  for (int i = 0; i < U; ++i) acc += A[i * stride] * g[8 * i];
+  return acc;
+}
 template <typename FT>
 __global__ void __launch_bounds__(256) k_dense_gemv_t(int N0, const FT* AinvT, const double* g, double* part,
                                                        const int* skip) {
@@ -1015,8 +1094,13 @@ __global__ void __launch_bounds__(256) k_dense_gemv_t(int N0, const FT* AinvT, c
   const int per = (N0 + gridDim.y - 1) / gridDim.y;
   const int c0 = blockIdx.y * per, c1 = min(N0, c0 + per);
   double acc = 0.0;
-  if (row < N0)
-    for (int col = c0 + wid; col < c1; col += 8) acc += (double)AinvT[(int64_t)col * N0 + row] * g[col];
+  if (row < N0) {
+    int col = c0 + wid;
+    const int64_t stride = 8 * (int64_t)N0;
+    for (; col + 56 < c1; col += 64) acc = gemv_terms<8>(AinvT + (int64_t)col * N0 + row, stride, g + col, acc);
+    for (; col + 8 < c1; col += 16) acc = gemv_terms<2>(AinvT + (int64_t)col * N0 + row, stride, g + col, acc);
+    if (col < c1) acc = gemv_terms<1>(AinvT + (int64_t)col * N0 + row, stride, g + col, acc);
+  }
   acc_s[wid][lane] = acc;
   __syncthreads();
   if (wid == 0 && row < N0) {
