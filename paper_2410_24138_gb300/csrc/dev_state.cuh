@@ -134,6 +134,7 @@ struct Dev {
   unsigned long long* phase = nullptr;  // k_local_newton phase clocks (profiling)
   void* ainv = nullptr;                 // explicit A_0^-1 (transposed, factor precision) for the tangent phase
   double* gpart = nullptr;              // GEMV chunk partials
+  unsigned* gticket = nullptr;          // CTAs done per GEMV row tile (0 between launches)
   double* cpart = nullptr;              // refinement of the explicit-inverse solves: per-CTA partial norms
   int* cflag = nullptr;                 // [0] refinement converged, [1] ticket counter
   bool ainv_valid = false;

@@ -1042,9 +1042,11 @@ __global__ void __launch_bounds__(256) k_coarse_inverse_blocks(int N0, int b0, c
 
 // z = A_0^-1 g with the explicit inverse (stored transposed).  Grid (row tiles of 32, column
 // chunks): lane = row, the 8 warps of a CTA stride over the chunk's columns (coalesced rows of
-// AinvT), warp partials are summed in shared memory in warp order, chunk partials go to
-// `part` and k_gemv_finish adds them in chunk order (no atomics: the result is reproducible).
-// With `skip` set (a refinement that has converged) both kernels return at once.
+// AinvT), warp partials are summed in shared memory in warp order, chunk partials go to `part`, and the
+// last CTA of a row tile (a ticket per tile) adds them in chunk order, so the result is reproducible
+// (a launch of its own for that sum: 3 to 6 us per application).  z = the sum (accumulate = 0) or z +=
+// it (accumulate = 1); `reset`, if given, is cleared (the refinement flag of the solve that starts
+// here).  With `skip` set (a refinement that has converged) the kernel returns at once.
 //
 // What bounds it is the FP64 unit: N_0^2 multiply-adds, and as long again for widening FP32 entries with
 // the conversion instruction, which runs there too (N_0 = 5235: 115 us, of which the 110 MB take 17).  So
@@ -1086,7 +1088,8 @@ __device__ __forceinline__ double gemv_terms(const double* A, int64_t stride, co
 }
 template <typename FT>
 __global__ void __launch_bounds__(256) k_dense_gemv_t(int N0, const FT* AinvT, const double* g, double* part,
-                                                       const int* skip) {
+                                                       unsigned* tickets, double* z, int accumulate, const int* skip,
+                                                       int* reset) {
   if (skip && *skip) return;
   __shared__ double acc_s[8][33];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1103,25 +1106,30 @@ __global__ void __launch_bounds__(256) k_dense_gemv_t(int N0, const FT* AinvT, c
   }
   acc_s[wid][lane] = acc;
   __syncthreads();
-  if (wid == 0 && row < N0) {
+  if (wid != 0) return;
+  if (row < N0) {
     double t = 0.0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) t += acc_s[w][lane];
     part[(int64_t)blockIdx.y * N0 + row] = t;
   }
-}
-
-// z = sum of the chunk partials (accumulate = 0) or z += it (accumulate = 1); `reset`, if
-// given, is cleared (the refinement flag of the solve that starts here).
-__global__ void k_gemv_finish(int N0, int chunks, const double* part, double* z, int accumulate, const int* skip,
-                              int* reset) {
-  if (skip && *skip) return;
-  if (reset && blockIdx.x == 0 && threadIdx.x == 0) *reset = 0;
-  for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < N0; row += gridDim.x * blockDim.x) {
-    double t = 0.0;
-    for (int c = 0; c < chunks; ++c) t += part[(int64_t)c * N0 + row];
-    z[row] = accumulate ? z[row] + t : t;
+  __threadfence();
+  __syncwarp();
+  unsigned n = 0;
+  if (lane == 0) n = atomicAdd(tickets + blockIdx.x, 1u);
+  if (__shfl_sync(0xffffffffu, n, 0) != kGemvChunks - 1) return;
+  __threadfence();
+  if (lane == 0) {
+    tickets[blockIdx.x] = 0;
+    if (reset && blockIdx.x == 0) *reset = 0;
   }
+  if (row >= N0) return;
+  double p[kGemvChunks], t = 0.0;
+#pragma unroll
+  for (int c = 0; c < kGemvChunks; ++c) p[c] = __ldcg(part + (int64_t)c * N0 + row);
+#pragma unroll
+  for (int c = 0; c < kGemvChunks; ++c) t += p[c];
+  z[row] = accumulate ? z[row] + t : t;
 }
 
 // One step of the refinement of an explicit-inverse coarse solve: r = g - A_0 z (FP64 band
@@ -2140,9 +2148,12 @@ void coarse_solve(Context& c, const double* g, double* z) {
     const dim3 gg((N0 + 31) / 32, kGemvChunks);
     const bool f32 = fp32_coarse(c);
     auto apply_inverse = [&](const double* rhs, int accumulate, const int* skip, int* reset) {
-      if (f32) LAUNCH(D, k_dense_gemv_t<float>, gg, 256, 0, N0, (const float*)D.ainv, rhs, D.gpart, skip);
-      else LAUNCH(D, k_dense_gemv_t<double>, gg, 256, 0, N0, (const double*)D.ainv, rhs, D.gpart, skip);
-      LAUNCH(D, k_gemv_finish, grid_for(N0), 256, 0, N0, kGemvChunks, D.gpart, z, accumulate, skip, reset);
+      if (f32)
+        LAUNCH(D, k_dense_gemv_t<float>, gg, 256, 0, N0, (const float*)D.ainv, rhs, D.gpart, D.gticket, z, accumulate,
+               skip, reset);
+      else
+        LAUNCH(D, k_dense_gemv_t<double>, gg, 256, 0, N0, (const double*)D.ainv, rhs, D.gpart, D.gticket, z, accumulate,
+               skip, reset);
     };
     apply_inverse(g, 0, nullptr, D.cflag);
     const int sweeps = f32 ? std::min(c.opt.ir_max_sweeps, 3) : 0;
@@ -2520,6 +2531,8 @@ int device_setup(Context& c) {
         if (fp32_coarse(c)) D.ainv = D.alloc<float>((size_t)cs.N0 * cs.N0);
         else D.ainv = D.alloc<double>((size_t)cs.N0 * cs.N0);
         D.gpart = D.alloc<double>((size_t)cs.N0 * kGemvChunks);
+        D.gticket = D.alloc<unsigned>((cs.N0 + 31) / 32);
+        CK(cudaMemsetAsync(D.gticket, 0, (cs.N0 + 31) / 32 * sizeof(unsigned), D.s));
         set_smem(k_coarse_inverse<float>, lim);
         set_smem(k_coarse_inverse<double>, lim);
         set_smem(k_coarse_inverse_blocks<float>, lim);
