@@ -4,18 +4,20 @@
 //   k_local_newton   one persistent launch per F_x evaluation: every overlapping subdomain
 //                    (longest first, pulled from a device work counter) runs its local
 //                    Newton loop for Eq. 4 -- colour-ordered element assembly of the FP64
-//                    residual and of the local Jacobian (CSR), sliding-window band LU in
-//                    FP32 or FP64, triangular solves with FP64 iterative refinement, Armijo
+//                    residual and of the local Jacobian (rows in slices of 32), tiled band LU
+//                    in FP32 or FP64, triangular solves with FP64 iterative refinement, Armijo
 //                    line search -- and refactors the Jacobian at the converged state for the
 //                    exact tangent (Eq. 6 / Eq. 12).  It writes P~_i T_i straight into F_x.
 //   k_local_apply    one CTA per subdomain: sum_i P~_i (R_i DF(v_i) P_i)^-1 R_i DF(v_i) y.
 //   k_harmonic       energy-minimising extension of the RGDSW interface values (setup).
 //   k_galerkin       per non-overlapping subdomain: Phi_j^T K^(j)(x) Phi_j (coarse matrix).
-//   k_coarse_*       band LU / solve of A_0 = P_0^T DF P_0 in one CTA (Eq. 9).
+//   k_local_factor   the refactorisation at the converged states, where it is a launch of its own.
+//   k_coarse_*       band LU / solve of A_0 = P_0^T DF P_0 in one CTA (Eq. 9), its explicit inverse;
+//                    k_dense_gemv_t applies that.
 //   k_elem_residual, k_node_residual   global residual F(u): element contributions, then fixed-order
 //                    sums per node.
 //   k_global_jacobian  colour-ordered global Jacobian DF(u) (Eq. 3).
-//   k_vec_*          GMRES vector kernels with fixed-order (deterministic) reductions.
+//   k_dots, k_gmres_*  GMRES vector kernels with fixed-order (deterministic) reductions.
 #include <cuda_runtime.h>
 
 #include <algorithm>
