@@ -1244,6 +1244,7 @@ __device__ __forceinline__ bool band_solve_ring(int n, int b, const FT* __restri
   constexpr int BS = SolveBlock<FT>::BS;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int cw = ring_warps<FT>(b), nblk = (n + BS - 1) / BS, nf = nblk - t0, steps = nf + nblk;
+  if (nblk == 0) return true;  // no unknowns: no operands are issued, so nothing may wait for them
   const int64_t PB = packed_block_entries<FT>(b);
   uint64_t* full = (uint64_t*)ring;
   uint64_t* empty = full + kRingMax;

@@ -1,0 +1,60 @@
+"""Problems at the edges of what setup accepts.
+
+* A subdomain without unknowns (every node of it and of its overlap pinned): F_x, the tangent and the
+  solve against the oracle, under the bounds of test_gpu_parity.py (F_x 1e-9; tangent 1e-9 in FP64 and,
+  FP32 factors being refined to 1e-10, 1e-7 in FP32; converged solutions 1e-8 and 1e-6).
+"""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from oracle import fem, schwarz as S
+from paper_2410_24138_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+TIGHT = dict(inner_rtol=1e-13, inner_atol=1e-15)
+
+
+@pytest.fixture(scope="module")
+def nls():
+    from paper_2410_24138_gb300 import build, nls as binding
+    build.build()
+    return binding
+
+
+def random_state(p, scale, seed=4):
+    rng = np.random.default_rng(seed)
+    free = fem.free_mask(p)
+    return np.where(free, scale * rng.random(free.size), 0.0), np.where(free, rng.random(free.size), 0.0)
+
+
+def compare(s, p, coupling, load, scale, tol, opts=TIGHT):
+    sw = S.Schwarz(p, S.Options(coupling=coupling, **opts))
+    u, v = random_state(p, scale)
+    Fx, _, st = s.eval_Fx(u, load)
+    Fo, sto = sw.evaluate(u, load)
+    assert np.all(st == 0)
+    assert np.linalg.norm(Fx - Fo) <= 1e-9 * np.linalg.norm(Fo)
+    y, yo = s.apply_tangent(v), sw.tangent(sto)(v)
+    assert np.linalg.norm(y - yo) <= tol * np.linalg.norm(yo)
+
+
+def pinned_corner():
+    """12 x 12 P1 cells in 3 x 3 boxes, overlap 1, every node of [0, 1/2]^2 pinned."""
+    p = I.diffusion_problem(12, I.box_partition(12, 3, 3), 9, 1)
+    pin = np.nonzero((p.xy <= 0.5).all(axis=1))[0]
+    return dataclasses.replace(p, dirichlet_nodes=np.union1d(p.dirichlet_nodes, pin).astype(np.int64))
+
+
+@pytest.mark.parametrize("coupling", ["one", "add", "hybrid"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_subdomain_without_unknowns(nls, coupling, precision):
+    p = pinned_corner()
+    s = nls.make_solver(p, coupling=coupling, precision=precision, outer_atol=1e-12, **TIGHT)
+    assert s.local_dofs(0)[0].size == 0 and s.local_dofs(8)[0].size > 0
+    compare(s, p, coupling, 0.5, 0.05, 1e-9 if precision == "fp64" else 1e-7)
+    u, rep = s.solve()
+    assert rep.status == 0
+    uo, _ = S.plain_newton(p, tol=1e-14)
+    assert np.linalg.norm(u - uo) <= (1e-8 if precision == "fp64" else 1e-6) * np.linalg.norm(uo)
