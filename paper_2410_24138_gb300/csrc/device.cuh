@@ -1263,12 +1263,12 @@ __device__ __forceinline__ bool band_solve_ring(int n, int b, const FT* __restri
   asm volatile("fence.proxy.async;" ::: "memory");
   __syncthreads();
   const size_t sb = ring_stage_bytes<FT>(b);
+  int issued = 0;  // steps whose copies the copying thread has sent out
   if (wid == cw) {
     if (lane == 0) {
       const uint32_t dbytes = sizeof(FT) * BS * BS, cbytes = (uint32_t)(sizeof(FT) * BS * b);
       int st = 0;
       uint32_t par = 1;  // parity of the previous use of the stage
-      int issued = 0;
       for (int s = 0; s < steps; ++s) {
         if (s >= stages && !tc::mbar_wait(empty + st, par)) {
           *dead = 1;
@@ -1287,10 +1287,6 @@ __device__ __forceinline__ bool band_solve_ring(int n, int b, const FT* __restri
           st = 0;
           par ^= 1;
         }
-      }
-      if (issued < steps) {  // gave up: see the copies in flight land before the memory is used again
-        for (int s = issued > stages ? issued - stages : 0; s < issued; ++s)
-          tc::mbar_wait(full + s % stages, (uint32_t)(s / stages) & 1u);
       }
     }
     __syncwarp();
@@ -1366,6 +1362,10 @@ __device__ __forceinline__ bool band_solve_ring(int n, int b, const FT* __restri
   }
   __syncthreads();
   const bool ok = *dead == 0;
+  // some wait gave up (on either side): see the copies in flight land before the memory is used again
+  if (!ok && wid == cw && lane == 0)
+    for (int s = issued > stages ? issued - stages : 0; s < issued; ++s)
+      tc::mbar_wait(full + s % stages, (uint32_t)(s / stages) & 1u);
   __syncthreads();
   if (tid == 0)
     for (int q = 0; q < stages; ++q) {

@@ -1,0 +1,58 @@
+// Device routines of the library behind plain C calls, for the tests that look at one routine alone.
+#include <cuda_runtime.h>
+
+#include "device.cuh"
+
+using namespace nls;
+
+namespace {
+
+template <typename FT>
+__global__ void k_ring(int n, int b, const FT* P, FT* x, int stages, int* ok) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  constexpr int BS = dev::SolveBlock<FT>::BS;
+  FT* y = (FT*)smem;
+  unsigned char* ring = smem + ((n + BS - 1) / BS * BS * sizeof(FT) + 127) / 128 * 128;
+  for (int a = threadIdx.x; a < n; a += blockDim.x) y[a] = x[a];
+  __syncthreads();
+  const bool r = dev::band_solve_ring<FT>(n, b, P, y, ring, stages);
+  if (threadIdx.x == 0) *ok = r ? 1 : 0;
+  for (int a = threadIdx.x; a < n; a += blockDim.x) x[a] = y[a];
+}
+
+// x = (packed operands P)^-1 x in one CTA, `host` arrays in and out; without_copies: the CTA comes
+// without its copying warp, so that no operand ever arrives.  Returns a CUDA error code.
+template <typename FT>
+int ring(int n, int b, const FT* P, FT* x, int stages, int without_copies, int* ok) {
+  constexpr int BS = dev::SolveBlock<FT>::BS;
+  const size_t nblk = (n + BS - 1) / BS, np = nblk * dev::packed_block_entries<FT>(b);
+  const size_t sm = (nblk * BS * sizeof(FT) + 127) / 128 * 128 + dev::kRingHead + stages * dev::ring_stage_bytes<FT>(b);
+  FT *dP = nullptr, *dx = nullptr;
+  int* dok = nullptr;
+  cudaMalloc(&dP, np * sizeof(FT));
+  cudaMalloc(&dx, n * sizeof(FT));
+  cudaMalloc(&dok, sizeof(int));
+  cudaMemcpy(dP, P, np * sizeof(FT), cudaMemcpyHostToDevice);
+  cudaMemcpy(dx, x, n * sizeof(FT), cudaMemcpyHostToDevice);
+  cudaFuncSetAttribute(k_ring<FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_ring<FT><<<1, dev::ring_threads<FT>(b) - (without_copies ? 32 : 0), sm>>>(n, b, dP, dx, stages, dok);
+  cudaMemcpy(x, dx, n * sizeof(FT), cudaMemcpyDeviceToHost);
+  cudaMemcpy(ok, dok, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaFree(dP);
+  cudaFree(dx);
+  cudaFree(dok);
+  return (int)cudaGetLastError();
+}
+
+}  // namespace
+
+extern "C" {
+
+int probe_ring_f32(int n, int b, const float* P, float* x, int stages, int without_copies, int* ok) {
+  return ring<float>(n, b, P, x, stages, without_copies, ok);
+}
+int probe_ring_f64(int n, int b, const double* P, double* x, int stages, int without_copies, int* ok) {
+  return ring<double>(n, b, P, x, stages, without_copies, ok);
+}
+
+}  // extern "C"
