@@ -63,7 +63,7 @@ struct TileLU {
   void* DG = nullptr;  // factored diagonal tiles (unit L below the diagonal, U on and above it)
   CUtensorMap map;     // FP32 tiles as a 2D tensor of rows of TS values (TMA, 32 x TS boxes)
   bool solve_tiles = false;  // FP32: inverted diagonal tiles and solve products for the cluster solve
-  int32_t* solve_status = nullptr;  // ST_TIMEOUT once a cluster solve gave up waiting (else 0)
+  int32_t* solve_status = nullptr;  // ST_TIMEOUT once a cluster solve of this call gave up waiting (else 0)
   int64_t launches_per_factor = 0;
 };
 
@@ -143,7 +143,7 @@ struct Dev {
   bool local_reuse_active = false;   // chord steps allowed (inside nls_solve with local_reuse)
   int clock_khz = 1;
   double* h_scal = nullptr;  // pinned
-  int *err_host = nullptr, *err_dev = nullptr;  // host-mapped: a local solve gave up waiting
+  int *err_host = nullptr, *err_dev = nullptr;  // host-mapped: [2], a triangular solve gave up waiting
   int m = 0;                 // GMRES restart length allocated
   bool tangent_ready = false;
   void* guess = nullptr;  // learned-guess attachment (guess.cu)

@@ -2066,6 +2066,15 @@ void check_local_waits(Dev& D) {
   throw DeviceTimeout("a triangular solve gave up waiting for its operands");
 }
 
+// Ends a call that failed: its work is awaited and what its waits reported is dropped, so that it is not
+// taken for a later call's.
+void forget_waits(Dev& D) {
+  if (D.tlu && D.tlu->solve_status) cudaMemsetAsync(D.tlu->solve_status, 0, sizeof(int32_t), D.s);
+  cudaStreamSynchronize(D.s);
+  if (D.s2) cudaStreamSynchronize(D.s2);
+  if (D.err_host) *(volatile int*)D.err_host = 0;
+}
+
 // Reads the coarse factorization's status word (synchronises the stream).
 bool coarse_status_ok(Dev& D) {
   int32_t st = 0;
@@ -2301,10 +2310,12 @@ CoarseResult coarse_newton(Context& c, const double* u, double load) {
 // ------------------------------------------------------------------------------------------
 namespace {
 
-// The flag that a kernel whose bounded wait gave up sets (host memory, mapped).
+// The flags that a kernel whose bounded wait gave up sets (host memory, mapped): [0] is read at the end of
+// the call that launched it; [1] takes those of the allocation-free corrections, which report it in the
+// subdomains' status words and return before their work is done.
 void alloc_err(Dev& D) {
-  CK(cudaHostAlloc(&D.err_host, sizeof(int), cudaHostAllocMapped));
-  *D.err_host = 0;
+  CK(cudaHostAlloc(&D.err_host, 2 * sizeof(int), cudaHostAllocMapped));
+  D.err_host[0] = D.err_host[1] = 0;
   CK(cudaHostGetDevicePointer((void**)&D.err_dev, D.err_host, 0));
 }
 
@@ -3128,12 +3139,15 @@ int solve(Context& c, double* u_user, int u_dev, nls_report* rep) {
   } catch (const DeviceTimeout& ex) {
     c.last_error = ex.what();
     status = NLS_E_DEVICE_TIMEOUT;
+    forget_waits(D);
   } catch (const CudaFailure& ex) {
     c.last_error = ex.what();
     status = NLS_E_CUDA;
+    forget_waits(D);
   } catch (const std::exception& ex) {
     c.last_error = ex.what();
     status = NLS_E_ARG;
+    forget_waits(D);
   }
   rp.kernel_launches = D.launches - launches0;
   rp.status = status;
@@ -3173,9 +3187,11 @@ int eval_Fx(Context& c, const double* u, double* Fx, int is_dev, double load, in
     if (fi.pivot_failure) return NLS_E_PIVOT;
   } catch (const DeviceTimeout& ex) {
     c.last_error = ex.what();
+    forget_waits(D);
     return NLS_E_DEVICE_TIMEOUT;
   } catch (const std::exception& ex) {
     c.last_error = ex.what();
+    forget_waits(D);
     return NLS_E_CUDA;
   }
   return NLS_OK;
@@ -3198,9 +3214,11 @@ int apply_tangent(Context& c, const double* v, double* y, int is_dev) {
     check_local_waits(D);
   } catch (const DeviceTimeout& ex) {
     c.last_error = ex.what();
+    forget_waits(D);
     return NLS_E_DEVICE_TIMEOUT;
   } catch (const std::exception& ex) {
     c.last_error = ex.what();
+    forget_waits(D);
     return NLS_E_CUDA;
   }
   return NLS_OK;
@@ -3525,6 +3543,7 @@ int local_corrections_noalloc(Context& c, const double* x, double* Fx, int32_t* 
     A.load = load;
     A.guess = nullptr;
     A.want_tangent = 0;
+    A.err = D.err_dev + 1;
     // the work counter must start at zero; the rest of the area is written before it is read
     CK(cudaMemsetAsync(A.queue, 0, sizeof(int32_t), D.s));
     LAUNCH(D, k_mask, grid_for(c.N), 256, 0, c.N, D.free_dof, Fx);

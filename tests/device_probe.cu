@@ -1,6 +1,8 @@
-// Device routines of the library behind plain C calls, for the tests that look at one routine alone.
+// Device routines of the library behind plain C calls, for the tests that look at one routine alone, and
+// the words in which a context's kernels report a wait that gave up.
 #include <cuda_runtime.h>
 
+#include "dev_state.cuh"
 #include "device.cuh"
 
 using namespace nls;
@@ -53,6 +55,17 @@ int probe_ring_f32(int n, int b, const float* P, float* x, int stages, int witho
 }
 int probe_ring_f64(int n, int b, const double* P, double* x, int stages, int without_copies, int* ok) {
   return ring<double>(n, b, P, x, stages, without_copies, ok);
+}
+
+// What a wait that gave up leaves behind: the flag of the triangular solves and, with a tiled coarse
+// factorization, the status of the coarse cluster solves.  Returns whether there is such a status.
+int probe_report_wait(void* ctx) {
+  Dev& D = *((Context*)ctx)->dev;  // an nls_ctx holds its Context and nothing else
+  *(volatile int*)D.err_host = 1;
+  if (!D.tlu || !D.tlu->solve_status) return 0;
+  const int32_t st = ST_TIMEOUT;
+  cudaMemcpy(D.tlu->solve_status, &st, sizeof(st), cudaMemcpyHostToDevice);
+  return 1;
 }
 
 }  // extern "C"

@@ -3,6 +3,7 @@
 * The operand ring of the triangular solves on operands that solve a diagonal matrix, exact in both
   precisions; and its bounded waits: a CTA whose copying warp is missing gets no operand, gives up after
   the limit, reports it, and leaves the device usable.
+* A wait that gave up in one call: that call reports it, the next one on the same context does not.
 """
 import ctypes
 import os
@@ -56,3 +57,29 @@ def test_ring(probe, n, b, stages, dtype):
     assert ok.value == 0
     assert run(n, b, ptr(P), ptr(x), stages, 0, ctypes.byref(ok)) == 0
     assert ok.value == 1 and np.array_equal(x, 0.0625 * np.arange(1, n + 1).astype(dtype))
+
+
+@pytest.mark.parametrize("factor", ["band", "tiles"])
+@pytest.mark.parametrize("call", ["solve", "eval_Fx", "apply_tangent"])
+def test_report_of_a_wait_ends_with_its_call(probe, call, factor):
+    from paper_2410_24138_gb300 import inputs as I, nls
+    p = I.diffusion_problem(24, I.box_partition(24, 4, 4), 16, 1)
+    s = nls.make_solver(p, coupling="hybrid", coarse_factor=getattr(nls, "COARSE_FACTOR_" + factor.upper()),
+                        coarse_reuse=0)  # a call then depends on its inputs alone
+    rng = np.random.default_rng(0)
+    u = 0.05 * rng.random(p.n_nodes)
+    u[p.dirichlet_nodes] = 0.0
+    s.eval_Fx(u)
+
+    def run():
+        out = getattr(s, call)(u.copy())
+        return out[0] if isinstance(out, tuple) else out
+
+    want = run()
+    tiles = probe.probe_report_wait(s.h)
+    assert tiles == (factor == "tiles")
+    with pytest.raises(nls.NLSError) as err:
+        run()
+    assert err.value.status == -9
+    s.eval_Fx(u)
+    assert np.array_equal(run(), want)
