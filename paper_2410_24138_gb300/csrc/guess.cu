@@ -68,9 +68,19 @@ struct GuessNet {
   template <typename T>
   T* alloc(size_t n) {
     void* q = nullptr;
-    CK(cudaMalloc(&q, std::max<size_t>(n, 1) * sizeof(T)));
+    const cudaError_t e = cudaMalloc(&q, std::max<size_t>(n, 1) * sizeof(T));
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // reported here, not by the next launch
+      throw CudaFailure(std::string("network buffers: ") + cudaGetErrorString(e));
+    }
     allocs.push_back(q);
     return (T*)q;
+  }
+  void release(void* q) {
+    const auto it = std::find(allocs.begin(), allocs.end(), q);
+    if (!q || it == allocs.end()) return;
+    allocs.erase(it);
+    cudaFree(q);
   }
   void ensure_batch(int B);
   void ensure_chunk(int batch);
@@ -589,20 +599,25 @@ __global__ void k_guess_harvest(GeoArgs G, int nsub, const double* w, float* dX,
 
 }  // namespace
 
+// The work buffers grow as a whole: a failed allocation leaves the network with those it had.
 void GuessNet::ensure_batch(int B) {
   if (B <= bmax) return;
+  const int wide = std::max({h1, h2, no});
+  float** const buf[9] = {&X, &T, &Z1, &A1, &Z2, &A2, &Y, &dA, &dZ};
+  const int width[9] = {nf, no, h1, h1, h2, h2, no, wide, wide};
+  float* grown[9] = {};
+  try {
+    if (!lossbuf) lossbuf = alloc<float>(1024);
+    for (int k = 0; k < 9; ++k) grown[k] = alloc<float>((size_t)B * width[k]);
+  } catch (...) {
+    for (float* q : grown) release(q);
+    throw;
+  }
+  for (int k = 0; k < 9; ++k) {
+    release(*buf[k]);
+    *buf[k] = grown[k];
+  }
   bmax = B;
-  X = alloc<float>((size_t)B * nf);
-  T = alloc<float>((size_t)B * no);
-  const int hm = std::max(h1, h2);
-  Z1 = alloc<float>((size_t)B * h1);
-  A1 = alloc<float>((size_t)B * h1);
-  Z2 = alloc<float>((size_t)B * h2);
-  A2 = alloc<float>((size_t)B * h2);
-  Y = alloc<float>((size_t)B * no);
-  dA = alloc<float>((size_t)B * std::max(hm, no));
-  dZ = alloc<float>((size_t)B * std::max(hm, no));
-  lossbuf = alloc<float>(1024);
 }
 
 constexpr int kTrainChunk = 256;  // training steps issued between two reads of their losses
@@ -649,8 +664,10 @@ float loss_of(const float* parts) {
 void GuessNet::ensure_chunk(int batch) {
   if (!loss_chunk) loss_chunk = alloc<float>((size_t)kTrainChunk * kLossParts);
   if (batch <= chunk_batch) return;
+  int32_t* const grown = alloc<int32_t>((size_t)kTrainChunk * batch);
+  release(idx_chunk);
+  idx_chunk = grown;
   chunk_batch = batch;
-  idx_chunk = alloc<int32_t>((size_t)kTrainChunk * batch);
 }
 
 namespace {

@@ -1,0 +1,44 @@
+"""Batch sizes of the learned-guess network at the edges of its buffers.
+
+* A batch too large for the device's memory is refused, and the network goes on with the buffers it had:
+  the training steps after it are those of a network that never saw the request, bit for bit.
+"""
+import numpy as np
+import pytest
+
+from paper_2410_24138_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nls():
+    from paper_2410_24138_gb300 import build, nls as binding
+    build.build()
+    return binding
+
+
+def harvested(nls, seed=3):
+    """A small network with the 16 pairs of one F_x evaluation."""
+    p = I.diffusion_problem(32, I.box_partition(32, 4, 4), 16, 1)
+    s = nls.make_solver(p, coupling="one")
+    net = nls.GuessNet(h1=16, h2=16, seed=seed, capacity=16)
+    nls.attach_guess(s, net, nls.GUESS_HARVEST)
+    s.eval_Fx(np.zeros(p.n_nodes))
+    nls.attach_guess(s, None, 0)
+    s.close()
+    assert net.pairs() == 16
+    return net
+
+
+def test_failed_growth_keeps_the_buffers(nls):
+    a, b = harvested(nls), harvested(nls)
+    la, lb = [a.train(3, batch=8)], [b.train(3, batch=8)]
+    for _ in range(2):
+        with pytest.raises(nls.NLSError):  # 2^31 - 1 rows of 391 inputs: 3.4 TB
+            b.train(1, batch=2 ** 31 - 1)
+    for batch in (8, 300, 16):
+        la.append(a.train(3, batch=batch))
+        lb.append(b.train(3, batch=batch))
+    assert np.array_equal(np.concatenate(la), np.concatenate(lb))
+    assert np.all(np.isfinite(np.concatenate(la))) and np.array_equal(a.params(), b.params())
