@@ -60,7 +60,7 @@ struct GuessNet {
   float *X = nullptr, *T = nullptr, *Z1 = nullptr, *A1 = nullptr, *Z2 = nullptr, *A2 = nullptr, *Y = nullptr;
   float *dA = nullptr, *dZ = nullptr, *lossbuf = nullptr;
   // training: minibatch indices and partial losses of a chunk of steps, sums of squares of the targets
-  int chunk_batch = 0;
+  int64_t chunk_indices = 0;
   int32_t* idx_chunk = nullptr;
   float* loss_chunk = nullptr;
   double* sq = nullptr;
@@ -83,7 +83,7 @@ struct GuessNet {
     cudaFree(q);
   }
   void ensure_batch(int B);
-  void ensure_chunk(int batch);
+  void ensure_chunk(int64_t indices);
 };
 
 // per-context attachment: geometry maps and buffers
@@ -620,7 +620,10 @@ void GuessNet::ensure_batch(int B) {
   bmax = B;
 }
 
-constexpr int kTrainChunk = 256;  // training steps issued between two reads of their losses
+// Training steps issued between two reads of their losses: kTrainChunk, or as many (one at least) as have
+// kTrainIndices minibatch indices together (16 MB; from 16,384 rows on a step outlasts the read).
+constexpr int kTrainChunk = 256;
+constexpr int64_t kTrainIndices = int64_t(1) << 22;
 
 namespace {
 
@@ -661,13 +664,13 @@ float loss_of(const float* parts) {
 
 }  // namespace
 
-void GuessNet::ensure_chunk(int batch) {
+void GuessNet::ensure_chunk(int64_t indices) {
   if (!loss_chunk) loss_chunk = alloc<float>((size_t)kTrainChunk * kLossParts);
-  if (batch <= chunk_batch) return;
-  int32_t* const grown = alloc<int32_t>((size_t)kTrainChunk * batch);
+  if (indices <= chunk_indices) return;
+  int32_t* const grown = alloc<int32_t>((size_t)indices);
   release(idx_chunk);
   idx_chunk = grown;
-  chunk_batch = batch;
+  chunk_indices = indices;
 }
 
 namespace {
@@ -1206,14 +1209,16 @@ int nls_guess_train(nls_guess_net* w, int32_t steps, int32_t batch, double lr, u
     for (double v : sq) sum += v;
     const double hr = std::sqrt(sum / (double)std::max<int64_t>(N.npairs * N.no, 1));
     N.tscale = (float)(hr > 1e-30 ? hr : 1.0);
-    // The steps go out without waiting for one another: the minibatches of up to kTrainChunk steps are
-    // drawn and copied ahead, their partial losses stay on the device until the chunk is done.
+    // The steps go out without waiting for one another: the minibatches of a chunk of steps are drawn and
+    // copied ahead, their partial losses stay on the device until the chunk is done.
     nls::SplitMix rng{seed};
-    N.ensure_chunk(batch);
+    const int chunk = (int)std::max<int64_t>(
+        1, std::min<int64_t>(nls::kTrainIndices / batch, std::min(nls::kTrainChunk, (int)steps)));
+    N.ensure_chunk((int64_t)chunk * batch);
     std::vector<int32_t> idx;
     std::vector<float> parts;
-    for (int s0 = 0; s0 < steps; s0 += nls::kTrainChunk) {
-      const int ns = std::min(nls::kTrainChunk, steps - s0);
+    for (int s0 = 0; s0 < steps; s0 += chunk) {
+      const int ns = std::min(chunk, steps - s0);
       idx.resize((size_t)ns * batch);
       for (auto& r : idx) r = (int32_t)(rng.next() % (uint64_t)N.npairs);
       CK(cudaMemcpy(N.idx_chunk, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice));

@@ -2,6 +2,9 @@
 
 * A batch too large for the device's memory is refused, and the network goes on with the buffers it had:
   the training steps after it are those of a network that never saw the request, bit for bit.
+* One step of a large batch takes the memory of its activations and little more: 64 MB cover the
+  indices of its own rows and the allocator's granularity, not those of a chunk of steps (134 MB).
+* Steps that go out in several chunks are those of single calls.
 """
 import numpy as np
 import pytest
@@ -42,3 +45,23 @@ def test_failed_growth_keeps_the_buffers(nls):
         lb.append(b.train(3, batch=batch))
     assert np.array_equal(np.concatenate(la), np.concatenate(lb))
     assert np.all(np.isfinite(np.concatenate(la))) and np.array_equal(a.params(), b.params())
+
+
+def test_memory_of_a_large_step(nls):
+    import torch
+    net = harvested(nls)
+    net.train(1, batch=8)
+    batch = 1 << 17
+    free = torch.cuda.mem_get_info()[0]
+    net.train(1, batch=batch)
+    used = free - torch.cuda.mem_get_info()[0]
+    wide = max(net.h1, net.h2, net.n_out)
+    assert used <= 4 * batch * (net.n_in + 2 * net.n_out + 2 * net.h1 + 2 * net.h2 + 2 * wide) + (64 << 20)
+
+
+def test_chunks_of_steps(nls):
+    a, b = harvested(nls), harvested(nls)
+    batch = 1 << 20  # four steps to a chunk
+    la, lb = a.train(4, batch=batch, seed=5), b.train(6, batch=batch, seed=5)
+    assert np.array_equal(la, lb[:4])
+    assert np.all(np.isfinite(lb)) and lb[5] < lb[0]
