@@ -335,16 +335,28 @@ __global__ void __launch_bounds__(256) k_gemm_f32(int M, int N, int K, const flo
 template <bool AK, bool BK>
 void gemm_t(cudaStream_t s, bool bf16, int M, int N, int K, const float* A, int64_t lda, const float* B, int64_t ldb,
             const GemmOut& out) {
-  auto grid = [&](int t) { return dim3((N + t - 1) / t, (M + t - 1) / t); };
+  // One launch has at most 65,535 tile rows: more rows (batches of over two million) go out in slabs.  (A
+  // third grid dimension made 40 training steps of 256 rows 8 % slower, 6.28 -> 6.85 ms; tiles numbered along
+  // one dimension 2 %.)
+  auto slabs = [&](int t, auto kernel, int threads) {
+    const int64_t most = (int64_t)t * 65535;
+    for (int64_t m = 0; m < M; m += most) {
+      const int rows = (int)std::min<int64_t>(most, M - m);
+      GemmOut o = out;
+      o.C += m * o.ld;
+      if (o.act) o.act += m * o.ld;
+      if (o.z) o.z += m * o.ld;
+      kernel<<<dim3((N + t - 1) / t, (rows + t - 1) / t), threads, 0, s>>>(rows, N, K, A + (AK ? m * lda : m), lda, B, ldb, o);
+      CK(cudaGetLastError());
+    }
+  };
   if (bf16) {
-    k_gemm_bf16<AK, BK><<<grid(32), 128, 0, s>>>(M, N, K, A, lda, B, ldb, out);
+    slabs(32, k_gemm_bf16<AK, BK>, 128);
   } else {
     // 64 x 64 tiles once they give most SMs a CTA (16 x 16 sums per thread read half as much), else 32 x 32
-    const dim3 g = grid(64);
-    if (g.x * g.y >= 100) k_gemm_f32<AK, BK, 4><<<g, 256, 0, s>>>(M, N, K, A, lda, B, ldb, out);
-    else k_gemm_f32<AK, BK, 2><<<grid(32), 256, 0, s>>>(M, N, K, A, lda, B, ldb, out);
+    if (((int64_t)N + 63) / 64 * (((int64_t)M + 63) / 64) >= 100) slabs(64, k_gemm_f32<AK, BK, 4>, 256);
+    else slabs(32, k_gemm_f32<AK, BK, 2>, 256);
   }
-  CK(cudaGetLastError());
 }
 
 // C(i, j) = sum_k A(i, k) B(k, j).  ak (bk): A (B) is stored with K contiguous, row i (column j) lda

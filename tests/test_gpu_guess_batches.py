@@ -5,6 +5,10 @@
 * One step of a large batch takes the memory of its activations and little more: 64 MB cover the
   indices of its own rows and the allocator's granularity, not those of a chunk of steps (134 MB).
 * Steps that go out in several chunks are those of single calls.
+* More rows than one grid dimension has tiles for (65,535 x 32): with one training pair every batch has
+  the same loss.  Both sides add n equal FP32 terms per thread before the fixed tree, n up to 2^21 x 1024
+  / 65,536 = 32,768, each addition rounding to 2^-24 relative: 2^15 x 2^-24 = 2e-3, and as much again for
+  the division by the batch size.
 """
 import numpy as np
 import pytest
@@ -65,3 +69,17 @@ def test_chunks_of_steps(nls):
     la, lb = a.train(4, batch=batch, seed=5), b.train(6, batch=batch, seed=5)
     assert np.array_equal(la, lb[:4])
     assert np.all(np.isfinite(lb)) and lb[5] < lb[0]
+
+
+def test_more_rows_than_a_grid_dimension(nls):
+    p = I.diffusion_problem(8, I.box_partition(8, 1, 1), 1, 1)
+    losses = []
+    for batch in (64, 65535 * 32 + 33):
+        s = nls.make_solver(p, coupling="one")
+        net = nls.GuessNet(h1=16, h2=16, seed=3, capacity=1)
+        nls.attach_guess(s, net, nls.GUESS_HARVEST)
+        s.eval_Fx(np.zeros(p.n_nodes))
+        nls.attach_guess(s, None, 0)
+        losses.append(net.train(1, batch=batch)[0])
+        net.close()
+    assert abs(losses[1] - losses[0]) <= 4e-3 * losses[0]
