@@ -1184,8 +1184,9 @@ __device__ void band_solve_packed(int n, int b, const FT* __restrict__ P, FT* y,
 // Ring in shared memory (16-byte aligned): 128 bytes of mbarriers and a flag, then the stages, each
 // the diagonal inverse and the coupling of one block and direction.  y: nblk BS entries, 16-byte
 // aligned.  Needs ring_threads(b) threads and two stages; every thread of the CTA calls it, after a
-// barrier that follows the writes of y and P.  The forward sweep starts at block t0: y must vanish in
-// the rows before it.  Returns false if a bounded wait gave up.
+// barrier that follows the writes of y and P.  n > 0: without unknowns there are no operands, and the
+// first wait would be for one.  The forward sweep starts at block t0: y must vanish in the rows before
+// it.  Returns false if a bounded wait gave up.
 // ------------------------------------------------------------------------------------------
 constexpr int kRingMax = 6;
 constexpr int kRingHead = 128;
@@ -1244,7 +1245,6 @@ __device__ __forceinline__ bool band_solve_ring(int n, int b, const FT* __restri
   constexpr int BS = SolveBlock<FT>::BS;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int cw = ring_warps<FT>(b), nblk = (n + BS - 1) / BS, nf = nblk - t0, steps = nf + nblk;
-  if (nblk == 0) return true;  // no unknowns: no operands are issued, so nothing may wait for them
   const int64_t PB = packed_block_entries<FT>(b);
   uint64_t* full = (uint64_t*)ring;
   uint64_t* empty = full + kRingMax;
@@ -1263,7 +1263,7 @@ __device__ __forceinline__ bool band_solve_ring(int n, int b, const FT* __restri
   asm volatile("fence.proxy.async;" ::: "memory");
   __syncthreads();
   const size_t sb = ring_stage_bytes<FT>(b);
-  int issued = 0;  // steps whose copies the copying thread has sent out
+  int issued = steps;  // steps whose copies the copying thread has sent out
   if (wid == cw) {
     if (lane == 0) {
       const uint32_t dbytes = sizeof(FT) * BS * BS, cbytes = (uint32_t)(sizeof(FT) * BS * b);
@@ -1272,6 +1272,7 @@ __device__ __forceinline__ bool band_solve_ring(int n, int b, const FT* __restri
       for (int s = 0; s < steps; ++s) {
         if (s >= stages && !tc::mbar_wait(empty + st, par)) {
           *dead = 1;
+          issued = s;
           break;
         }
         const bool fwd = s < nf;
@@ -1282,7 +1283,6 @@ __device__ __forceinline__ bool band_solve_ring(int n, int b, const FT* __restri
         tc::mbar_arrive_expect_tx(full + st, dbytes + cbytes);
         tc::bulk_load(dst, d, dbytes, full + st);
         if (cbytes) tc::bulk_load(dst + dbytes, c, cbytes, full + st);
-        issued = s + 1;
         if (++st == stages) {
           st = 0;
           par ^= 1;

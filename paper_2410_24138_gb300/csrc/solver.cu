@@ -339,8 +339,8 @@ __device__ __forceinline__ void for_row(const LocalArgs& A, const SubMeta& m, in
   for (; k < bw.y; ++k) f(v[k * h], c[k * h]);
 }
 
-// y = (packed operands)^-1 y through the ring where it has two stages and the CTA the threads, else
-// with the operands in registers.  Returns false if a bounded wait gave up.
+// y = (packed operands)^-1 y through the ring where it has two stages (none without unknowns) and the CTA
+// the threads, else with the operands in registers.  Returns false if a bounded wait gave up.
 struct Ring {
   unsigned char* mem;
   int stages;
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : LAW == NLS_LAW_DIFFUS
     double* s = A.work + A.work_stride + m.vec_off;  // Newton step
     // the LU window serves the solves: the solve vector, then the ring of operands
     const size_t ring_at = align_up(P.win + sizeof(FT) * align_up(n, dev::SolveBlock<FT>::BS), 128);
-    const Ring ring{smem + ring_at, ring_at < P.flag ? dev::ring_stages<FT>(m.b, P.flag - ring_at) : 0};
+    const Ring ring{smem + ring_at, n > 0 && ring_at < P.flag ? dev::ring_stages<FT>(m.b, P.flag - ring_at) : 0};
     for (int t = tid; t < m.nt; t += blockDim.x)
       xt[t] = A.x[(int64_t)A.tnode_gid[m.tnode_off + t / nd] * nd + t % nd];
     __syncthreads();
@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 128 ? 3 : 1) k_local_apply(Local
   const int sub = A.order[blockIdx.x], tid = threadIdx.x, nd = A.ndof;
   const SubMeta m = A.meta[sub];
   const int n = m.n;
-  const Ring ring{smem + P.flag, A.ring ? dev::ring_stages<FT>(m.b, P.total - P.flag) : 0};
+  const Ring ring{smem + P.flag, A.ring && n > 0 ? dev::ring_stages<FT>(m.b, P.total - P.flag) : 0};
   const FT* Dv = (const FT*)A.dinv + m.dinv_off;
   double* q = A.work + m.vec_off;
   for (int t = tid; t < m.nt; t += blockDim.x) yt[t] = A.v[(int64_t)A.tnode_gid[m.tnode_off + t / nd] * nd + t % nd];
