@@ -78,6 +78,7 @@ struct LocalArgs {
   double rtol, atol, armijo, ir_rtol;
   int maxit, ls_trials, ir_max;
   int l2_dist;            // L2 prefetch distance of the triangular solves (blocks; 0 = off)
+  int gal_rows;           // coarse blocks: rows of Phi and K Phi in shared memory
   int ring;               // tangent application: stages of the operand ring (0: operands in registers)
   int* err;               // host-mapped: set when a bounded wait gave up
   const double* x;        // evaluation point (global)
@@ -722,10 +723,16 @@ __global__ void __launch_bounds__(256) k_harmonic(LocalArgs A) {
   }
 }
 
-// Rows of Phi_j and K^(j) Phi_j that the Galerkin kernel keeps in shared memory at a time.
+// Rows of Phi_j and K^(j) Phi_j that the Galerkin kernel keeps in shared memory at a time: kGalRows, or as
+// many (one at least) as leave room for two CTAs per SM where a subdomain has more than 226 coarse dofs (a
+// long one beside many small ones).  The sums run over the rows in order, however many are kept.
 constexpr int kGalRows = 32;
-size_t galerkin_smem(int max_nt, int max_nc) {
-  return sizeof(double) * std::max((size_t)max_nt, (size_t)2 * kGalRows * max_nc);
+int galerkin_rows(size_t smem_optin, int max_nc) {
+  const size_t half = (smem_optin + 1024) / 2 - 1024;  // 1 KB of every CTA is the system's
+  return (int)std::min<size_t>(kGalRows, std::max<size_t>(1, half / (2 * sizeof(double) * std::max(max_nc, 1))));
+}
+size_t galerkin_smem(size_t smem_optin, int max_nt, int max_nc) {
+  return sizeof(double) * std::max((size_t)max_nt, (size_t)2 * galerkin_rows(smem_optin, max_nc) * max_nc);
 }
 
 template <int LAW>
@@ -752,11 +759,11 @@ __global__ void __launch_bounds__(256, 2) k_galerkin(LocalArgs A) {
     Y[idx] = acc;
   }
   __syncthreads();
-  // block = Phi_j^T Y: rows of Phi and Y through shared memory, kGalRows at a time, one thread per entry
+  // block = Phi_j^T Y: rows of Phi and Y through shared memory, A.gal_rows at a time, one thread per entry
   // (a warp per entry read both arrays 8 bytes at a time, nc entries apart).  Eq. 2's tangent is
   // symmetric: the entries c <= d are formed, and mirrored.
-  double* ps = xt;  // the table vector has been used; kGalRows x nc of Phi, then of Y
-  double* ys = ps + kGalRows * nc;
+  double* ps = xt;  // the table vector has been used; A.gal_rows x nc of Phi, then of Y
+  double* ys = ps + A.gal_rows * nc;
   double* blk = A.blk + A.blk_off[j];
   const bool sym = LAW == NLS_LAW_NEOHOOKE;
   const int pairs = sym ? nc * (nc + 1) / 2 : nc * nc;
@@ -773,8 +780,8 @@ __global__ void __launch_bounds__(256, 2) k_galerkin(LocalArgs A) {
       d = e % nc;
     }
     double acc = 0.0;
-    for (int t0 = 0; t0 < m.nt; t0 += kGalRows) {
-      const int rows = min(kGalRows, m.nt - t0);
+    for (int t0 = 0; t0 < m.nt; t0 += A.gal_rows) {
+      const int rows = min(A.gal_rows, m.nt - t0);
       __syncthreads();
       for (int q = tid; q < rows * nc; q += blockDim.x) {
         ps[q] = phi[(int64_t)t0 * nc + q];
@@ -2101,7 +2108,8 @@ void coarse_assemble_launch(Context& c, const double* x) {
   LocalArgs A = coarse_args(c);
   A.x = x;
   const int T = 256;
-  const size_t sm = galerkin_smem(c.nov.max_nt, c.cs.max_nc);
+  A.gal_rows = galerkin_rows(D.smem_optin, c.cs.max_nc);
+  const size_t sm = galerkin_smem(D.smem_optin, c.nov.max_nt, c.cs.max_nc);
   if (c.law == NLS_LAW_DIFFUSION) LAUNCH(D, (k_galerkin<NLS_LAW_DIFFUSION>), c.nov.count, T, sm, A);
   else LAUNCH(D, (k_galerkin<NLS_LAW_NEOHOOKE>), c.nov.count, T, sm, A);
   const int64_t ne = (int64_t)c.cs.N0 * (2 * c.cs.b0 + 1);
@@ -2513,6 +2521,7 @@ int device_setup(Context& c) {
       Coarse& cs = c.cs;
       if (cs.N0 == 0) throw std::runtime_error("the partition has no coarse nodes (one subdomain?)");
       if (!coarse_tiles(c)) need(coarse_factor_smem(c, fp32_coarse(c)), "coarse band factorization");
+      need(galerkin_smem(lim, c.nov.max_nt, cs.max_nc), "coarse blocks");
       need((fp32_coarse(c) ? sizeof(float) : sizeof(double)) * (size_t)cs.N0, "coarse band solve");
       upload_set(D, c.nov, D.nov, false, false);
       D.phi = D.upload(cs.phi_host);

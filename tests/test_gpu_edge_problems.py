@@ -3,6 +3,10 @@
 * A subdomain without unknowns (every node of it and of its overlap pinned): F_x, the tangent and the
   solve against the oracle, under the bounds of test_gpu_parity.py (F_x 1e-9; tangent 1e-9 in FP64 and,
   FP32 factors being refined to 1e-10, 1e-7 in FP32; converged solutions 1e-8 and 1e-6).
+* A long thin subdomain beside hundreds of small ones: some 460 coarse dofs meet in it, more than the
+  shared memory of an SM holds 2 x 32 rows of, and A_0 is as good as full, which in FP64 also takes the
+  coarse inverse's form with one operand buffer (half bandwidth above 430).  F_x and the tangent under the
+  same bounds (A_0 has a condition below 100, the global tangent one below 200).
 """
 import dataclasses
 
@@ -58,3 +62,28 @@ def test_subdomain_without_unknowns(nls, coupling, precision):
     assert rep.status == 0
     uo, _ = S.plain_newton(p, tol=1e-14)
     assert np.linalg.norm(u - uo) <= (1e-8 if precision == "fp64" else 1e-6) * np.linalg.norm(uo)
+
+
+def strip_problem(law, boxes):
+    """4 x 2 boxes cells: columns 0 and 1 are one subdomain, columns 2 and 3 are boxes of 2 x 2; the left edge is
+    clamped."""
+    nx, ny = 4, 2 * boxes
+    if law == "p1":
+        p = I.diffusion_problem(2, np.zeros(4, dtype=np.int32), 1, 1)
+    else:
+        p = dataclasses.replace(I.neohooke_problem(2, np.zeros(4, dtype=np.int32), 1, 1, traction_max=0.0),
+                                traction_edges=None, traction=None)
+    xy, conn = I.structured_rect_mesh(nx, ny, p.elem_type, 1.0, ny / nx)
+    cell = np.arange(nx * ny)
+    sub = np.where(cell % nx < 2, 0, 1 + cell // nx // 2).astype(np.int32)
+    return dataclasses.replace(p, n=nx, xy=xy, conn=conn, dirichlet_nodes=np.nonzero(xy[:, 0] == 0)[0].astype(np.int64),
+                               elem_to_sub=I.cell_to_elem_partition(sub, p.elem_type), n_sub=1 + boxes, overlap=1)
+
+
+@pytest.mark.parametrize("law,boxes", [("p1", 460), ("q1", 158)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_subdomain_with_many_coarse_dofs(nls, law, boxes, precision):
+    p = strip_problem(law, boxes)
+    s = nls.make_solver(p, coupling="hybrid", precision=precision, **TIGHT)
+    assert s.sizes().n_coarse_dofs > 454 and s.sizes().coarse_half_band > 430
+    compare(s, p, "hybrid", 0.5, 0.02, 1e-9 if precision == "fp64" else 1e-7)
