@@ -1,12 +1,21 @@
 // Internal host-side structures of the nls library (not part of the C ABI).
 #pragma once
 #include <cstdint>
+#include <stdexcept>
 #include <string>
 #include <vector>
 
 #include "nls.h"
 
 namespace nls {
+
+// Sizes of a sliced matrix: `entries` are counted in int32_t, positions among the `padded` ones are kept as
+// 32-bit words and read as unsigned, which leaves room for the padding.
+inline void check_sliced(int64_t entries, int64_t padded, const char* what) {
+  if (entries > INT32_MAX || padded > (int64_t)UINT32_MAX)
+    throw std::runtime_error(std::string(what) + " too large for 32-bit positions");
+}
+inline int32_t position32(int64_t at) { return (int32_t)(uint32_t)at; }
 
 // Per-subdomain metadata, uploaded verbatim to the device (plain old data).
 struct SubMeta {
@@ -82,7 +91,7 @@ struct Coarse {
   std::vector<int32_t> p0_col;
   std::vector<int64_t> p0_src;     // index into the concatenated Phi blocks, -1 for padding
   std::vector<int32_t> p0t_rowptr, p0t_col;  // transpose: rows = coarse dofs, col = global dof
-  std::vector<int32_t> p0t_src;    // index into p0 values
+  std::vector<int32_t> p0t_src;    // index into p0 values (position32)
   // per non-overlapping subdomain j: columns C_j and dense Phi_j [nt_j x nc_j] (row-major)
   std::vector<int32_t> cj_ptr, cj_col;
   std::vector<int64_t> phi_off;    // offset of Phi_j in the concatenated array
@@ -133,7 +142,7 @@ struct Context {
   // rows (and rows past N) are padded with column 0 and a value that stays zero
   std::vector<int64_t> g_slice;
   std::vector<int32_t> g_col;
-  std::vector<int32_t> g_epos;               // [elem][(nen*ndof)^2], element order = conn order
+  std::vector<int32_t> g_epos;               // [elem][(nen*ndof)^2] (position32), element order = conn order
   std::vector<double> geom;                  // per element geometry
   int geom_stride = 0;
   std::vector<double> fext;                  // per dof, load factor 1

@@ -382,10 +382,9 @@ void build_global(Context& c) {
       rowptr[v * nd + da + 1] = (int32_t)c.g_col.size();
     }
   }
-  if (c.g_col.size() > (size_t)INT32_MAX) throw std::runtime_error("global Jacobian too large for 32-bit positions");
+  check_sliced((int64_t)c.g_col.size(), 0, "global Jacobian");
   c.g_slice = slice_starts(rowptr);
-  // positions are kept as 32-bit words, read as unsigned: room for the padding
-  if (c.g_slice.back() > (int64_t)UINT32_MAX) throw std::runtime_error("global Jacobian too large for 32-bit positions");
+  check_sliced((int64_t)c.g_col.size(), c.g_slice.back(), "global Jacobian");
   c.g_epos.assign((size_t)c.n_elems * ned * ned, 0);
   in_ranges(c.n_elems, [&](int64_t e0, int64_t e1) {
     for (int64_t e = e0; e < e1; ++e)
@@ -398,7 +397,7 @@ void build_global(Context& c) {
             for (int db = 0; db < nd; ++db) {
               int32_t col = c.conn[e * nen + bb] * nd + db;
               c.g_epos[(size_t)e * ned * ned + (a * nd + da) * ned + bb * nd + db] =
-                  (int32_t)(uint32_t)sliced(c.g_slice, row, std::lower_bound(b0, b1, col) - b0);
+                  position32(sliced(c.g_slice, row, std::lower_bound(b0, b1, col) - b0));
             }
         }
   });
@@ -687,6 +686,7 @@ void build_coarse(Context& c) {
       }
       rowptr[g + 1] = (int32_t)cs.p0_col.size();
     }
+  check_sliced((int64_t)cs.p0_col.size(), 0, "coarse basis");
   // transpose (CSR), with the positions of the sliced P_0
   std::vector<int32_t> cnt(cs.N0 + 1, 0);
   for (int32_t col : cs.p0_col) cnt[col + 1] += 1;
@@ -696,6 +696,7 @@ void build_coarse(Context& c) {
   cs.p0t_src.assign(cs.p0_col.size(), 0);
   {
     cs.p0_slice = slice_starts(rowptr);
+    check_sliced((int64_t)cs.p0_col.size(), cs.p0_slice.back(), "coarse basis");
     std::vector<int32_t> col(cs.p0_slice.back(), 0);
     std::vector<int64_t> src(cs.p0_slice.back(), -1);
     std::vector<int32_t> fill(cnt.begin(), cnt.end() - 1);
@@ -706,7 +707,7 @@ void build_coarse(Context& c) {
         src[at] = cs.p0_src[k];
         int32_t pos = fill[cs.p0_col[k]]++;
         cs.p0t_col[pos] = (int32_t)g;
-        cs.p0t_src[pos] = (int32_t)at;
+        cs.p0t_src[pos] = position32(at);
       }
     cs.p0_col.swap(col);
     cs.p0_src.swap(src);

@@ -812,9 +812,10 @@ __global__ void k_gather_values(int64_t n, const int64_t* src, const double* fro
     to[k] = src[k] >= 0 ? from[src[k]] : 0.0;
 }
 
+// the same for positions kept by position32
 __global__ void k_gather_values32(int64_t n, const int32_t* src, const double* from, double* to) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    to[k] = from[src[k]];
+    to[k] = from[(uint32_t)src[k]];
 }
 
 // coarse band factorization (one CTA); the window also holds the packing scratch of at least four
