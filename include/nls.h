@@ -330,7 +330,8 @@ int nls_get_coarse_matrix(const nls_ctx* ctx, double* A0_out);
 int nls_band_solve(int device, int32_t n, int32_t b, const double* band, const double* rhs, double* x,
                    int32_t precision, int32_t method, double* factors_out);
 
-/* F(u) of Eq. 3 (Dirichlet rows zero) at load factor `load`; u, F of length n_dofs. */
+/* F(u) of Eq. 3 (Dirichlet rows zero) at load factor `load`; u, F of length n_dofs, which may be one array or
+ * overlap.  After an error other than NLS_E_ARG the contents of F are unspecified. */
 int nls_eval_F(nls_ctx* ctx, const double* u, double* F, int is_device, double load);
 
 /* F_x(u) (Eq. 5, 10 or 11 per the coupling option) at load factor `load`, and keep the
@@ -340,7 +341,8 @@ int nls_eval_F(nls_ctx* ctx, const double* u, double* F, int is_device, double l
 int nls_eval_Fx(nls_ctx* ctx, const double* u, double* Fx, int is_device, double load,
                 int32_t* local_its_out, int32_t* local_status_out);
 
-/* y = DF_x(u) v (Eqs. 6, 12) at the u of the last nls_eval_Fx. */
+/* y = DF_x(u) v (Eqs. 6, 12) at the u of the last nls_eval_Fx.  v and y may be one array or overlap; after an
+ * error other than NLS_E_ARG the contents of y are unspecified. */
 int nls_apply_tangent(nls_ctx* ctx, const double* v, double* y, int is_device);
 
 /* Converged local states w_i = R_i (u - P_i T_i(u)) of the last nls_eval_Fx, concatenated in

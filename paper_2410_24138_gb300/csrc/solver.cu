@@ -3215,9 +3215,13 @@ int apply_tangent(Context& c, const double* v, double* y, int is_dev) {
   }
   D.prof = c.opt.profile_kernels != 0;
   try {
-    if (!is_dev) CK(cudaMemcpyAsync(D.t1, v, sizeof(double) * c.N, cudaMemcpyHostToDevice, D.s));
+    // device arrays are used in place; where y overlaps v at an offset, it would be cleared over parts of v
+    // not read yet
+    const uintptr_t pv = (uintptr_t)v, py = (uintptr_t)y, bytes = sizeof(double) * c.N;
+    const bool staged = !is_dev || (pv != py && pv < py + bytes && py < pv + bytes);
+    if (staged) CK(cudaMemcpyAsync(D.t1, v, bytes, is_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, D.s));
     double* out = is_dev ? y : D.gx;
-    LAUNCH(D, k_masked_copy, grid_for(c.N), 256, 0, c.N, D.free_dof, is_dev ? v : D.t1, D.x, out);
+    LAUNCH(D, k_masked_copy, grid_for(c.N), 256, 0, c.N, D.free_dof, staged ? D.t1 : v, D.x, out);
     tangent(c, D.x, out);
     if (!is_dev) CK(cudaMemcpyAsync(y, D.gx, sizeof(double) * c.N, cudaMemcpyDeviceToHost, D.s));
     sync(D);

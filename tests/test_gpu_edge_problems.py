@@ -7,6 +7,7 @@
   shared memory of an SM holds 2 x 32 rows of, and A_0 is as good as full, which in FP64 also takes the
   coarse inverse's form with one operand buffer (half bandwidth above 430).  F_x and the tangent under the
   same bounds (A_0 has a condition below 100, the global tangent one below 200).
+* Device arrays that overlap, in F and in the tangent: the results of separate arrays, bit for bit.
 """
 import dataclasses
 
@@ -87,3 +88,21 @@ def test_subdomain_with_many_coarse_dofs(nls, law, boxes, precision):
     s = nls.make_solver(p, coupling="hybrid", precision=precision, **TIGHT)
     assert s.sizes().n_coarse_dofs > 454 and s.sizes().coarse_half_band > 430
     compare(s, p, "hybrid", 0.5, 0.02, 1e-9 if precision == "fp64" else 1e-7)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 37, -1, -500])
+def test_overlapping_device_arrays(nls, shift):
+    import torch
+    p = I.neohooke_problem(24, I.brick_partition(24, 2, 3, 5), 6, 1, traction_max=4.0, load_steps=1)
+    s = nls.make_solver(p, coupling="hybrid")
+    u, v = random_state(p, 1e-3)
+    n, at = u.size, 512
+    s.eval_Fx(u, 0.3)
+    for call, x, tail in ((s.lib.nls_apply_tangent, v, ()), (s.lib.nls_eval_F, u, (0.3,))):
+        want = s.apply_tangent(v) if not tail else s.eval_F(u, 0.3)
+        both = torch.zeros(n + 2 * at, dtype=torch.float64, device="cuda")
+        both[at:at + n] = torch.from_numpy(x).cuda()
+        first = both.data_ptr()
+        torch.cuda.synchronize()
+        assert call(s.h, first + 8 * at, first + 8 * (at + shift), 1, *tail) == 0
+        assert np.array_equal(both[at + shift:at + shift + n].cpu().numpy(), want)
