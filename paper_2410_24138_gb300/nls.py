@@ -344,8 +344,14 @@ class Solver:
         self._check(self.lib.nls_get_coarse_matrix(self.h, _ptr(out)), "nls_get_coarse_matrix")
         return out
 
+    def _result_like(self, a):
+        """An array for a result of the shape of `a`: the library writes its n_dofs entries, any beyond are 0."""
+        if isinstance(a, np.ndarray):
+            return np.zeros_like(a)
+        return a.new_empty(a.shape) if a.numel() == self.n_nodes * self.ndof else a.new_zeros(a.shape)
+
     def eval_F(self, u, load: float = 1.0):
-        F = np.zeros_like(u) if isinstance(u, np.ndarray) else u.new_empty(u.shape)  # every entry is written
+        F = self._result_like(u)
         self._check(self.lib.nls_eval_F(self.h, _ptr(u), _ptr(F), _is_device(u), load), "nls_eval_F")
         return F
 
@@ -358,7 +364,7 @@ class Solver:
         return Fx, its, st
 
     def apply_tangent(self, v):
-        y = np.zeros_like(v) if isinstance(v, np.ndarray) else v.new_empty(v.shape)  # every entry is written
+        y = self._result_like(v)
         self._check(self.lib.nls_apply_tangent(self.h, _ptr(v), _ptr(y), _is_device(v)), "nls_apply_tangent")
         return y
 

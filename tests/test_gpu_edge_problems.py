@@ -8,6 +8,8 @@
   coarse inverse's form with one operand buffer (half bandwidth above 430).  F_x and the tangent under the
   same bounds (A_0 has a condition below 100, the global tangent one below 200).
 * Device arrays that overlap, in F and in the tangent: the results of separate arrays, bit for bit.
+* A device array longer than the problem: the entries beyond come back as zeros, also in memory that the
+  allocator hands out again.
 """
 import dataclasses
 
@@ -106,3 +108,18 @@ def test_overlapping_device_arrays(nls, shift):
         torch.cuda.synchronize()
         assert call(s.h, first + 8 * at, first + 8 * (at + shift), 1, *tail) == 0
         assert np.array_equal(both[at + shift:at + shift + n].cpu().numpy(), want)
+
+
+def test_longer_device_arrays(nls):
+    import torch
+    p = I.diffusion_problem(16, I.box_partition(16, 2, 2), 4, 1)
+    s = nls.make_solver(p, coupling="one")
+    u, v = random_state(p, 0.05)
+    s.eval_Fx(u)
+    for call, x in ((s.eval_F, u), (s.apply_tangent, v)):
+        long = torch.from_numpy(np.concatenate([x, np.ones(7)])).cuda()
+        for _ in range(3):
+            used = [torch.full_like(long, 5.0) for _ in range(4)]
+            del used
+            out = call(long).cpu().numpy()
+            assert np.array_equal(out[:x.size], call(x)) and not out[x.size:].any()
