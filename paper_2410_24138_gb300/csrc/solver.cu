@@ -119,7 +119,7 @@ struct LocalPlan {
   size_t xt, racc, red, win, flag, total;
 };
 
-// Shared memory a CTA can opt in to (227 KB), less the kernels' static shared memory.
+// Shared memory a CTA can opt in to (227 KB), less one unit of its alignment.
 constexpr size_t kSmemFull = 227 * 1024 - 128;
 
 // Shared memory of the harmonic extension (k_harmonic): the table state, the solve vector and
@@ -435,7 +435,8 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : LAW == NLS_LAW_DIFFUS
   FT* win = (FT*)(smem + P.win);
   FT* yv = win;  // the solve vector lives in the LU window once the factors are packed
   int* flag = (int*)(smem + P.flag);
-  __shared__ int s_item;
+  // no static shared memory: in front of an array aligned to 128 bytes it would take as many of the limit
+  int* const s_item = flag + 3;
   const int tid = threadIdx.x, nd = A.ndof;
   const size_t win_cap = (P.flag - P.win) / sizeof(FT);
   const int inv_warps = min((int)(blockDim.x >> 5), (int)(win_cap / dev::pack_scratch<FT>()));
@@ -449,9 +450,9 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 128 ? 4 : LAW == NLS_LAW_DIFFUS
     }
   };
   for (;;) {
-    if (tid == 0) s_item = atomicAdd(A.queue, 1);
+    if (tid == 0) *s_item = atomicAdd(A.queue, 1);
     __syncthreads();
-    const int item = s_item;
+    const int item = *s_item;
     __syncthreads();
     if (item >= A.count) break;
     const int sub = A.order[item];

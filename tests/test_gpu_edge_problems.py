@@ -8,6 +8,10 @@
   coarse inverse's form with one operand buffer (half bandwidth above 430).  F_x and the tangent under the
   same bounds (A_0 has a condition below 100, the global tangent one below 200).
 * Device arrays that overlap, in F and in the tangent: the results of separate arrays, bit for bit.
+* One subdomain that takes the last of the shared memory that setup accepts (227 KB; the sizes below are
+  those of the limit: two FP64 vectors, the larger of the solve vector and a band window, and the rest),
+  under the bounds of test_gpu_band_tiles.py for such a subdomain: F_x 1e-9, the tangent, which is the
+  identity, 1e-6.
 * A device array longer than the problem: the entries beyond come back as zeros, also in memory that the
   allocator hands out again.
 """
@@ -123,3 +127,28 @@ def test_longer_device_arrays(nls):
             del used
             out = call(long).cpu().numpy()
             assert np.array_equal(out[:x.size], call(x)) and not out[x.size:].any()
+
+
+def test_subdomain_at_the_limit_of_shared_memory(nls):
+    nx, ny = 4, 2635
+    p = I.diffusion_problem(2, np.zeros(4, dtype=np.int32), 1, 1)
+    xy, conn = I.structured_rect_mesh(nx, ny, I.P1_TRI, 1.0, ny / nx)
+    nt, b, limit = xy.shape[0], nx + 1, 227 * 1024
+    pinned = np.nonzero(xy[:, 0] == 0)[0].astype(np.int64)
+    n = nt - pinned.size
+
+    def up16(k):
+        return (k + 15) // 16 * 16
+
+    assert limit - 128 < 8 * (nt + n) + 320 + up16(4 * n) + up16(4 * (b + 10)) + 16 <= limit - 16
+    p = dataclasses.replace(p, n=nx, xy=xy, conn=conn, dirichlet_nodes=pinned,
+                            elem_to_sub=np.zeros(conn.shape[0], dtype=np.int32), n_sub=1, overlap=1)
+    tight = dict(inner_rtol=1e-12, inner_atol=1e-13)
+    s = nls.make_solver(p, coupling="one", precision="fp32", **tight)
+    assert s.sizes().max_local_dofs == n and s.sizes().max_half_band == b
+    u, v = random_state(p, 0.05)
+    Fx, _, st = s.eval_Fx(u, 0.05)
+    Fo, _ = S.Schwarz(p, S.Options(coupling="one", **tight)).evaluate(u, 0.05)
+    assert np.all(st == 0)
+    assert np.linalg.norm(Fx - Fo) <= 1e-9 * np.linalg.norm(Fo)
+    assert np.linalg.norm(s.apply_tangent(v) - v) <= 1e-6 * np.linalg.norm(v)
