@@ -1647,14 +1647,21 @@ int local_threads(const Context& c) {
   return std::max(pick, min_local_threads(c));
 }
 
+// Threads of the operand ring at the largest half bandwidth, and the largest CTA of the tangent application:
+// in FP64 half bandwidths from 113 on need more, and keep the operands in registers (32 + b threads).
+constexpr int kApplyMax = 256;
+int apply_ring_threads(const Context& c) {
+  return c.opt.local_precision == NLS_PREC_FP32_IR ? dev::ring_threads<float>(c.ov.max_b)
+                                                   : dev::ring_threads<double>(c.ov.max_b);
+}
+
 // CTA size of the tangent application: the solving warps and the copying one, and enough threads for
 // the matrix products -- 256 while every subdomain has an SM to itself, else 128, three CTAs of which
 // share an SM.  (A kernel for 512 threads is held to 128 registers, and a solve step took 1900 cycles
 // instead of 750.)
 int apply_threads(const Context& c) {
-  const int ring = c.opt.local_precision == NLS_PREC_FP32_IR ? dev::ring_threads<float>(c.ov.max_b)
-                                                            : dev::ring_threads<double>(c.ov.max_b);
-  const int need = std::max(64, std::max(ring, min_local_threads(c)));
+  const int ring = apply_ring_threads(c);
+  const int need = std::max(64, std::max(ring <= kApplyMax ? ring : 0, min_local_threads(c)));
   if (c.dev && c.dev->apply_T) return std::max(c.dev->apply_T, need);
   const int nsm = c.dev ? c.dev->nsm : 152;
   return std::max(need, c.ov.count <= nsm ? 256 : 128);
@@ -1942,6 +1949,7 @@ void launch_local_newton(Context& c, const double* x, double* out, double load, 
 template <typename FT>
 int apply_ring_stages(const Context& c) {
   const Dev& D = *c.dev;
+  if (apply_ring_threads(c) > kApplyMax) return 0;
   const size_t per_sm = D.smem_optin + 1024, want = std::min(3, (c.ov.count + D.nsm - 1) / D.nsm);
   for (int st = dev::kRingMax; st >= 2; --st) {
     const size_t sm = apply_plan<FT>(c.ov.max_n, c.ov.max_nt, c.ov.max_b, st).total;

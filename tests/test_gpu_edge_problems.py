@@ -12,6 +12,9 @@
   those of the limit: two FP64 vectors, the larger of the solve vector and a band window, and the rest),
   under the bounds of test_gpu_band_tiles.py for such a subdomain: F_x 1e-9, the tangent, which is the
   identity, 1e-6.
+* FP64 and a half bandwidth of 113 (a small mesh numbered so that the first and the last unknown are
+  neighbours), where the operand ring would take more threads than the tangent's kernel has: F_x and the
+  tangent under the bounds above, and the same bits with the prefetch of the operands off and on.
 * A device array longer than the problem: the entries beyond come back as zeros, also in memory that the
   allocator hands out again.
 """
@@ -152,3 +155,21 @@ def test_subdomain_at_the_limit_of_shared_memory(nls):
     assert np.all(st == 0)
     assert np.linalg.norm(Fx - Fo) <= 1e-9 * np.linalg.norm(Fo)
     assert np.linalg.norm(s.apply_tangent(v) - v) <= 1e-6 * np.linalg.norm(v)
+
+
+def test_widest_band_in_fp64(nls):
+    p = I.diffusion_problem(2, np.zeros(4, dtype=np.int32), 1, 1)
+    xy, conn = I.structured_rect_mesh(4, 22, I.P1_TRI, 1.0, 5.5)
+    n = xy.shape[0] - 1
+    old = np.concatenate([[0], np.arange(2, n), [1, n]])  # node 1 becomes the last unknown; the last node is pinned
+    new = np.empty(n + 1, dtype=np.int32)
+    new[old] = np.arange(n + 1)
+    p = dataclasses.replace(p, n=4, xy=xy[old], conn=new[conn], dirichlet_nodes=np.array([n], dtype=np.int64),
+                            elem_to_sub=np.zeros(conn.shape[0], dtype=np.int32), n_sub=1, overlap=1)
+    got = []
+    for dist in (0, 4):
+        s = nls.make_solver(p, coupling="one", precision="fp64", l2_prefetch=dist, **TIGHT)
+        assert s.sizes().max_half_band == 113 and s.sizes().max_local_dofs == n
+        compare(s, p, "one", 0.05, 0.05, 1e-9)
+        got.append(s.apply_tangent(random_state(p, 0.05)[1]))
+    assert np.array_equal(*got)
