@@ -10,7 +10,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+#include <cstring>
 #include <type_traits>
+#include <vector>
 
 #include "nls_internal.h"
 #include "tcgen05.cuh"
@@ -120,6 +123,25 @@ __device__ inline void p1_jacobian(const double* geo, const P1State& s, T K[9]) 
 // Anything outside [2^-1007, 2^1007) (zero, negative, NaN and infinite among it) goes to log() and a
 // division.
 constexpr int kLogBins = 128;  // tab[i] = {r, -log r}, see log_table()
+// The table of log_inv: per bin of m in [0.75, 1.5) the reciprocal r of its middle (1 for the two
+// bins next to 1, where log must keep its relative accuracy) and -log r.
+inline std::vector<double2> log_table() {
+  auto from_hi = [](uint32_t hi) {
+    const uint64_t bits = (uint64_t)hi << 32;
+    double x;
+    std::memcpy(&x, &bits, sizeof(x));
+    return x;
+  };
+  std::vector<double2> t(kLogBins);
+  for (int i = 0; i < kLogBins; ++i) {
+    const double a = from_hi(0x3fe80000u + ((uint32_t)i << 13)), b = from_hi(0x3fe80000u + ((uint32_t)(i + 1) << 13));
+    const double r = (a == 1.0 || b == 1.0) ? 1.0 : (double)(2.0L / ((long double)a + (long double)b));
+    t[i].x = r;
+    t[i].y = (double)-std::log((long double)r);
+  }
+  return t;
+}
+
 struct LogInv {
   double log, inv;
 };

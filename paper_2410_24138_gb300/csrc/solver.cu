@@ -1687,27 +1687,8 @@ int coarse_solve_threads(const Context& c) { return std::max(256, (32 + c.cs.b0 
 dev::NHLaw nh_law(const Context& c) {
   dev::NHLaw law;
   lame(c, law.mu, law.lam);
-  law.tab = c.dev->logtab;
+  law.tab = c.dev->logtab;  // null for Eq. 1, which does not read it
   return law;
-}
-
-// The table of dev::log_inv: per bin of m in [0.75, 1.5) the reciprocal r of its middle (1 for the two
-// bins next to 1, where log must keep its relative accuracy) and -log r.
-std::vector<double2> log_table() {
-  auto from_hi = [](uint32_t hi) {
-    const uint64_t bits = (uint64_t)hi << 32;
-    double x;
-    std::memcpy(&x, &bits, sizeof(x));
-    return x;
-  };
-  std::vector<double2> t(dev::kLogBins);
-  for (int i = 0; i < dev::kLogBins; ++i) {
-    const double a = from_hi(0x3fe80000u + ((uint32_t)i << 13)), b = from_hi(0x3fe80000u + ((uint32_t)(i + 1) << 13));
-    const double r = (a == 1.0 || b == 1.0) ? 1.0 : (double)(2.0L / ((long double)a + (long double)b));
-    t[i].x = r;
-    t[i].y = (double)-std::log((long double)r);
-  }
-  return t;
 }
 
 LocalArgs make_args(const Context& c, const LocalSet& hs, const DeviceLocalSet& ds) {
@@ -2428,7 +2409,7 @@ int device_setup(Context& c) {
     D.smem_optin = prop.sharedMemPerBlockOptin;
     D.conn = D.upload(c.conn);
     D.geom = D.upload(c.geom);
-    D.logtab = D.upload(log_table());
+    if (c.law == NLS_LAW_NEOHOOKE) D.logtab = D.upload(dev::log_table());
     std::vector<double> k = c.k_elem;
     if (k.empty()) k.assign(c.n_elems, 1.0);
     D.kcoef = D.upload(k);
