@@ -4,6 +4,15 @@
   precisions; and its bounded waits: a CTA whose copying warp is missing gets no operand, gives up after
   the limit, reports it, and leaves the device usable.
 * A wait that gave up in one call: that call reports it, the next one on the same context does not.
+* log x and 1 / x of the element routines against extended precision, over the whole range, next to 1, at the
+  ends of the table's bins and binades, and on both sides of 2^-1007 and 2^1007, where log() and a division
+  take over.  log x = (e log 2 + c) + l, |c| < 0.41, |l| < 2^-7: for |log x| < 1 (|e| <= 2) half an ulp of c
+  (2.8e-17), of both sums (5.6e-17 each) and of log 2 (5.6e-17 x |e| / 2), and a few roundings of l (2e-18
+  each): 2.1e-16 absolute; beyond, one ulp of the result more than covers the two sums and e times log 2's
+  rounding (0.3 ulp), and log() has one: 2 ulp.  The reciprocal is one Newton step with one rounding in
+  the residual and one at the end: 1 ulp.
+* The pivots' reciprocal: in FP64 one rounding and a truncation of 2^-69 inside [2^-100, 2^100), a division
+  outside; in FP32 the correctly rounded one.
 """
 import ctypes
 import os
@@ -83,3 +92,64 @@ def test_report_of_a_wait_ends_with_its_call(probe, call, factor):
     assert err.value.status == -9
     s.eval_Fx(u)
     assert np.array_equal(run(), want)
+
+
+def special(dtype):
+    info = np.finfo(dtype)
+    return np.array([0.0, -0.0, -1.0, -3.5, info.tiny, info.smallest_subnormal, 3 * info.smallest_subnormal, info.max,
+                     np.inf, -np.inf, np.nan], dtype=dtype)
+
+
+def ulps(got, want):
+    """|got - want| in units in the last place of `want` (extended precision)."""
+    return np.abs(got.astype(np.longdouble) - want) / np.spacing(np.abs(want).astype(got.dtype)).astype(np.longdouble)
+
+
+def test_logarithm_and_reciprocal(probe):
+    rng = np.random.default_rng(2)
+    m = 200000
+    edges = np.concatenate([1.0 + np.arange(-32, 65) / 128.0, [0.75, 1.5]])
+    edges = np.outer(2.0 ** np.array([-1006, -500, -2, -1, 0, 1, 2, 500, 1005]), edges).ravel()
+    ends = np.array([2.0 ** -1007, 2.0 ** 1007, 2.0 ** -1006, 2.0 ** 1006])
+    x = np.concatenate([np.exp(rng.uniform(-1, 1, m)), rng.uniform(0.98, 1.02, m), np.exp(rng.uniform(-690, 690, m)),
+                        edges, np.nextafter(edges, 0), np.nextafter(edges, np.inf),
+                        ends, np.nextafter(ends, 0), np.nextafter(ends, np.inf)])
+    log, inv = np.empty_like(x), np.empty_like(x)
+    assert probe.probe_log_inv(x.size, ptr(x), ptr(log), ptr(inv)) == 0
+    want = np.log(x.astype(np.longdouble))
+    small = np.abs(want) < 1
+    assert np.max(np.abs(log[small] - want[small])) <= 2.1e-16
+    assert np.max(ulps(log[~small], want[~small])) <= 2
+    assert np.max(ulps(inv, 1 / x.astype(np.longdouble))) <= 1
+    assert log[x == 1.0][0] == 0.0
+    x = special(np.float64)
+    log, inv = np.empty_like(x), np.empty_like(x)
+    assert probe.probe_log_inv(x.size, ptr(x), ptr(log), ptr(inv)) == 0
+    with np.errstate(all="ignore"):
+        want, winv = np.where(x > 0, np.log(x), 0.0), 1 / x
+    finite = np.isfinite(want)
+    assert np.array_equal(log[~finite], want[~finite])
+    assert np.all(np.abs(log[finite] - want[finite]) <= 2 * np.spacing(np.abs(want[finite])))
+    assert np.array_equal(inv, winv, equal_nan=True)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_reciprocal_of_a_pivot(probe, dtype):
+    rng = np.random.default_rng(3)
+    run = probe.probe_recip_f32 if dtype == np.float32 else probe.probe_recip_f64
+    top = 120 if dtype == np.float32 else 1000
+    powers = 2.0 ** np.array([-1000, -120, -101, -100, -99, -1, 0, 1, 99, 100, 101, 120, 1000])
+    powers = powers[np.abs(np.log2(powers)) <= top].astype(dtype)
+    wide, near = 2.0 ** rng.uniform(-top, top, 200000), 2.0 ** rng.uniform(-100, 100, 200000)
+    x = np.concatenate([wide.astype(dtype), -near.astype(dtype), powers, np.nextafter(powers, dtype(0)),
+                        np.nextafter(powers, dtype(np.inf)), special(dtype)])
+    y = np.empty_like(x)
+    assert run(x.size, ptr(x), ptr(y)) == 0
+    with np.errstate(all="ignore"):
+        exact = dtype(1) / x
+    if dtype == np.float32:
+        assert np.array_equal(y, exact, equal_nan=True)
+        return
+    plain = np.isfinite(exact) & np.isfinite(x) & (np.abs(exact) >= np.finfo(dtype).tiny)
+    assert np.array_equal(y[~plain], exact[~plain], equal_nan=True)
+    assert np.max(ulps(y[plain], 1 / x[plain].astype(np.longdouble))) <= 0.501
