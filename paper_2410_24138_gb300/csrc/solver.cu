@@ -1750,9 +1750,12 @@ void set_smem(K kernel, size_t optin) {
 
 void sync(Dev& D) { CK(cudaStreamSynchronize(D.s)); }
 
-// Elements per thread of the tiled vector kernels: one while the tiles then fill the SMs at most once,
-// four up to a million elements, sixteen beyond (fewer partial sums to add).
-int tile_elems(const Dev& D, int64_t n) { return n <= (int64_t)kTile * D.nsm ? 1 : n <= (1 << 20) ? 4 : 16; }
+// Elements per thread of the tiled vector kernels: one while the tiles then fill the SMs at most once, four
+// beyond.  An iteration's orthogonalisation against 10 vectors (four launches) with 1 / 4 / 16 elements:
+// 35 / 44 / 81 us at n = 4,225, 46 / 47 / 84 at 50,000, 100 / 66 / 88 at 296,450, 259 / 152 / 151 at 1,050,625,
+// 1902 / 959 / 1136 at 8,396,802; against 40 vectors at the last size 5256 / 3033 / 4377 (sixteen elements
+// of w and of the sums leave a thread too few registers for several vectors in flight).
+int tile_elems(const Dev& D, int64_t n) { return n <= (int64_t)kTile * D.nsm ? 1 : 4; }
 int tile_grid(const Dev& D, int64_t n) {
   const int64_t t = (int64_t)kTile * tile_elems(D, n);
   return (int)std::max<int64_t>(1, (n + t - 1) / t);
@@ -1761,8 +1764,7 @@ int tile_grid(const Dev& D, int64_t n) {
 void dots(Dev& D, int64_t n, int nv, const double* V, int64_t ld, const double* coef, double* w, double* out) {
   const int E = tile_elems(D, n), grid = tile_grid(D, n);
   if (E == 1) LAUNCH_NAMED(D, "k_dots", k_dots<1>, grid, kTile, 0, n, nv, V, ld, coef, w, D.partial, D.ticket, out);
-  else if (E == 4) LAUNCH_NAMED(D, "k_dots", k_dots<4>, grid, kTile, 0, n, nv, V, ld, coef, w, D.partial, D.ticket, out);
-  else LAUNCH_NAMED(D, "k_dots", k_dots<16>, grid, kTile, 0, n, nv, V, ld, coef, w, D.partial, D.ticket, out);
+  else LAUNCH_NAMED(D, "k_dots", k_dots<4>, grid, kTile, 0, n, nv, V, ld, coef, w, D.partial, D.ticket, out);
 }
 
 // ---- reductions with a host read-back ---------------------------------------------------------
@@ -2950,8 +2952,7 @@ GmresResult gmres(Context& c, const double* b) {
                    D.gR, D.gcs, D.gsn, D.gg, D.gst, h, use_handle);
     };
     if (E == 1) update(k_gmres_update<1>);
-    else if (E == 4) update(k_gmres_update<4>);
-    else update(k_gmres_update<16>);
+    else update(k_gmres_update<4>);
     LAUNCH(D, k_scale_inv, grid_for(N), 256, 0, N, w, D.scal + kMaxGmresVecs, w);
   };
   GmresState st;
