@@ -86,7 +86,8 @@ struct Coarse {
   int N0 = 0;                      // coarse dofs
   int b0 = 0;                      // half bandwidth of A_0
   std::vector<int32_t> first_node; // smallest global node id per coarse node
-  // P_0 over global dofs in slices of 32 rows (as Context::g_slice; values filled on the device)
+  // P_0 over global dofs in slices of 32 rows (as Context::g_slice, but padded with column 0; values filled
+  // on the device)
   std::vector<int64_t> p0_slice;
   std::vector<int32_t> p0_col;
   std::vector<int64_t> p0_src;     // index into the concatenated Phi blocks, -1 for padding
@@ -139,7 +140,7 @@ struct Context {
   Coarse cs;
   std::vector<int32_t> g_color_ptr, g_elem;  // global element colouring
   // global matrix DF in slices of 32 rows: entry k of row i at g_slice[i / 32] + 32 k + i % 32; shorter
-  // rows (and rows past N) are padded with column 0 and a value that stays zero
+  // rows are padded with the row's own index (rows past N with N - 1) and a value that stays zero
   std::vector<int64_t> g_slice;
   std::vector<int32_t> g_col;
   std::vector<int32_t> g_epos;               // [elem][(nen*ndof)^2] (position32), element order = conn order

@@ -1067,7 +1067,11 @@ constexpr int kGemvChunks = 16;
 // Largest coarse dimension with an explicit inverse (N0^2 entries in the factors' precision:
 // 1 GB in FP32 at the limit); larger coarse problems use the one-CTA band solve.
 constexpr int kMaxInverseN0 = 16384;
-constexpr int kInverseColumns = 2048;  // coarse dofs up to which the inverse is formed column by column
+// Coarse dofs up to which the inverse is formed column by column.  FP32 launches beside the local solves, by
+// columns and 32 columns per CTA: 27 / 81 us at N_0 = 402, 207 / 232 at 1149, 407 / 527 at 1428, 402 / 539 at 2268,
+// 1046 / 860 at 3600 (b_0 = 59 .. 167); FP64, whose CTAs end at b_0 = 112: 86 / 695 us at 402, 967 / 3425 at
+// 1428.  The line lies below the crossing, where the two are within a third of each other.
+constexpr int kInverseColumns = 2048;
 // acc += sum_i AinvT[i * stride] * g[8 i], i < U, in order
 template <int U>
 __device__ __forceinline__ double gemv_terms(const float* A, int64_t stride, const double* g, double acc) {
@@ -2674,8 +2678,8 @@ void coarse_inverse_launch(Context& c) {
   const int N0 = c.cs.N0;
   const int b0 = c.cs.b0;
   // one CTA per column while that is bound by the latency of a column's steps: up to kInverseColumns
-  // columns and the half bandwidth of a 256-thread CTA (N_0 = 699, b_0 = 77: 158 us with 32 columns per
-  // CTA), then 32 columns per CTA, which read the operands 32 times less often
+  // columns and the half bandwidth of a 256-thread CTA, then 32 columns per CTA, which read the operands 32
+  // times less often
   auto run = [&](auto columns, auto blocks, const char* name, int threads, size_t vec, size_t stage, size_t two,
                  size_t one, auto* Dinv, auto* Ainv) {
     const size_t ring = vec + dev::kRingHead + 3 * stage;
